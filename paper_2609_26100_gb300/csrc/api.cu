@@ -154,7 +154,7 @@ struct tss_ctx {
   unsigned long long epoch = 0;
   float* ssp = nullptr;
   unsigned long long* flags = nullptr;  // hflag | qkvflag | guflag | attflag
-  int* mk_zero = nullptr;               // counters [7][max_tiles] | abort word | attention counters
+  int* mk_zero = nullptr;               // counters, finished shares [7][max_tiles] each | abort word | attention counters
   int mk_max_tiles = 0, mk_n_zero = 0;
   float *mk_part0 = nullptr, *mk_part1 = nullptr;
   size_t mk_part_floats = 0;
@@ -607,7 +607,7 @@ tss_status enqueue_step_mk(tss_ctx* c, const StepPlan& sp, cudaStream_t s, Prof*
   p.partials0 = c->mk_part0;
   p.partials1 = c->mk_part1;
   p.counters = c->mk_zero;
-  p.abort_word = c->mk_zero + 7 * c->mk_max_tiles;
+  p.abort_word = c->mk_zero + 14 * c->mk_max_tiles;
   p.ssp = c->ssp;
   p.hflag = c->flags;
   p.qkvflag = c->flags + nt;
@@ -877,10 +877,10 @@ tss_status build_workspaces(tss_ctx* c) {
     TSS_CU(cudaMemset(c->flags, 0, nflags * sizeof(unsigned long long)));
     // stream-K counters, the abort word and the attention's split counters: zeroed by every
     // step's prologue, so that a step after one that gave up on a timeout starts clean
-    c->mk_n_zero = 7 * max_tiles + 1 + c->a.max_batch * c->H;
+    c->mk_n_zero = 14 * max_tiles + 1 + c->a.max_batch * c->H;
     TSS_TRY(c->alloc(&c->mk_zero, static_cast<size_t>(c->mk_n_zero)));
     TSS_CU(cudaMemset(c->mk_zero, 0, static_cast<size_t>(c->mk_n_zero) * sizeof(int)));
-    c->attn_cnt = c->mk_zero + 7 * max_tiles + 1;
+    c->attn_cnt = c->mk_zero + 14 * max_tiles + 1;
     // partial tiles are strided by the MMA width of the split B operand (up to 256 rows)
     int xs_rows_max = 16;
     for (int m = 1; m <= c->a.max_rows; ++m) xs_rows_max = std::max(xs_rows_max, xs_layout(m).rows);

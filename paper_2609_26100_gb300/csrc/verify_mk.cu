@@ -45,6 +45,7 @@ __host__ __device__ inline int mk_acc_bufs(int n_pad) {
   return nb;
 }
 constexpr uint32_t kMkWBytes = 128 * 64 * 2;
+constexpr int kMkWholeKb = 20;  // mk_seg: extra k-blocks for which a tile is left whole
 
 enum MkKind : int { kMkQkv = 1, kMkAtt = 2, kMkO = 3, kMkGu = 4, kMkDown = 5, kMkLm = 6 };
 
@@ -117,6 +118,23 @@ __device__ bool mk_wait_flag(const unsigned long long* f, unsigned long long tar
       }
     }
     __nanosleep(64);
+  }
+}
+
+// Bounded wait for the arrival counter *f to reach `target`.
+__device__ bool mk_wait_count(const int* f, int target, const MkShared& sh) {
+  const uint64_t t0 = globaltimer_ns();
+  for (uint32_t i = 1;; ++i) {
+    int v;
+    asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(f) : "memory");
+    if (v >= target) return true;
+    if ((i & 63) == 0) {
+      if (mk_aborted(sh)) return false;
+      if (globaltimer_ns() - t0 > sh.limit_ns) {
+        mk_fail(sh);
+        return false;
+      }
+    }
   }
 }
 
@@ -218,6 +236,10 @@ __device__ __forceinline__ MkSeg mk_seg(const MkParams& p, const MkPhase& ph, in
   }
   s.T = static_cast<long long>(n_split) * ph.kb;
   s.geff = static_cast<int>(s.T < G ? s.T : G);
+  // Few short tiles (small models): whole tiles when streaming one takes at most kMkWholeKb
+  // k-blocks (16 KiB, about 0.23 us each) more than a CTA's even share -- about what the partial
+  // sums' store, counter and reload cost.
+  if (s.whole < 0 && n_split <= G && ph.kb <= s.T / s.geff + kMkWholeKb) s.geff = n_split;
   if (c >= s.geff) {
     s.it = s.it1 = 0;
   } else {
@@ -291,32 +313,28 @@ struct MkEpi {
   int* pos;         // [kMaxRows] RoPE position of each compacted row (QKV)
   int* kvslot;      // [kMaxRows] KV-cache slot and row of each compacted row (QKV)
   int* kvrow;
-  int nM;           // rows of the next norm phase (residual phases) and their list
+  // residual phases: the next norm phase's B operand bf16(h * g_next) is written by the epilogue
+  // that updates h.  npos[j]: compacted row j's place in the next phase, -1 if it skips it; the next
+  // phase's rows that this phase does not run (h unchanged) are nrows[x] >= 0 at place x.
+  int nM, n_extra;
+  const int* npos;
   const int* nrows;
+  const float* gnext;  // RMSNorm gain of the next norm phase
   float* xch;    // [16][128]
-  float* redv;   // [4][16]
-  int* redi;     // [4][16]
   float* rs;     // [kMaxRows] per-row RMSNorm factors of the current phase
   const float* rcos;  // [16][D/2] RoPE cos / sin of the first 16 rows (QKV), staged at phase start
   const float* rsin;
-  const float* gnext;  // residual phases: RMSNorm gain of the next norm phase
-  bool direct_xn;      // residual phases: the next norm phase runs the same rows in the same order,
-                       // so the epilogue writes its B operand straight from the updated h
-  int hpre_tile;       // residual phases: tile whose h rows were preloaded into xch (-1: none)
-  float gn_pre;        // ... and this thread's next-norm gain on that tile
-  // values the epilogue chunks would otherwise load from the step descriptor in global memory
+  // values the epilogues would otherwise load from the step descriptor in global memory
   __nv_bfloat16* kv_base;  // QKV: this layer's KV cache
   size_t kv_cap;
   float* logits;           // LM head: caller's logits or null
+  bool logits_vec;         // ... and whether 16-byte stores fit its rows
   int q, lane, et;
 };
 
 // Wait until every 128-feature tile of h has reached `dep`, then compute the RMSNorm factors of
 // the phase's rows from the partial sums of squares (fixed order, deterministic).
-__device__ bool mk_prepare_rs(const MkParams& p, const MkEpi& e, unsigned long long dep, const MkShared& sh,
-                              bool& ready) {
-  if (ready) return true;  // once per phase
-  ready = true;
+__device__ bool mk_prepare_rs(const MkParams& p, const MkEpi& e, unsigned long long dep, const MkShared& sh) {
   const int nt = p.d / 128;
   bool ok = true;
   for (int t = e.et; dep != 0ull && t < nt && ok; t += 128) ok = mk_wait_flag(&p.hflag[t], dep, sh);
@@ -332,173 +350,20 @@ __device__ bool mk_prepare_rs(const MkParams& p, const MkEpi& e, unsigned long l
   return true;
 }
 
-// Fused epilogue of one 16-token chunk (tokens ch*16 ..) of output row r of tile t.
-// hv (residual phases, optional): h of these 16 rows at this thread's feature, loaded by the caller
-// together with the partial sums.
-__device__ void mk_epilogue_chunk(const MkParams& p, const MkPhase& ph, const MkEpi& e, int t, int r, int ch,
-                                  const float* v, const float* hv = nullptr) {
-  const StepDesc* st = p.step;
-  const int j0 = ch * 16;
-  if (ph.kind == kMkQkv) {
-    const int d = p.d, D = p.D, half = D >> 1;
-    const int o = t * 128 + r;
-    const int sec = o / d;
-    const int f = o - sec * d;
-    const int head = f / D, dim = f - head * D;
-    float val[16];
-#pragma unroll
-    for (int jj = 0; jj < 16; ++jj) val[jj] = j0 + jj < e.M ? v[jj] * e.rs[j0 + jj] : 0.f;
-    if (sec < 2) {
-      // rotation factors first (the first 16 rows staged in shared memory, later rows' loads in
-      // flight during the exchange of the partner elements)
-      const int i = dim & (half - 1);
-      float cs[16], sn[16];
-      if (j0 == 0) {
-#pragma unroll
-        for (int jj = 0; jj < 16; ++jj) {
-          cs[jj] = e.rcos[jj * half + i];
-          sn[jj] = e.rsin[jj * half + i];
-        }
-      } else {
-#pragma unroll
-        for (int jj = 0; jj < 16; ++jj) {
-          const bool in = j0 + jj < e.M;
-          const size_t pe = static_cast<size_t>(in ? e.pos[j0 + jj] : 0) * half + i;
-          cs[jj] = in ? __ldg(&p.rope_cos[pe]) : 0.f;
-          sn[jj] = in ? __ldg(&p.rope_sin[pe]) : 0.f;
-        }
-      }
-#pragma unroll
-      for (int jj = 0; jj < 16; ++jj) e.xch[jj * 128 + r] = val[jj];
-      named_bar_sync(1, 128);
-      const int pr = r ^ half;
-      float rot[16];
-#pragma unroll
-      for (int jj = 0; jj < 16; ++jj) {
-        const float pv = e.xch[jj * 128 + pr];
-        rot[jj] = j0 + jj < e.M ? (dim < half ? val[jj] * cs[jj] - pv * sn[jj] : val[jj] * cs[jj] + pv * sn[jj]) : 0.f;
-      }
-      named_bar_sync(1, 128);
-#pragma unroll
-      for (int jj = 0; jj < 16; ++jj) val[jj] = rot[jj];
-    }
-#pragma unroll
-    for (int jj = 0; jj < 16; ++jj) {
-      const int j = j0 + jj;
-      if (j >= e.M) continue;
-      if (sec == 0) {
-        // q in fp16 (11 significant bits), split exactly into bf16 hi + lo by the attention
-        reinterpret_cast<__half*>(p.qbuf)[static_cast<size_t>(j) * d + f] = __float2half_rn(val[jj]);
-      } else {
-        const size_t off = ((static_cast<size_t>(e.kvslot[j]) * 2 + (sec - 1)) * p.H + head) *
-                               e.kv_cap +
-                           e.kvrow[j];
-        e.kv_base[off * D + dim] = __float2bfloat16_rn(val[jj]);
-      }
-    }
-  } else if (ph.kind == kMkO || ph.kind == kMkDown) {
-    // residual add, then this tile's partial sum of squares of the updated rows
-    const int o = t * 128 + r;
-    const float gn = e.direct_xn ? (t == e.hpre_tile ? e.gn_pre : e.gnext[o]) : 0.f;
-    float sq[16];
-#pragma unroll
-    for (int jj = 0; jj < 16; ++jj) {
-      const int j = j0 + jj;
-      sq[jj] = 0.f;
-      if (j < e.M) {
-        float* hp = p.h + static_cast<size_t>(e.rows[j]) * p.d + o;
-        // h of the CTA's last tile was loaded at phase start (off the critical path)
-        const float nv = (t == e.hpre_tile ? e.xch[jj * 128 + r] : hv ? hv[jj] : __ldcg(hp)) + v[jj];
-        *hp = nv;
-        sq[jj] = nv * nv;
-        if (e.direct_xn) store_split(p.xn, p.xs, j, o, nv * gn);
-      }
-    }
-#pragma unroll
-    for (int jj = 0; jj < 16; ++jj) {
-#pragma unroll
-      for (int off = 16; off > 0; off >>= 1) sq[jj] += __shfl_xor_sync(0xffffffffu, sq[jj], off);
-    }
-    if (e.lane == 0) {
-#pragma unroll
-      for (int jj = 0; jj < 16; ++jj) e.redv[e.q * 16 + jj] = sq[jj];
-    }
-    named_bar_sync(1, 128);
-    if (e.et < 16 && j0 + e.et < e.M) {
-      const int jj = e.et;
-      const float s4 = (e.redv[jj] + e.redv[16 + jj]) + (e.redv[32 + jj] + e.redv[48 + jj]);
-      p.ssp[static_cast<size_t>(t) * kMaxRows + e.rows[j0 + jj]] = s4;
-    }
-    named_bar_sync(1, 128);
-  } else if (ph.kind == kMkGu) {
-#pragma unroll
-    for (int jj = 0; jj < 16; ++jj) e.xch[jj * 128 + r] = v[jj];
-    named_bar_sync(1, 128);
-    if (r < 64) {
-      const int fcol = t * 64 + r;
-#pragma unroll
-      for (int jj = 0; jj < 16; ++jj) {
-        const int j = j0 + jj;
-        if (j < e.M) {
-          const float g = v[jj] * e.rs[j];
-          const float u = e.xch[jj * 128 + r + 64] * e.rs[j];
-          store_split(p.act, p.xs, j, fcol, g / (1.f + expf(-g)) * u);
-        }
-      }
-    }
-    named_bar_sync(1, 128);
-  } else {  // LM head: logits (optional) and per-tile argmax, lowest index on ties
-    const int o = t * 128 + r;
-    const bool valid = o < p.V;
-    float* logits = e.logits;
-#pragma unroll
-    for (int jj = 0; jj < 16; ++jj) {
-      const int j = j0 + jj;
-      float val = -INFINITY;
-      if (valid && j < e.M) {
-        val = v[jj] * e.rs[j];
-        if (logits) logits[static_cast<size_t>(e.rows[j]) * p.V + o] = val;
-        if (val != val) report(p.status, kStatusCheck);
-      }
-      int idx = o;
-#pragma unroll
-      for (int off = 16; off > 0; off >>= 1) {
-        const float ov = __shfl_xor_sync(0xffffffffu, val, off);
-        const int oi = __shfl_xor_sync(0xffffffffu, idx, off);
-        if (ov > val || (ov == val && oi < idx)) {
-          val = ov;
-          idx = oi;
-        }
-      }
-      if (e.lane == 0) {
-        e.redv[e.q * 16 + jj] = val;
-        e.redi[e.q * 16 + jj] = idx;
-      }
-    }
-    named_bar_sync(1, 128);
-    if (e.et < 16 && j0 + e.et < e.M) {
-      const int jj = e.et;
-      float bv = e.redv[jj];
-      int bi = e.redi[jj];
-#pragma unroll
-      for (int w = 1; w < 4; ++w) {
-        const float ov = e.redv[w * 16 + jj];
-        const int oi = e.redi[w * 16 + jj];
-        if (ov > bv || (ov == bv && oi < bi)) {
-          bv = ov;
-          bi = oi;
-        }
-      }
-      p.amax_val[static_cast<size_t>(t) * kMaxRows + e.rows[j0 + jj]] = bv;
-      p.amax_idx[static_cast<size_t>(t) * kMaxRows + e.rows[j0 + jj]] = bi;
-    }
-    named_bar_sync(1, 128);
-  }
+// Stores of 4 consecutive features (k % 4 == 0) into the split hi/lo layout: they are adjacent in
+// the swizzled 64-element rows, so each part is one 8-byte store.  The part of the address that does
+// not depend on the row is kept per lane, and the lo part lies at a constant distance (half is a
+// multiple of 8, so both parts' rows are swizzled alike).
+struct SplitAt {
+  __nv_bfloat16* base;  // of feature k's k-block, plus k & 7
+  uint32_t c8, lo;      // 16-byte chunk within the 64-element row; elements from a hi to its lo part
+};
+__device__ __forceinline__ SplitAt split_at(__nv_bfloat16* buf, const XsLayout& L, int k) {
+  const uint32_t kb = static_cast<uint32_t>(k) >> 6, kc = static_cast<uint32_t>(k) & 63u;
+  return SplitAt{buf + kb * static_cast<uint32_t>(L.parts * L.rows * 64) + (kc & 7u), kc >> 3,
+                 static_cast<uint32_t>(L.parts == 1 ? L.half : L.rows) * 64u};
 }
-
-// Stores of 4 consecutive features (k % 4 == 0) of row j into the split hi/lo layout: they are
-// adjacent in the swizzled 64-element rows, so each part is one 8-byte store.
-__device__ __forceinline__ void store_split4(__nv_bfloat16* buf, const XsLayout& L, int j, int k, const float* x) {
+__device__ __forceinline__ void store_split4(const SplitAt& s, int j, const float* x) {
   uint32_t hi[2], lo[2];
 #pragma unroll
   for (int i = 0; i < 2; ++i) {
@@ -506,36 +371,107 @@ __device__ __forceinline__ void store_split4(__nv_bfloat16* buf, const XsLayout&
     const float h0 = __uint_as_float(hi[i] << 16), h1 = __uint_as_float(hi[i] & 0xffff0000u);
     lo[i] = pack_bf16(x[2 * i] - h0, x[2 * i + 1] - h1);
   }
-  *reinterpret_cast<uint2*>(buf + xs_elem(L, j, k, 0)) = make_uint2(hi[0], hi[1]);
-  *reinterpret_cast<uint2*>(buf + xs_elem(L, j, k, 1)) = make_uint2(lo[0], lo[1]);
+  const uint32_t row = static_cast<uint32_t>(j);
+  __nv_bfloat16* d = s.base + row * 64u + ((s.c8 ^ (row & 7u)) << 3);
+  *reinterpret_cast<uint2*>(d) = make_uint2(hi[0], hi[1]);
+  *reinterpret_cast<uint2*>(d + s.lo) = make_uint2(lo[0], lo[1]);
 }
 
-// Fix-up of tile t from the partials of contributors cf..cl (in that order): warp q takes the
-// groups of G rows q, q + 4, ... and each lane 4 adjacent features of all 128, so that the
-// partner elements of RoPE and SwiGLU and the reductions over the tile's features (sums of
-// squares, argmax) stay within one warp -- no exchange between the warps and no barrier -- and
-// every load and store is a 16- or 8-byte vector.  CB contributors' partials per round of loads.
-template <int G, int CB>
-__device__ void mk_finalize_by_warps(const MkParams& p, const MkPhase& ph, const MkEpi& e, int t, int cf, int cl,
-                                     const float* partials, int n_pad) {
+// Sums of G values per lane over the warp's 32 lanes, G a power of two: the values are halved
+// between lane pairs first (G - 1 shuffles), then one value each remains to be summed.  Lane l ends
+// with the sum of value l & (G - 1).
+template <int G>
+__device__ __forceinline__ float warp_sums(const float* x, int lane) {
+  float y[G];
+#pragma unroll
+  for (int i = 0; i < G; ++i) y[i] = x[i];
+#pragma unroll
+  for (int w = G / 2; w >= 1; w >>= 1) {
+    const bool up = lane & w;
+#pragma unroll
+    for (int i = 0; i < w; ++i) {
+      const float give = up ? y[i] : y[i + w];
+      y[i] = (up ? y[i + w] : y[i]) + __shfl_xor_sync(0xffffffffu, give, w);
+    }
+  }
+  float r = y[0];
+#pragma unroll
+  for (int w = G; w < 32; w <<= 1) r += __shfl_xor_sync(0xffffffffu, r, w);
+  return r;
+}
+
+__device__ __forceinline__ bool mk_resid(const MkPhase& ph) { return ph.kind == kMkO || ph.kind == kMkDown; }
+
+// Finishes rows of output tile t: the fused epilogue of the phase on the tile's fp32 sums.  A
+// unit is G rows; a warp takes units u0, u0 + du, ... below n_units and each lane 4 adjacent
+// features of all 128, so that the partner elements of RoPE and SwiGLU and the reductions over
+// the tile's features (sums of squares, argmax) stay within one warp and every load and store is
+// a 16- or 8-byte vector.  The sums are
+//   whole: the accumulator in this CTA's tensor memory, read 4 G rows at a time (thread = feature)
+//          and turned around through shared memory; u0 = warp, du = 4, every warp the same number
+//          of turns; the accumulator buffer is released after the last read;
+//   else:  the partials of contributors cf..cl, added in that order (deterministic), CB of them per
+//          round of loads.
+template <int D, int G, int CB>
+__device__ void mk_finish_rows(const MkParams& p, const MkPhase& ph, const MkEpi& e, int t, bool whole, uint32_t tb,
+                               uint64_t* acce, int u0, int du, int cf, int cl, const float* partials, int n_pad) {
   const int lane = e.lane, f0 = 4 * lane;  // features f0 .. f0 + 3 of the tile
-  const int n_groups = (e.M + G - 1) / G;
-  const bool resid = ph.kind == kMkO || ph.kind == kMkDown;
+  const int n_units = (e.M + G - 1) / G;
+  const int n_it = whole ? (n_units + 3) >> 2 : (n_units - u0 + du - 1) / du;
+  const bool resid = mk_resid(ph);
+  constexpr int half = D / 2;
+  const int d = p.d;
+  const int sec = ph.kind != kMkQkv || t * 128 < d ? 0 : t * 128 < 2 * d ? 1 : 2;  // QKV: q, k or v (one per tile)
+  const int fs = t * 128 + f0 - sec * d;
+  const int head = fs / D, dim0 = fs % D;
   float4 gn = make_float4(0.f, 0.f, 0.f, 0.f);
-  if (resid && e.direct_xn) gn = *reinterpret_cast<const float4*>(e.gnext + t * 128 + f0);
-  for (int grp = e.q; grp < n_groups; grp += 4) {
-    {
-      const int j0 = grp * G;
-      float v[G][4], hv[G][4];
+  if (resid) gn = *reinterpret_cast<const float4*>(e.gnext + t * 128 + f0);
+  const SplitAt xat = resid ? split_at(p.xn, p.xs, t * 128 + f0) : split_at(p.act, p.xs, t * 64 + (f0 & 63));
+  for (int it = 0; it < n_it; ++it) {
+    const int j0 = (u0 + it * du) * G;
+    // residual phases: h; QKV: the rotation factors -- requested before the sums
+    float4 ha[G], hb[G];
+#pragma unroll
+    for (int jj = 0; jj < G; ++jj) {
+      const int j = j0 + jj;
+      ha[jj] = hb[jj] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (j < e.M) {
+        if (resid) {
+          ha[jj] = __ldcg(reinterpret_cast<const float4*>(p.h + static_cast<size_t>(e.rows[j]) * d + t * 128 + f0));
+        } else if (ph.kind == kMkQkv && sec < 2) {
+          const int ii = dim0 & (half - 1);
+          if (j < 16) {
+            ha[jj] = *reinterpret_cast<const float4*>(e.rcos + j * half + ii);
+            hb[jj] = *reinterpret_cast<const float4*>(e.rsin + j * half + ii);
+          } else {
+            const size_t pe = static_cast<size_t>(e.pos[j]) * half + ii;
+            ha[jj] = __ldg(reinterpret_cast<const float4*>(p.rope_cos + pe));
+            hb[jj] = __ldg(reinterpret_cast<const float4*>(p.rope_sin + pe));
+          }
+        }
+      }
+    }
+    float v[G][4];
+    if (whole) {
+      const int r = e.q * 32 + lane;
+      float a[16];
+      mk_acc_tokens(tb, it, p.xs, a);
+      if (it == n_it - 1) {
+        tc_fence_before();
+        mbar_arrive(acce);
+      }
+#pragma unroll
+      for (int jj = 0; jj < 4 * G; ++jj) e.xch[jj * 128 + r] = a[jj];
+      named_bar_sync(1, 128);
 #pragma unroll
       for (int jj = 0; jj < G; ++jj) {
-        const bool in = j0 + jj < e.M;
-        float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (resid && in) x = __ldcg(reinterpret_cast<const float4*>(p.h + static_cast<size_t>(e.rows[j0 + jj]) * p.d + t * 128 + f0));
-        hv[jj][0] = x.x; hv[jj][1] = x.y; hv[jj][2] = x.z; hv[jj][3] = x.w;
-        v[jj][0] = v[jj][1] = v[jj][2] = v[jj][3] = 0.f;
+        const float4 x = *reinterpret_cast<const float4*>(e.xch + (e.q * G + jj) * 128 + f0);
+        v[jj][0] = x.x; v[jj][1] = x.y; v[jj][2] = x.z; v[jj][3] = x.w;
       }
-      // contributors in order (deterministic sum), CB partials' loads in flight at once
+      if (it < n_it - 1) named_bar_sync(1, 128);  // (after the last turn the caller's barrier follows)
+    } else {
+#pragma unroll
+      for (int jj = 0; jj < G; ++jj) v[jj][0] = v[jj][1] = v[jj][2] = v[jj][3] = 0.f;
       for (int c0 = cf; c0 <= cl; c0 += CB) {
         float4 a[CB][G];
 #pragma unroll
@@ -557,134 +493,139 @@ __device__ void mk_finalize_by_warps(const MkParams& p, const MkPhase& ph, const
             v[jj][3] += a[q][jj].w;
           }
       }
+    }
+    if (ph.kind == kMkQkv) {
 #pragma unroll
       for (int jj = 0; jj < G; ++jj) {
         const int j = j0 + jj;
         const bool in = j < e.M;  // uniform over the warp
-        if (ph.kind == kMkQkv) {
-          const int d = p.d, D = p.D, half = D >> 1;
-          const int sec = (t * 128) / d;  // q, k or v: one per tile
-          const int fs = t * 128 + f0 - sec * d;
-          const int head = fs / D, dim0 = fs - head * D;
-          const float rsj = in ? e.rs[j] : 0.f;
-          float val[4];
+        const float rsj = in ? e.rs[j] : 0.f;
+        float val[4];
 #pragma unroll
-          for (int i = 0; i < 4; ++i) val[i] = v[jj][i] * rsj;
-          if (sec < 2) {  // rotate-half RoPE: the partner feature dim ^ half sits in lane ^ half / 4
-            float rot[4];
-            const int pos = in ? e.pos[j] : 0;
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-              const float pv = __shfl_xor_sync(0xffffffffu, val[i], half >> 2);
-              const int ii = (dim0 + i) & (half - 1);
-              const float c = j < 16 ? e.rcos[j * half + ii] : __ldg(&p.rope_cos[static_cast<size_t>(pos) * half + ii]);
-              const float sn = j < 16 ? e.rsin[j * half + ii] : __ldg(&p.rope_sin[static_cast<size_t>(pos) * half + ii]);
-              rot[i] = dim0 < half ? val[i] * c - pv * sn : val[i] * c + pv * sn;
-            }
-#pragma unroll
-            for (int i = 0; i < 4; ++i) val[i] = rot[i];
-          }
-          if (in) {
-            if (sec == 0) {  // q in fp16 (11 significant bits), split exactly into bf16 hi + lo by the attention
-              const uint32_t w0 = pack_f16(val[0], val[1]), w1 = pack_f16(val[2], val[3]);
-              *reinterpret_cast<uint2*>(reinterpret_cast<__half*>(p.qbuf) + static_cast<size_t>(j) * d + fs) =
-                  make_uint2(w0, w1);
-            } else {
-              const size_t off = ((static_cast<size_t>(e.kvslot[j]) * 2 + (sec - 1)) * p.H + head) * e.kv_cap + e.kvrow[j];
-              *reinterpret_cast<uint2*>(e.kv_base + off * D + dim0) =
-                  make_uint2(pack_bf16(val[0], val[1]), pack_bf16(val[2], val[3]));
-            }
-          }
-        } else if (resid) {
-          float nv[4];
-#pragma unroll
-          for (int i = 0; i < 4; ++i) nv[i] = hv[jj][i] + v[jj][i];
-          float sq = (nv[0] * nv[0] + nv[1] * nv[1]) + (nv[2] * nv[2] + nv[3] * nv[3]);
-#pragma unroll
-          for (int off = 16; off > 0; off >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, off);
-          if (in) {
-            const int m = e.rows[j];
-            *reinterpret_cast<float4*>(p.h + static_cast<size_t>(m) * p.d + t * 128 + f0) =
-                make_float4(nv[0], nv[1], nv[2], nv[3]);
-            if (e.direct_xn) {
-              const float xg[4] = {nv[0] * gn.x, nv[1] * gn.y, nv[2] * gn.z, nv[3] * gn.w};
-              store_split4(p.xn, p.xs, j, t * 128 + f0, xg);
-            }
-            if (lane == 0) p.ssp[static_cast<size_t>(t) * kMaxRows + m] = sq;
-          }
-        } else if (ph.kind == kMkGu) {  // lanes 0-15: gate features, 16-31: the matching up features
-          const float rsj = in ? e.rs[j] : 0.f;
-          float x[4], act[4];
+        for (int i = 0; i < 4; ++i) val[i] = v[jj][i] * rsj;
+        if (sec < 2) {  // rotate-half RoPE: the partner feature dim ^ half sits in lane ^ half / 4
+          const float cs[4] = {ha[jj].x, ha[jj].y, ha[jj].z, ha[jj].w}, sn[4] = {hb[jj].x, hb[jj].y, hb[jj].z, hb[jj].w};
+          float rot[4];
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
-            x[i] = v[jj][i] * rsj;
-            const float u = __shfl_xor_sync(0xffffffffu, x[i], 16);
-            act[i] = x[i] / (1.f + expf(-x[i])) * u;
-          }
-          if (in && lane < 16) store_split4(p.act, p.xs, j, t * 64 + f0, act);
-        } else {  // LM head: logits and the tile's argmax of row j, lowest index on ties
-          const float rsj = in ? e.rs[j] : 0.f;
-          float bv = -INFINITY;
-          int bi = t * 128 + f0;
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const int o = t * 128 + f0 + i;
-            const float val = o < p.V && in ? v[jj][i] * rsj : -INFINITY;
-            if (o < p.V && in) {
-              if (e.logits) e.logits[static_cast<size_t>(e.rows[j]) * p.V + o] = val;
-              if (val != val) report(p.status, kStatusCheck);
-            }
-            if (val > bv) {
-              bv = val;
-              bi = o;
-            }
+            const float pv = __shfl_xor_sync(0xffffffffu, val[i], half >> 2);
+            rot[i] = dim0 < half ? val[i] * cs[i] - pv * sn[i] : val[i] * cs[i] + pv * sn[i];
           }
 #pragma unroll
-          for (int off = 16; off > 0; off >>= 1) {
-            const float ov = __shfl_xor_sync(0xffffffffu, bv, off);
-            const int oi = __shfl_xor_sync(0xffffffffu, bi, off);
-            if (ov > bv || (ov == bv && oi < bi)) {
-              bv = ov;
-              bi = oi;
-            }
+          for (int i = 0; i < 4; ++i) val[i] = rot[i];
+        }
+        if (in) {
+          if (sec == 0) {  // q in fp16 (11 significant bits), split exactly into bf16 hi + lo by the attention
+            const uint32_t w0 = pack_f16(val[0], val[1]), w1 = pack_f16(val[2], val[3]);
+            *reinterpret_cast<uint2*>(reinterpret_cast<__half*>(p.qbuf) + static_cast<size_t>(j) * d + fs) =
+                make_uint2(w0, w1);
+          } else {
+            const size_t off = ((static_cast<size_t>(e.kvslot[j]) * 2 + (sec - 1)) * p.H + head) * e.kv_cap + e.kvrow[j];
+            *reinterpret_cast<uint2*>(e.kv_base + off * D + dim0) =
+                make_uint2(pack_bf16(val[0], val[1]), pack_bf16(val[2], val[3]));
           }
-          if (in && lane == 0) {
-            p.amax_val[static_cast<size_t>(t) * kMaxRows + e.rows[j]] = bv;
-            p.amax_idx[static_cast<size_t>(t) * kMaxRows + e.rows[j]] = bi;
+        }
+      }
+    } else if (resid) {  // residual add, the rows' partial sums of squares, the next phase's B operand
+      float sq[G];
+#pragma unroll
+      for (int jj = 0; jj < G; ++jj) {
+        const int j = j0 + jj;
+        const float nv[4] = {ha[jj].x + v[jj][0], ha[jj].y + v[jj][1], ha[jj].z + v[jj][2], ha[jj].w + v[jj][3]};
+        sq[jj] = (nv[0] * nv[0] + nv[1] * nv[1]) + (nv[2] * nv[2] + nv[3] * nv[3]);
+        if (j < e.M) {
+          const int m = e.rows[j], np = e.npos[j];
+          *reinterpret_cast<float4*>(p.h + static_cast<size_t>(m) * d + t * 128 + f0) =
+              make_float4(nv[0], nv[1], nv[2], nv[3]);
+          if (np >= 0) {
+            const float xg[4] = {nv[0] * gn.x, nv[1] * gn.y, nv[2] * gn.z, nv[3] * gn.w};
+            store_split4(xat, np, xg);
           }
+        }
+      }
+      const float sum = warp_sums<G>(sq, lane);
+      if (lane < G && j0 + lane < e.M) p.ssp[static_cast<size_t>(t) * kMaxRows + e.rows[j0 + lane]] = sum;
+    } else if (ph.kind == kMkGu) {
+      // lanes 0-15 hold gate features, lanes 16-31 the matching up features: of two rows the lower
+      // half-warp finishes the first and the upper the second (one exchange, one division per value)
+#pragma unroll
+      for (int jj = 0; jj < G; jj += 2) {
+        const bool upper = lane >= 16;
+        const int ja = j0 + jj, jb = ja + 1, j = upper ? jb : ja;
+        const float ra = ja < e.M ? e.rs[ja] : 0.f, rb = jb < e.M ? e.rs[jb] : 0.f;
+        float act[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const float xa = v[jj][i] * ra, xb = v[jj + 1][i] * rb;
+          const float y = __shfl_xor_sync(0xffffffffu, upper ? xa : xb, 16);
+          const float g = upper ? y : xa, u = upper ? xb : y;
+          act[i] = __fdividef(g, 1.f + expf(-g)) * u;
+        }
+        if (j < e.M) store_split4(xat, j, act);
+      }
+    } else {  // LM head: logits and the tile's argmax of each row, lowest index on ties
+      const int o0 = t * 128 + f0;
+#pragma unroll
+      for (int jj = 0; jj < G; ++jj) {
+        const int j = j0 + jj;
+        const bool in = j < e.M;
+        const float rsj = in ? e.rs[j] : 0.f;
+        float bv = -INFINITY;
+        int bi = o0;
+        float val[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const bool on = o0 + i < p.V && in;
+          val[i] = on ? v[jj][i] * rsj : -INFINITY;
+          if (on && val[i] != val[i]) report(p.status, kStatusCheck);
+          if (val[i] > bv) {
+            bv = val[i];
+            bi = o0 + i;
+          }
+        }
+        if (e.logits && in) {
+          float* lg = e.logits + static_cast<size_t>(e.rows[j]) * p.V + o0;
+          if (e.logits_vec) {  // (V is a multiple of 4: all four features exist, or none)
+            if (o0 < p.V) *reinterpret_cast<float4*>(lg) = make_float4(val[0], val[1], val[2], val[3]);
+          } else {
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+              if (o0 + i < p.V) lg[i] = val[i];
+          }
+        }
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) {
+          const float ov = __shfl_xor_sync(0xffffffffu, bv, off);
+          const int oi = __shfl_xor_sync(0xffffffffu, bi, off);
+          if (ov > bv || (ov == bv && oi < bi)) {
+            bv = ov;
+            bi = oi;
+          }
+        }
+        if (in && lane == 0) {
+          p.amax_val[static_cast<size_t>(t) * kMaxRows + e.rows[j]] = bv;
+          p.amax_idx[static_cast<size_t>(t) * kMaxRows + e.rows[j]] = bi;
         }
       }
     }
   }
+  // residual phases: the next phase's rows that skip this layer (mixed skip sets), a warp each
+  if (resid && e.n_extra > 0) {
+    for (int x = u0; x < e.nM; x += du) {
+      const int m = e.nrows[x];
+      if (m < 0) continue;
+      const float4 hv = __ldcg(reinterpret_cast<const float4*>(p.h + static_cast<size_t>(m) * d + t * 128 + f0));
+      const float xg[4] = {hv.x * gn.x, hv.y * gn.y, hv.z * gn.z, hv.w * gn.w};
+      store_split4(xat, x, xg);
+    }
+  }
 }
 
-// After a residual phase finalised tile t of h: write the next norm phase's B operand
-// bf16(h * g_next) for features [128t, 128t+128) of every row that phase runs, in its compacted
-// order (O -> gate/up of the same layer; down -> QKV of the next layer, or the LM head).
+// The plan slot whose rows the next norm phase runs (O -> gate/up of the same layer; down -> QKV
+// of the next layer, or the LM head).
 __device__ __forceinline__ int mk_next_slot(const MkParams& p, const MkPhase& ph) {
   if (ph.kind == kMkO) return ph.slot;
   return ph.slot + 1 < p.n_act ? ph.slot + 1 : kFinalSlot;
-}
-
-__device__ void mk_write_next_xn(const MkParams& p, const PlanDev* pl, const MkPhase& ph, const MkEpi& e, int t,
-                                 int r) {
-  const int nslot = mk_next_slot(p, ph);
-  const float* g = ph.kind == kMkO ? p.g_mlp + static_cast<size_t>(ph.layer) * p.d
-                   : nslot != kFinalSlot ? p.g_attn + static_cast<size_t>(pl->act_layer[nslot]) * p.d
-                                         : p.g_final;
-  const int M = e.nM;
-  const int* rows = e.nrows;
-  const int f = t * 128 + r;
-  const float gf = g[f];
-  for (int n0 = 0; n0 < M; n0 += 8) {
-    float hv[8];
-#pragma unroll
-    for (int u = 0; u < 8; ++u)
-      hv[u] = n0 + u < M ? __ldcg(&p.h[static_cast<size_t>(rows[n0 + u]) * p.d + f]) : 0.f;
-#pragma unroll
-    for (int u = 0; u < 8; ++u)
-      if (n0 + u < M) store_split(p.xn, p.xs, n0 + u, f, hv[u] * gf);
-  }
 }
 
 __device__ __forceinline__ unsigned long long* mk_tile_flag(const MkParams& p, int kind, int t) {
@@ -768,13 +709,14 @@ __global__ void __launch_bounds__(kMkThreads, 1)
   uint64_t* acce = accf + kMkMaxAcc;
   uint64_t* team = acce + kMkMaxAcc;  // all 256 threads: entry to / exit from a layer's attention
   int* misc = reinterpret_cast<int*>(team + 1);  // [0] tmem addr, [1] abort, [2..4] bcast, [5] s_last
-  float* xch = reinterpret_cast<float*>(misc + 16);
-  float* redv = xch + 16 * 128;
-  int* redi = reinterpret_cast<int*>(redv + 64);
-  float* rs = reinterpret_cast<float*>(redi + 64);
+  // (16-byte vectors from here on: the mbarriers before are an odd number of 8-byte words)
+  float* xch = reinterpret_cast<float*>((reinterpret_cast<uintptr_t>(misc + 16) + 15) & ~uintptr_t(15));
+  int* s_pend = reinterpret_cast<int*>(xch + 16 * 128);  // [2][4] split tiles of this CTA's phase: t, cf, cl, complete
+  float* rs = reinterpret_cast<float*>(s_pend + 128);
   float (*sM)[16] = reinterpret_cast<float (*)[16]>(rs + kMaxRows);  // [8][16] per attention warp
   float (*sL)[16] = reinterpret_cast<float (*)[16]>(rs + kMaxRows + 128);
-  int* s_rows = reinterpret_cast<int*>(rs + kMaxRows + 256);  // [kMaxRows] x 5: rows, pos, kv slot, kv row, next rows
+  // [kMaxRows] x 5: rows, pos (residual phases: places in the next phase), kv slot, kv row, next rows
+  int* s_rows = reinterpret_cast<int*>(rs + kMaxRows + 256);
   int* s_pos = s_rows + kMaxRows;
   int* s_kvslot = s_pos + kMaxRows;
   int* s_kvrow = s_kvslot + kMaxRows;
@@ -857,8 +799,6 @@ __global__ void __launch_bounds__(kMkThreads, 1)
   e.lane = lane;
   e.et = threadIdx.x - 128;
   e.xch = xch;
-  e.redv = redv;
-  e.redi = redi;
   e.rs = rs;
   e.rcos = s_rope;
   e.rsin = s_rope + 16 * 64;
@@ -1045,7 +985,9 @@ __global__ void __launch_bounds__(kMkThreads, 1)
     } else if (warp >= 4) {
       // ---------------- epilogues ----------------
       MkSeg seg = mk_seg(p, ph, c, G);
-      if (seg.done() && ph.kind != kMkQkv) continue;
+      // (a CTA without work in a QKV or gate/up phase still waits for h there: its residual
+      // epilogues read h of the phases before)
+      if (seg.done() && ph.kind != kMkQkv && ph.kind != kMkGu) continue;
       // per-phase row metadata in shared memory (loaded while the first accumulator is pending)
       const int rslot = mk_row_slot(ph);
       e.M = pl->slot_M[rslot];
@@ -1060,17 +1002,22 @@ __global__ void __launch_bounds__(kMkThreads, 1)
           s_kvrow[j] = p.step->req_ctx[b] + (m - p.step->req_rowoff[b]);
         }
       }
-      e.direct_xn = false;
-      if (ph.kind == kMkO || ph.kind == kMkDown) {
+      e.n_extra = 0;
+      if (mk_resid(ph)) {
         const int ns = mk_next_slot(p, ph);
         e.nM = pl->slot_M[ns];
-        bool same = e.nM == e.M;
-        for (int j = e.et; j < e.nM; j += 128) {
-          const int m = pl->slot_rows[ns][j];
-          s_nrows[j] = m;
-          same = same && j < e.M && pl->slot_rows[rslot][j] == m;
+        for (int j = e.et; j < e.M; j += 128) {
+          const int m = pl->slot_rows[rslot][j], b = p.step->row_req[m], c0 = pl->slot_crow[ns][b];
+          s_pos[j] = c0 < 0 ? -1 : c0 + (m - p.step->req_rowoff[b]);
         }
-        e.direct_xn = bar_and(1, 128, same);
+        bool all_run = true;
+        for (int x = e.et; x < e.nM; x += 128) {
+          const int m = pl->slot_rows[ns][x];
+          const bool runs = pl->slot_crow[rslot][p.step->row_req[m]] >= 0;
+          s_nrows[x] = runs ? -1 : m;
+          all_run = all_run && runs;
+        }
+        e.n_extra = bar_and(1, 128, all_run) ? 0 : 1;
         e.gnext = ph.kind == kMkO ? p.g_mlp + static_cast<size_t>(ph.layer) * p.d
                   : ns != kFinalSlot ? p.g_attn + static_cast<size_t>(pl->act_layer[ns]) * p.d
                                      : p.g_final;
@@ -1080,28 +1027,16 @@ __global__ void __launch_bounds__(kMkThreads, 1)
       e.pos = s_pos;
       e.kvslot = s_kvslot;
       e.kvrow = s_kvrow;
+      e.npos = s_pos;
       e.nrows = s_nrows;
-      e.hpre_tile = -1;
-      if ((ph.kind == kMkO || ph.kind == kMkDown) && !seg.done() && e.M <= 16) {
-        // h is final for this phase (only this phase's finaliser of a tile writes it): load the
-        // rows of the CTA's last tile now, one thread per feature, into xch (unused by residual
-        // epilogues), so that finalising that tile -- typically the phase's last -- skips a
-        // memory round trip
-        const int tl = static_cast<int>((seg.it1 - 1) / ph.kb);  // (residual phases: plain stream-K)
-        float hv[16];
-#pragma unroll
-        for (int jj = 0; jj < 16; ++jj)
-          hv[jj] = jj < e.M ? __ldcg(&p.h[static_cast<size_t>(s_rows[jj]) * p.d + tl * 128 + e.q * 32 + lane]) : 0.f;
-#pragma unroll
-        for (int jj = 0; jj < 16; ++jj) xch[jj * 128 + e.q * 32 + lane] = hv[jj];
-        e.hpre_tile = tl;
-        e.gn_pre = e.direct_xn ? e.gnext[tl * 128 + e.q * 32 + lane] : 0.f;
-      }
       if (ph.kind == kMkQkv) {
         e.kv_base = p.step->kv_layer[ph.layer];
         e.kv_cap = static_cast<size_t>(p.step->kv_cap);
       }
-      if (ph.kind == kMkLm) e.logits = p.step->logits;
+      if (ph.kind == kMkLm) {
+        e.logits = p.step->logits;
+        e.logits_vec = (p.V & 3) == 0 && (reinterpret_cast<uintptr_t>(e.logits) & 15) == 0;
+      }
       if (ph.kind == kMkQkv) {
         // stage the RoPE factors of the first 16 rows; warm L2 with the context keys and values
         // this CTA's attention items will read (they do not depend on this step)
@@ -1134,18 +1069,23 @@ __global__ void __launch_bounds__(kMkThreads, 1)
         }
         named_bar_sync(1, 128);
       }
-      bool rs_ready = false;
       const long long T = seg.T;
       const int geff = seg.geff;
       float* partials = (pi & 1) ? p.partials1 : p.partials0;
       int* counters = p.counters + static_cast<size_t>(ph.kind) * p.max_tiles;
+      int* done = counters + static_cast<size_t>(7) * p.max_tiles;
       const bool needs_rs = ph.kind == kMkQkv || ph.kind == kMkGu || ph.kind == kMkLm;
-      const unsigned long long hdep = needs_rs ? mk_h_dep(p, ph) : 0ull;
       // the norm factors need only h, which is final before this phase's first accumulator
-      if (needs_rs && !mk_prepare_rs(p, e, hdep, sh, rs_ready)) {
+      if (needs_rs && !mk_prepare_rs(p, e, mk_h_dep(p, ph), sh)) {
         ok = false;
         break;
       }
+      // Tiles whose k-blocks several CTAs share: with up to 8 rows the last CTA to arrive finishes
+      // the tile (two rows a warp, one round of loads).  With more rows that CTA would be busy for
+      // many rounds while the others wait, so every contributor waits for the tile's partial sums
+      // and finishes its own share of the rows, once its last split segment is stored.
+      const bool share = e.M > 8;
+      int n_pend = 0;
       int t, k0, k1;
       bool first = true;
       while (ok && seg.next(t, k0, k1)) {
@@ -1159,25 +1099,12 @@ __global__ void __launch_bounds__(kMkThreads, 1)
         first = false;
         tc_fence_after();
         const uint32_t tb = tmem_base + (static_cast<uint32_t>(e.q * 32) << 16) + static_cast<uint32_t>(buf * n_pad);
-        const int n_ch = (e.M + 15) >> 4;  // 16-token chunks of the accumulator
         const bool tr_last = e.et == 0 && seg.done();
         if (tr_last) mk_trace(p, kMkTraceSub + pi * 8 + 0);
-        bool finalize = false;
-        int cf = 0, cl = 0;
-        if (k0 == 0 && k1 == ph.kb) {
-          if (needs_rs && !mk_prepare_rs(p, e, hdep, sh, rs_ready)) {
-            ok = false;
-            break;
-          }
-          for (int ch = 0; ch < n_ch; ++ch) {
-            float v[16];
-            mk_acc_tokens(tb, ch, p.xs, v);
-            mk_epilogue_chunk(p, ph, e, t, r, ch, v);
-          }
-          tc_fence_before();
-          mbar_arrive(&acce[buf]);
-          finalize = true;
-        } else {
+        const bool whole = k0 == 0 && k1 == ph.kb;
+        bool finish = whole;
+        if (!whole) {
+          const int n_ch = (e.M + 15) >> 4;  // 16-token chunks of the accumulator
           float* part = partials + static_cast<size_t>(c + t) * 128 * n_pad;
           for (int ch = 0; ch < n_ch; ++ch) {
             float v[16];
@@ -1193,77 +1120,69 @@ __global__ void __launch_bounds__(kMkThreads, 1)
           if (e.et == 0) {
             const int f = mk_cta_of(static_cast<long long>(t) * ph.kb, T, geff);
             const int l = mk_cta_of(static_cast<long long>(t + 1) * ph.kb - 1, T, geff);
-            const int old = atom_add_acq_rel_gpu(&counters[t], 1);
-            const int last = old == l - f;
-            if (last) atomicExch(&counters[t], 0);
-            bcast[0] = last;
-            bcast[1] = f;
-            bcast[2] = l;
+            const int last = atom_add_acq_rel_gpu(&counters[t], 1) == l - f;
+            if (last && !share) atomicExch(&counters[t], 0);
+            int* pd = s_pend + 4 * n_pend;
+            pd[0] = t;
+            pd[1] = f;
+            pd[2] = l;
+            pd[3] = last;
           }
-          named_bar_sync(1, 128);
-          finalize = bcast[0] != 0;
-          cf = bcast[1];
-          cl = bcast[2];
-          named_bar_sync(1, 128);
           if (tr_last) mk_trace(p, kMkTraceSub + pi * 8 + 2);
-          if (finalize) {  // (the counter's acquire, then the barrier: the other partials are visible)
-            if (needs_rs && !mk_prepare_rs(p, e, hdep, sh, rs_ready)) {
-              ok = false;
-              break;
-            }
-            if (tr_last) mk_trace(p, kMkTraceSub + pi * 8 + 3);
-            if (e.M <= 8 && cl - cf < 8) {
-              // up to 8 rows and 8 contributors: every partial in one round of loads, two rows a warp
-              mk_finalize_by_warps<2, 8>(p, ph, e, t, cf, cl, partials, n_pad);
-              if (tr_last) mk_trace(p, kMkTraceSub + pi * 8 + 7);
-            } else if (e.M > 16) {
-              mk_finalize_by_warps<8, 2>(p, ph, e, t, cf, cl, partials, n_pad);
+          ++n_pend;  // (at most two: only a CTA's first and last stream-K segments are partial tiles)
+        }
+        // finished now: this whole tile; the pending split tiles once the CTA has stored its last
+        // partial (the last arriver's own tile at once)
+        const int n_fin = (whole ? 1 : 0) + (!share || seg.it >= seg.it1 ? n_pend : 0);
+        if (n_pend) named_bar_sync(1, 128);  // s_pend is written (and the counter's acquire done)
+        for (int k = 0; k < n_fin; ++k) {
+          const bool wh = whole && k == 0;
+          const int* pd = s_pend + 4 * (k - (whole ? 1 : 0));
+          int ft = t, cf = c, cl = c, u0 = e.q, du = 4;
+          if (!wh) {
+            ft = pd[0];
+            cf = pd[1];
+            cl = pd[2];
+            const bool full = pd[3] != 0;
+            if (!share) {
+              finish = full;
             } else {
-              // contributors in order (deterministic sum), four partials' loads in flight at once
-              const bool pre_h = (ph.kind == kMkO || ph.kind == kMkDown) && t != e.hpre_tile;
-              for (int ch = 0; ch < n_ch; ++ch) {
-                float v[16], hv[16];
-#pragma unroll
-                for (int jj = 0; jj < 16; ++jj) {
-                  v[jj] = 0.f;
-                  hv[jj] = pre_h && ch * 16 + jj < e.M
-                               ? __ldcg(&p.h[static_cast<size_t>(e.rows[ch * 16 + jj]) * p.d + t * 128 + r])
-                               : 0.f;
-                }
-                for (int c0 = cf; c0 <= cl; c0 += 4) {
-                  float pv[4][16];
-#pragma unroll
-                  for (int q = 0; q < 4; ++q) {
-                    const bool cin = c0 + q <= cl;
-                    const float* pa = partials + static_cast<size_t>(c0 + q + t) * 128 * n_pad;
-#pragma unroll
-                    for (int jj = 0; jj < 16; ++jj)
-                      pv[q][jj] = cin && ch * 16 + jj < e.M ? __ldcg(&pa[(ch * 16 + jj) * 128 + r]) : 0.f;
-                  }
-#pragma unroll
-                  for (int q = 0; q < 4; ++q)
-#pragma unroll
-                    for (int jj = 0; jj < 16; ++jj) v[jj] += pv[q][jj];
-                }
-                mk_epilogue_chunk(p, ph, e, t, r, ch, v, pre_h ? hv : nullptr);
+              const bool all = e.et == 0 && !full ? mk_wait_count(&counters[ft], cl - cf + 1, sh) : true;
+              ok = bar_and(1, 128, all);
+              if (!ok) break;
+              finish = true;
+              u0 = 4 * (c - cf) + e.q;
+              du = 4 * (cl - cf + 1);
+            }
+          }
+          if (!finish) continue;
+          if (tr_last) mk_trace(p, kMkTraceSub + pi * 8 + 3);
+          if (share)
+            mk_finish_rows<D, 4, 5>(p, ph, e, ft, wh, tb, &acce[buf], u0, du, cf, cl, partials, n_pad);
+          else
+            mk_finish_rows<D, 2, 8>(p, ph, e, ft, wh, tb, &acce[buf], u0, du, cf, cl, partials, n_pad);
+          if (tr_last) mk_trace(p, kMkTraceSub + pi * 8 + 4);
+          named_bar_sync(1, 128);  // the tile's outputs precede the release below
+          if (tr_last) mk_trace(p, kMkTraceSub + pi * 8 + 6);
+          if (e.et == 0) {
+            bool publish = true;
+            if (share && !wh) {
+              publish = atom_add_acq_rel_gpu(&done[ft], 1) == cl - cf;
+              if (publish) {
+                atomicExch(&counters[ft], 0);
+                atomicExch(&done[ft], 0);
               }
             }
-            if (tr_last) mk_trace(p, kMkTraceSub + pi * 8 + 4);
+            unsigned long long* flag = mk_tile_flag(p, ph.kind, ft);
+            // (fault injection for the timeout path: the first h tile of the first layer's down
+            // phase is never flagged, so its consumers' bounded waits run out)
+            const bool withheld = p.withhold_flag && ph.kind == kMkDown && ph.slot == 0 && ft == 0;
+            if (publish && flag && !withheld) st_release_u64(flag, mk_seq(p.seq_base, ph.slot, ph.kind));
           }
         }
-        if (finalize) {
-          unsigned long long* flag = mk_tile_flag(p, ph.kind, t);
-          if ((ph.kind == kMkO || ph.kind == kMkDown) && !e.direct_xn) {
-            named_bar_sync(1, 128);  // h of this tile is final for every row of the phase
-            mk_write_next_xn(p, pl, ph, e, t, r);
-          }
-          if (tr_last) mk_trace(p, kMkTraceSub + pi * 8 + 5);
-          named_bar_sync(1, 128);  // the tile's outputs precede the flag's release
-          if (tr_last) mk_trace(p, kMkTraceSub + pi * 8 + 6);
-          // (fault injection for the timeout path: the first h tile of the first layer's down
-          // phase is never flagged, so its consumers' bounded waits run out)
-          const bool withheld = p.withhold_flag && ph.kind == kMkDown && ph.slot == 0 && t == 0;
-          if (flag && e.et == 0 && !withheld) st_release_u64(flag, mk_seq(p.seq_base, ph.slot, ph.kind));
+        if (n_fin > (whole ? 1 : 0)) {
+          n_pend = 0;
+          if (!share) named_bar_sync(1, 128);  // s_pend is rewritten by the next segment
         }
         if (e.et == 0 && seg.done()) mk_trace(p, pi * 8 + 7);
         ++use;
