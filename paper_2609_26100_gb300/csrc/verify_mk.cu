@@ -14,7 +14,7 @@
 //               bf16(h * g) for QKV / gate-up / LM head, the attention output for O, the SwiGLU
 //               activations for down.
 //   warp 3      attention only.
-//   warps 4-7   epilogues (TMEM -> registers, stream-K fixup, fused op).
+//   warps 4-7   epilogues (TMEM -> registers, stream-K fix-up, fused op).
 // All roles run one loop over the phases; at each O phase (when the attention runs in this
 // kernel) the eight warps first run the layer's attention items together, in the ring that every
 // role has stopped using by then.
@@ -238,7 +238,8 @@ __device__ __forceinline__ MkSeg mk_seg(const MkParams& p, const MkPhase& ph, in
   s.geff = static_cast<int>(s.T < G ? s.T : G);
   // Few short tiles (small models): whole tiles when streaming one takes at most kMkWholeKb
   // k-blocks (16 KiB, about 0.23 us each) more than a CTA's even share -- about what the partial
-  // sums' store, counter and reload cost.
+  // sums' store, counter and reload cost (the tiny decoder's tiles of 4 k-blocks, split over 4
+  // CTAs: 6.5 us from MMA to flag against 3 us whole).
   if (s.whole < 0 && n_split <= G && ph.kb <= s.T / s.geff + kMkWholeKb) s.geff = n_split;
   if (c >= s.geff) {
     s.it = s.it1 = 0;
@@ -412,6 +413,10 @@ __device__ __forceinline__ bool mk_resid(const MkPhase& ph) { return ph.kind == 
 //          of turns; the accumulator buffer is released after the last read;
 //   else:  the partials of contributors cf..cl, added in that order (deterministic), CB of them per
 //          round of loads.
+// Bound: issue of one warp per scheduler (a row's exponentials, divisions, splits and shuffles) and,
+// for partials, one L2 round trip per round.  In row form a 61-row whole tile of gate/up takes
+// 5.3 us and a 6-row one 1.4 us (9.8 and 2.3 us with a division and an address computation per
+// element and a barrier pair per 16 rows of one thread per feature).
 template <int D, int G, int CB>
 __device__ void mk_finish_rows(const MkParams& p, const MkPhase& ph, const MkEpi& e, int t, bool whole, uint32_t tb,
                                uint64_t* acce, int u0, int du, int cf, int cl, const float* partials, int n_pad) {
@@ -1082,8 +1087,12 @@ __global__ void __launch_bounds__(kMkThreads, 1)
       }
       // Tiles whose k-blocks several CTAs share: with up to 8 rows the last CTA to arrive finishes
       // the tile (two rows a warp, one round of loads).  With more rows that CTA would be busy for
-      // many rounds while the others wait, so every contributor waits for the tile's partial sums
-      // and finishes its own share of the rows, once its last split segment is stored.
+      // many rounds while the others wait -- the 32 tiles of an O phase on 32 of 152 SMs, 34 us after
+      // the last MMA for 144 rows -- so every contributor waits for the tile's partial sums and
+      // finishes its own share of the rows, once its last split segment is stored (18 us; and
+      // QKV 47 -> 25, down 31 -> 14 us).  Waiting costs a round trip more, so up to 8 rows, which
+      // one CTA finishes in a single round, stay with the last arriver.  No CTA waits before it
+      // has stored every partial sum of the phase that others wait for, and all are resident.
       const bool share = e.M > 8;
       int n_pend = 0;
       int t, k0, k1;
