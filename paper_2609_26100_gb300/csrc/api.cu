@@ -147,6 +147,8 @@ struct tss_ctx {
   int* pf_tok = nullptr;
   int *pf_pos = nullptr, *pf_slot = nullptr;
   int4* pf_qt = nullptr;
+  float* pf_part = nullptr;  // parts of split GEMM items, and their arrival counters
+  int* pf_cnt = nullptr;
   CUtensorMap pf_tm_xh, pf_tm_xl, pf_tm_qh, pf_tm_ql, pf_tm_ah, pf_tm_al, pf_tm_uh, pf_tm_ul;
   unsigned long long* trace = nullptr;  // persistent-kernel timeline when TSS_TRACE is set
   unsigned long long wait_ns = 2000000000ull;  // bound of the persistent kernel's waits (TSS_WAIT_LIMIT_MS)
@@ -1036,6 +1038,8 @@ tss_status pf_workspaces(tss_ctx* c) {
   TSS_TRY(c->alloc(&c->pf_pos, T));
   TSS_TRY(c->alloc(&c->pf_slot, T));
   TSS_TRY(c->alloc(&c->pf_qt, T / 128));
+  TSS_TRY(c->alloc(&c->pf_part, pf_partial_floats(c->num_sms)));
+  TSS_TRY(c->alloc(&c->pf_cnt, pf_counters(c->num_sms)));
   // (rows past a pass's rows are read by the last tile of each GEMM and attention: finite)
   TSS_CU(cudaMemset(c->pf_xh, 0, T * d * 2));
   TSS_CU(cudaMemset(c->pf_xl, 0, T * d * 2));
@@ -1087,6 +1091,9 @@ tss_status pf_pass(tss_ctx* c, int T, int n_qtiles, unsigned long long skip, con
   p.uh = c->pf_uh;
   p.ul = c->pf_ul;
   p.u_ld = c->F_pad;
+  p.partials = c->pf_part;
+  p.counters = c->pf_cnt;
+  p.n_counters = pf_counters(c->num_sms);
   p.rope_cos = c->rope_cos;
   p.rope_sin = c->rope_sin;
   p.status = c->d_status;
@@ -1102,15 +1109,15 @@ tss_status pf_pass(tss_ctx* c, int T, int n_qtiles, unsigned long long skip, con
     p.kv = static_cast<__nv_bfloat16*>(kv->layer[l]);
     TSS_CU(launch_pf_norm(p, c->g_attn + static_cast<size_t>(l) * d, s));
     TSS_CU(launch_pf_gemm(kPfEpiQkv, c->pf_tm_xh, c->pf_tm_xl, p,
-                          PfGemm{c->wqkv, static_cast<long long>(3 * dd), l, 3 * d / 128, kbd, inject ? 1 : 0}, G, s));
+                          PfGemm{c->wqkv, static_cast<long long>(3 * dd), l, 3 * d / 128, kbd, inject ? 1 : 0, 0, 0}, G, s));
     inject = false;
     TSS_CU(launch_pf_attn(c->pf_tm_qh, c->pf_tm_ql, tkv, p, s));
-    TSS_CU(launch_pf_gemm(kPfEpiResid, c->pf_tm_ah, c->pf_tm_al, p, PfGemm{c->wo, static_cast<long long>(dd), l, d / 128, kbd, 0}, G, s));
+    TSS_CU(launch_pf_gemm(kPfEpiResid, c->pf_tm_ah, c->pf_tm_al, p, PfGemm{c->wo, static_cast<long long>(dd), l, d / 128, kbd, 0, 0, 0}, G, s));
     TSS_CU(launch_pf_norm(p, c->g_mlp + static_cast<size_t>(l) * d, s));
     TSS_CU(launch_pf_gemm(kPfEpiSwiglu, c->pf_tm_xh, c->pf_tm_xl, p,
-                          PfGemm{c->wgu, static_cast<long long>(c->Ft) * 128 * d, l, c->Ft, kbd, 0}, G, s));
+                          PfGemm{c->wgu, static_cast<long long>(c->Ft) * 128 * d, l, c->Ft, kbd, 0, 0, 0}, G, s));
     TSS_CU(launch_pf_gemm(kPfEpiResid, c->pf_tm_uh, c->pf_tm_ul, p,
-                          PfGemm{c->wdown, static_cast<long long>(d) * c->F_pad, l, d / 128, c->F_pad / 64, 0}, G, s));
+                          PfGemm{c->wdown, static_cast<long long>(d) * c->F_pad, l, d / 128, c->F_pad / 64, 0, 0, 0}, G, s));
   }
   return TSS_OK;
 }

@@ -118,6 +118,9 @@ struct PfParams {
   __nv_bfloat16* kv;               // this layer's cache [n_slots][2][H][cap][D]
   const float* rope_cos;           // [max_positions][D / 2]
   const float* rope_sin;
+  float* partials;                 // parts of split GEMM items: [CTA][2][weight tile][token][weight row]
+  int* counters;                   // [n_counters] arrivals per split item (zero between launches)
+  int n_counters;
   int* status;
 };
 struct PfGemm {
@@ -125,12 +128,15 @@ struct PfGemm {
   long long w_layer_elems;
   int layer, n_o, kb;              // layer, 128-row weight tiles, 64-column k-blocks
   int withhold;                    // fault injection: CTA 0 issues no MMA (its waits run out)
+  int n_sk, geff;                  // items split over the first geff CTAs (set by the launch)
 };
+size_t pf_partial_floats(int sms);
+int pf_counters(int sms);
 cudaError_t pf_prepare();
 cudaError_t launch_pf_embed(const PfParams& p, cudaStream_t s);
 cudaError_t launch_pf_norm(const PfParams& p, const float* g, cudaStream_t s);
 cudaError_t launch_pf_gemm(int epi, const CUtensorMap& xh, const CUtensorMap& xl, const PfParams& p, const PfGemm& g,
-                           int grid, cudaStream_t s);
+                           int sms, cudaStream_t s);
 cudaError_t launch_pf_attn(const CUtensorMap& qh, const CUtensorMap& ql, const CUtensorMap& kv, const PfParams& p,
                            cudaStream_t s);
 

@@ -13,7 +13,7 @@
 // 128 tokens on the N side; a CTA takes two weight tiles against one token tile at a time (two
 // accumulators sharing the token operand) through its whole K loop (no split); items are taken
 // weight-pair-major by a persistent grid so that the CTAs working at the same time share weight
-// tiles through L2; four groups of epilogue warps keep up with the MMAs.  X is held as two bf16
+// tiles through L2; three groups of epilogue warps keep up with the MMAs.  X is held as two bf16
 // parts (hi = bf16(x), lo = bf16(x - hi)), both multiplied by the weights into one fp32
 // accumulator in tensor memory, as on the verification path.  Attention (pf_attn_kernel): one CTA
 // per (head, 128-query tile of one request), queries on the MMA's M side, 64-key tiles of the
@@ -26,7 +26,8 @@ namespace tss {
 namespace {
 
 constexpr int kPfThreads = 192;  // attention: warp 0 TMA, warp 1 MMA (+ TMEM), warps 2-5 softmax
-constexpr int kPgGroups = 4;     // GEMM epilogue groups of four warps (one per TMEM lane quarter)
+constexpr int kPgGroups = 3;     // GEMM epilogue groups of four warps (one per TMEM lane quarter): 14 warps
+                                 // leave a thread 128 registers (four groups: 96, with spills)
 constexpr int kPgThreads = 64 + 128 * kPgGroups;  // warp 0 copies, warp 1 MMA (+ TMEM), then the epilogue groups
 constexpr int kPfStages = 3;
 constexpr uint32_t kPfA = 128 * 64 * 2;      // weight block: 16 KiB
@@ -40,10 +41,16 @@ __host__ __device__ inline size_t pf_gemm_smem() {
 
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
-__device__ __forceinline__ void pf_split_store(__nv_bfloat16* hi, __nv_bfloat16* lo, size_t i, float x) {
-  const __nv_bfloat16 h = __float2bfloat16_rn(x);
-  hi[i] = h;
-  lo[i] = __float2bfloat16_rn(x - __bfloat162float(h));
+// Four consecutive elements as bf16 hi and lo parts: one 8-byte store each.
+__device__ __forceinline__ void pf_split_store4(__nv_bfloat16* hi, __nv_bfloat16* lo, size_t i, const float* x) {
+  uint32_t h[2], l[2];
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    h[k] = pack_bf16(x[2 * k], x[2 * k + 1]);
+    l[k] = pack_bf16(x[2 * k] - __uint_as_float(h[k] << 16), x[2 * k + 1] - __uint_as_float(h[k] & 0xffff0000u));
+  }
+  *reinterpret_cast<uint2*>(hi + i) = make_uint2(h[0], h[1]);
+  *reinterpret_cast<uint2*>(lo + i) = make_uint2(l[0], l[1]);
 }
 
 }  // namespace
@@ -53,6 +60,8 @@ __device__ __forceinline__ void pf_split_store(__nv_bfloat16* hi, __nv_bfloat16*
 // ---------------------------------------------------------------------------------------------
 __global__ void pf_embed_kernel(const PfParams p) {
   const int j = blockIdx.x;
+  if (j == 0)  // the GEMMs' arrival counters start every pass at zero, even after one that gave up on a wait
+    for (int i = threadIdx.x; i < p.n_counters; i += blockDim.x) p.counters[i] = 0;
   if (j >= p.T) return;
   int tok = p.tokens[j];
   if (tok < 0 || tok >= p.vocab) {
@@ -134,87 +143,151 @@ __device__ __forceinline__ bool pf_epi_or(bool v) {
   return r != 0;
 }
 
-// One 16-token chunk (tokens j0 .. j0 + 15) of output row r of weight tile t; xch: [16][128]
-// exchange (the group's own, synchronised by named barrier `bar` of its 128 threads) for the row
-// pairs of RoPE (r, r ^ head_dim / 2) and SwiGLU (gate r, up r + 64).
+// The fused epilogue of 4 tokens j0 .. j0 + 3 of weight tile t in row form: a warp per 4 tokens, lane
+// l holds features f0 = 4 l .. f0 + 3 of each, so that the partners of RoPE (feature ^ 64) and SwiGLU
+// (gate f, up f + 64) sit in lane ^ 16 and every access is an 8- or 16-byte vector.  pre() requests what
+// the tokens need from global memory; finish() takes the sums.  With a thread per feature and a
+// branch, a position load and 2-byte stores per element, a 16-token chunk of QKV took 8-10 us and
+// bound the GEMM at short prompts (QKV at 200 tokens 81 us, in this form 58; O at 4096 tokens, with
+// the residual's 16 dependent loads and stores, 215 us, 172 with its loads first and its items split).
 template <int EPI>
-__device__ __forceinline__ void pf_epilogue(const PfParams& p, const PfGemm& g, float* xch, int t, int r, int j0,
-                                            const float* v, int bar) {
-  if constexpr (EPI == kPfEpiResid) {
-    const int o = t * 128 + r;
+struct PfRows {
+  int4 pos, slot;      // QKV: the tokens' positions (-1: gap row) and KV slots
+  float4 c[4], s[4];   // QKV, q and k: rotation factors; residual: h in c
+  __device__ __forceinline__ void pre(const PfParams& p, int t, int j0, int f0) {
+    if constexpr (EPI == kPfEpiResid) {
 #pragma unroll
-    for (int jj = 0; jj < 16; ++jj) {
-      const int j = j0 + jj;
-      if (j < p.T) p.h[static_cast<size_t>(j) * p.d_model + o] += v[jj];
-    }
-  } else if constexpr (EPI == kPfEpiQkv) {
-    const int d = p.d_model, D = p.head_dim, half = D >> 1;
-    const int o = t * 128 + r;
-    const int sec = o / d;  // 0: q, 1: k, 2: v (uniform over the tile: d is a multiple of 128)
-    const int f = o - sec * d;
-    const int head = f / D, dim = f - head * D;
-    float out[16];
-    if (sec < 2) {
+      for (int i = 0; i < 4; ++i)
+        c[i] = *reinterpret_cast<const float4*>(p.h + static_cast<size_t>(j0 + i) * p.d_model + t * 128 + f0);
+    } else if constexpr (EPI == kPfEpiQkv) {
+      pos = *reinterpret_cast<const int4*>(p.row_pos + j0);
+      slot = *reinterpret_cast<const int4*>(p.row_slot + j0);
+      if (t * 128 < 2 * p.d_model) {
+        const int ps[4] = {pos.x, pos.y, pos.z, pos.w};
 #pragma unroll
-      for (int jj = 0; jj < 16; ++jj) xch[jj * 128 + r] = v[jj];
-      named_bar_sync(bar, 128);
-      const int pr = r ^ half, i = dim & (half - 1);
-#pragma unroll
-      for (int jj = 0; jj < 16; ++jj) {
-        const int pos = j0 + jj < p.T ? p.row_pos[j0 + jj] : -1;
-        out[jj] = 0.f;
-        if (pos >= 0) {
-          const float c = p.rope_cos[static_cast<size_t>(pos) * half + i];
-          const float s = p.rope_sin[static_cast<size_t>(pos) * half + i];
-          const float pv = xch[jj * 128 + pr];
-          out[jj] = dim < half ? v[jj] * c - pv * s : v[jj] * c + pv * s;
-        }
-      }
-      named_bar_sync(bar, 128);
-    } else {
-#pragma unroll
-      for (int jj = 0; jj < 16; ++jj) out[jj] = v[jj];
-    }
-#pragma unroll
-    for (int jj = 0; jj < 16; ++jj) {
-      const int j = j0 + jj;
-      if (j >= p.T) continue;
-      const int pos = p.row_pos[j];
-      if (pos < 0) continue;  // gap row
-      if (sec == 0) {
-        pf_split_store(p.qh, p.ql, static_cast<size_t>(j) * d + f, out[jj]);
-      } else {
-        const size_t row =
-            ((static_cast<size_t>(p.row_slot[j]) * 2 + (sec - 1)) * p.n_heads + head) * static_cast<size_t>(p.kv_cap) +
-            static_cast<size_t>(pos);
-        p.kv[row * D + dim] = __float2bfloat16_rn(out[jj]);
-      }
-    }
-  } else if constexpr (EPI == kPfEpiSwiglu) {
-#pragma unroll
-    for (int jj = 0; jj < 16; ++jj) xch[jj * 128 + r] = v[jj];
-    named_bar_sync(bar, 128);
-    if (r < 64) {
-      const int fcol = t * 64 + r;
-#pragma unroll
-      for (int jj = 0; jj < 16; ++jj) {
-        const int j = j0 + jj;
-        if (j < p.T) {
-          const float gt = v[jj], up = xch[jj * 128 + r + 64];
-          pf_split_store(p.uh, p.ul, static_cast<size_t>(j) * p.u_ld + fcol, gt / (1.f + expf(-gt)) * up);
+        for (int i = 0; i < 4; ++i) {
+          const size_t e = static_cast<size_t>(ps[i] < 0 ? 0 : ps[i]) * 64 + (f0 & 63);
+          c[i] = __ldg(reinterpret_cast<const float4*>(p.rope_cos + e));
+          s[i] = __ldg(reinterpret_cast<const float4*>(p.rope_sin + e));
         }
       }
     }
-    named_bar_sync(bar, 128);
   }
-  (void)g;
-}
+  __device__ __forceinline__ void finish(const PfParams& p, int t, int j0, int f0, const float (*v)[4]) const {
+    const int d = p.d_model;
+    if constexpr (EPI == kPfEpiResid) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        *reinterpret_cast<float4*>(p.h + static_cast<size_t>(j0 + i) * d + t * 128 + f0) =
+            make_float4(c[i].x + v[i][0], c[i].y + v[i][1], c[i].z + v[i][2], c[i].w + v[i][3]);
+    } else if constexpr (EPI == kPfEpiQkv) {
+      const int sec = t * 128 < d ? 0 : t * 128 < 2 * d ? 1 : 2;  // q, k or v (one per tile)
+      const int f = t * 128 - sec * d + f0, head = f >> 7;
+      const int ps[4] = {pos.x, pos.y, pos.z, pos.w}, sl[4] = {slot.x, slot.y, slot.z, slot.w};
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        float x[4] = {v[i][0], v[i][1], v[i][2], v[i][3]};
+        if (sec < 2) {
+          const float cs[4] = {c[i].x, c[i].y, c[i].z, c[i].w}, sn[4] = {s[i].x, s[i].y, s[i].z, s[i].w};
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            const float y = __shfl_xor_sync(0xffffffffu, v[i][k], 16);
+            x[k] = f0 < 64 ? x[k] * cs[k] - y * sn[k] : x[k] * cs[k] + y * sn[k];
+          }
+        }
+        if (ps[i] < 0) continue;  // gap row
+        if (sec == 0) {
+          pf_split_store4(p.qh, p.ql, static_cast<size_t>(j0 + i) * d + f, x);
+        } else {
+          const size_t row = ((static_cast<size_t>(sl[i]) * 2 + (sec - 1)) * p.n_heads + head) * static_cast<size_t>(p.kv_cap) +
+                             static_cast<size_t>(ps[i]);
+          *reinterpret_cast<uint2*>(p.kv + row * 128 + f0) = make_uint2(pack_bf16(x[0], x[1]), pack_bf16(x[2], x[3]));
+        }
+      }
+    } else {
+      // of two tokens the lower half-warp finishes the first and the upper the second
+      const bool upper = f0 >= 64;
+#pragma unroll
+      for (int i = 0; i < 4; i += 2) {
+        float a[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const float y = __shfl_xor_sync(0xffffffffu, upper ? v[i][k] : v[i + 1][k], 16);
+          const float gt = upper ? y : v[i][k], up = upper ? v[i + 1][k] : y;
+          a[k] = __fdividef(gt, 1.f + expf(-gt)) * up;
+        }
+        pf_split_store4(p.uh, p.ul, static_cast<size_t>(j0 + i + (upper ? 1 : 0)) * p.u_ld + t * 64 + (f0 & 63), a);
+      }
+    }
+  }
+};
 
 }  // namespace
 
 // Work item = (pair of weight tiles 2w, 2w + 1; token tile u): the two weight tiles share every
 // stage's token operand, so a stage of 64 KiB feeds 4 MMAs of 128 x 128 x 16 per k16 step (the
 // copy bytes per MMA are half those of one weight tile per item, which L2 bandwidth binds).
+//
+// Split of the items over the G CTAs (pf_plan): whole items round-robin leave SMs idle in the last
+// wave (512 items of an O or down projection at 4096 rows: 3.4 waves in 4) and all but a few SMs
+// idle on a short prompt (64 items at 512 rows).  So the first g.n_sk items -- fewer than two
+// waves -- are laid end to end and cut into equal ranges of k-blocks, one per CTA, and the rest
+// follow as whole items, one per CTA and wave.  A CTA's range starts and ends inside an item, at
+// most; such a part goes to the CTA's slot of partial sums, and once the CTA has stored its last
+// part, each contributor waits for the item's parts and finishes its own share of the item's 16
+// (weight tile, 16-token) units, adding the parts in CTA order.  Every CTA stores before it waits
+// and all are resident (cooperative launch), so the waits end.  Bound: the tensor pipe at full
+// passes (4096 rows of a 7B layer: QKV 541 -> 497, O 215 -> 172, gate/up 893 -> 841, down 508 -> 487 us
+// against whole items); at 200 tokens (O, down: 32 items) the parts' store, wait and reload, about
+// 20 us of each launch (a layer 470 -> 254 us).
+struct PfCursor {  // (a pass has at most 4096 / 128 x 32768 / 256 items and 2 x SMs x 512 split k-blocks)
+  uint32_t it, it1, dp, n_items;  // k-blocks of the split items still to take; next whole item
+  uint32_t kb, G;
+  __device__ __forceinline__ void start(const PfGemm& g, uint32_t items, uint32_t c, uint32_t grid) {
+    kb = g.kb;
+    G = grid;
+    const uint32_t T = g.n_sk * kb, geff = g.geff;
+    it = c < geff ? T * c / geff : 0;
+    it1 = c < geff ? T * (c + 1) / geff : 0;
+    dp = g.n_sk + c;
+    n_items = items;
+  }
+  __device__ __forceinline__ bool next(uint32_t& item, int& k0, int& k1) {
+    if (it < it1) {
+      item = it / kb;
+      const uint32_t i0 = item * kb;
+      k0 = static_cast<int>(it - i0);
+      k1 = static_cast<int>(min(kb, it1 - i0));
+      it += k1 - k0;
+      return true;
+    }
+    if (dp >= n_items) return false;
+    item = dp;
+    dp += G;
+    k0 = 0;
+    k1 = static_cast<int>(kb);
+    return true;
+  }
+};
+
+// Bounded wait for the arrivals of an item's parts.
+__device__ bool pf_wait_count(const int* f, int target, volatile int* abort, int* status) {
+  const uint64_t t0 = globaltimer_ns();
+  for (uint32_t i = 1;; ++i) {
+    int v;
+    asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(f) : "memory");
+    if (v >= target) return true;
+    if ((i & 63) == 0) {
+      if (*abort) return false;
+      if (globaltimer_ns() - t0 > kWaitLimitNs) {
+        *abort = 1;
+        report(status, kStatusTimeout);
+        return false;
+      }
+    }
+  }
+}
+
 template <int EPI>
 __global__ void __launch_bounds__(kPgThreads, 1) pf_gemm_kernel(const __grid_constant__ CUtensorMap tm_xh,
                                                                  const __grid_constant__ CUtensorMap tm_xl,
@@ -226,9 +299,9 @@ __global__ void __launch_bounds__(kPgThreads, 1) pf_gemm_kernel(const __grid_con
   __shared__ uint32_t tslot;
   __shared__ int abort_s;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int n_u = (p.T + 127) >> 7;         // token tiles
-  const int n_w = (g.n_o + 1) >> 1;         // weight-tile pairs (the last may hold one tile)
-  const long long n_items = static_cast<long long>(n_w) * n_u;
+  const uint32_t n_u = (p.T + 127) >> 7;    // token tiles
+  const uint32_t n_w = (g.n_o + 1) >> 1;    // weight-tile pairs (the last may hold one tile)
+  const uint32_t n_items = n_w * n_u;
   if (tid == 0) {
     for (int i = 0; i < kPfStages; ++i) {
       mbar_init(&full[i], 1);
@@ -259,12 +332,16 @@ __global__ void __launch_bounds__(kPgThreads, 1) pf_gemm_kernel(const __grid_con
       prefetch_tmap(&tm_xh);
       prefetch_tmap(&tm_xl);
       long long it = 0;
+      uint32_t item;
       bool ok = true;
-      for (long long item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
-        const int w = static_cast<int>(item / n_u), u = static_cast<int>(item - static_cast<long long>(w) * n_u);
+      int k0, k1;
+      PfCursor cur;
+      cur.start(g, n_items, blockIdx.x, gridDim.x);
+      while (ok && cur.next(item, k0, k1)) {
+        const int w = static_cast<int>(item / n_u), u = static_cast<int>(item) - w * n_u;
         const int t0 = 2 * w;
         const bool two = t0 + 1 < g.n_o;
-        for (int k = 0; k < g.kb; ++k, ++it) {
+        for (int k = k0; k < k1; ++k, ++it) {
           const int s = static_cast<int>(it % kPfStages);
           if (it >= kPfStages && !mbar_wait(&empty[s], static_cast<uint32_t>((it / kPfStages) - 1) & 1u, abort, p.status)) {
             ok = false;
@@ -289,18 +366,20 @@ __global__ void __launch_bounds__(kPgThreads, 1) pf_gemm_kernel(const __grid_con
     if (lane == 0) {
       const uint32_t idesc = idesc_bf16_m128(128);
       long long it = 0;
-      int n = 0;
-      bool ok = true;
+      uint32_t item;
+      int n = 0, k0, k1;
       // fault injection: CTA 0 issues no MMA, so its epilogue's first wait runs out
-      const long long n_issue = g.withhold && blockIdx.x == 0 ? 0 : n_items;
-      for (long long item = blockIdx.x; item < n_issue && ok; item += gridDim.x, ++n) {
+      bool ok = !(g.withhold && blockIdx.x == 0);
+      PfCursor cur;
+      cur.start(g, n_items, blockIdx.x, gridDim.x);
+      for (; ok && cur.next(item, k0, k1); ++n) {
         const int w = static_cast<int>(item / n_u);
         const bool two = 2 * w + 1 < g.n_o;
         const int buf = n & 1;
         if (n >= 2 && !mbar_wait(&acc_empty[buf], static_cast<uint32_t>((n >> 1) - 1) & 1u, abort, p.status)) break;
         tc_fence_after();
         const uint32_t d0 = tm + buf * 2 * kPfAccCols, d1 = d0 + kPfAccCols;
-        for (int k = 0; k < g.kb; ++k, ++it) {
+        for (int k = k0; k < k1; ++k, ++it) {
           const int s = static_cast<int>(it % kPfStages);
           if (!mbar_wait(&full[s], static_cast<uint32_t>(it / kPfStages) & 1u, abort, p.status)) {
             ok = false;
@@ -312,11 +391,11 @@ __global__ void __launch_bounds__(kPgThreads, 1) pf_gemm_kernel(const __grid_con
           for (int k16 = 0; k16 < 4; ++k16) {
             const uint64_t bh = sdesc_sw128(b + k16 * 32), bl = sdesc_sw128(b + kPfB + k16 * 32);
             const uint64_t a0 = sdesc_sw128(a + k16 * 32);
-            umma_bf16(d0, a0, bh, idesc, (k | k16) ? 1u : 0u);
+            umma_bf16(d0, a0, bh, idesc, (k > k0 || k16) ? 1u : 0u);
             umma_bf16(d0, a0, bl, idesc, 1u);
             if (two) {
               const uint64_t a1 = sdesc_sw128(a + kPfA + k16 * 32);
-              umma_bf16(d1, a1, bh, idesc, (k | k16) ? 1u : 0u);
+              umma_bf16(d1, a1, bh, idesc, (k > k0 || k16) ? 1u : 0u);
               umma_bf16(d1, a1, bl, idesc, 1u);
             }
           }
@@ -332,31 +411,107 @@ __global__ void __launch_bounds__(kPgThreads, 1) pf_gemm_kernel(const __grid_con
     }
   } else {
     // ---------------- epilogue warps: TMEM lane quarter = warp & 3, thread r = weight row; group
-    // (warp - 2) / 4 takes its share of the 8 token chunks of each accumulator ----------------
-    constexpr int kCh = 8 / kPgGroups;
-    const int q = warp & 3, r = q * 32 + lane, grp = (warp - 2) >> 2;
+    // (warp - 2) / 4 takes every kPgGroups-th of the item's 16-token chunks ----------------
+    const int q = warp & 3, r = q * 32 + lane, grp = (warp - 2) >> 2, f0 = 4 * lane;
     float* xch = xch0 + grp * 16 * 128;
     const int bar = grp == 0 ? 1 : 2 + grp;  // (2 is the vote barrier)
-    int n = 0;
-    for (long long item = blockIdx.x; item < n_items; item += gridDim.x, ++n) {
-      const int w = static_cast<int>(item / n_u), u = static_cast<int>(item - static_cast<long long>(w) * n_u);
+    const uint32_t T = g.n_sk * g.kb, geff = g.geff;
+    auto cta_of = [&](uint32_t i) { return static_cast<int>(((i + 1) * geff - 1) / T); };
+    // slot of CTA cc's part of split item x: its first part, or its last when its range begins earlier
+    auto slot_of = [&](uint32_t cc, uint32_t x) { return 2 * cc + (T * cc / geff < x * g.kb ? 1 : 0); };
+    constexpr size_t kSlot = static_cast<size_t>(2) * 128 * 128;  // floats: [tile of the pair][token][weight row]
+    int n = 0, n_pend = 0, k0, k1;
+    uint32_t item, pend[2] = {0, 0};
+    PfCursor cur;
+    cur.start(g, n_items, blockIdx.x, gridDim.x);
+    for (; cur.next(item, k0, k1); ++n) {
+      const int w = static_cast<int>(item / n_u), u = static_cast<int>(item) - w * n_u;
       const int buf = n & 1;
+      const bool whole = k0 == 0 && k1 == g.kb;
       const bool ok = mbar_wait(&acc_full[buf], static_cast<uint32_t>(n >> 1) & 1u, abort, p.status);
       if (pf_epi_or(!ok)) break;
       tc_fence_after();
-      for (int a = 0; a < 2; ++a) {
-        const int t = 2 * w + a;
-        if (t >= g.n_o) break;
-        const uint32_t tb = tm + (static_cast<uint32_t>(q * 32) << 16) + (buf * 2 + a) * kPfAccCols;
-        for (int ch = kCh * grp; ch < kCh * grp + kCh; ++ch) {
-          float v[16];
-          tmem_ld16(tb + ch * 16, v);
-          pf_epilogue<EPI>(p, g, xch, t, r, u * 128 + ch * 16, v, bar);
+      float* part = p.partials + (whole ? 0 : slot_of(blockIdx.x, item)) * kSlot;
+      const int units = 2 * w + 1 < g.n_o ? 16 : 8;  // 16-token chunks of both accumulators
+      for (int y = grp; y < units; y += kPgGroups) {
+        const int a = y >> 3, ch = y & 7, t = 2 * w + a;
+        const int j0 = u * 128 + ch * 16 + 4 * q;  // this warp's tokens of the chunk
+        PfRows<EPI> rows;
+        if (whole) rows.pre(p, t, j0, f0);
+        float v[16];
+        tmem_ld16(tm + (static_cast<uint32_t>(q * 32) << 16) + (buf * 2 + a) * kPfAccCols + ch * 16, v);
+        if (whole) {
+#pragma unroll
+          for (int jj = 0; jj < 16; ++jj) xch[jj * 128 + r] = v[jj];
+          named_bar_sync(bar, 128);
+          float x[4][4];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const float4 z = *reinterpret_cast<const float4*>(xch + (4 * q + i) * 128 + f0);
+            x[i][0] = z.x; x[i][1] = z.y; x[i][2] = z.z; x[i][3] = z.w;
+          }
+          named_bar_sync(bar, 128);
+          rows.finish(p, t, j0, f0, x);
+        } else {
+#pragma unroll
+          for (int jj = 0; jj < 16; ++jj) __stcg(&part[(a * 128 + ch * 16 + jj) * 128 + r], v[jj]);
         }
       }
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(&acc_empty[buf]);
+      if (!whole) {
+        pf_epi_or(false);  // every thread's part precedes the release below
+        if (tid == 64) atom_add_acq_rel_gpu(&p.counters[item], 1);
+        pend[n_pend++] = item;  // (at most two: a range's first and last items)
+      }
+      if (n_pend == 0 || cur.it < cur.it1) continue;
+      bool failed = false;
+      for (int x = 0; x < n_pend && !failed; ++x) {
+        const uint32_t pi = pend[x];
+        const int pw = static_cast<int>(pi / n_u), pu = static_cast<int>(pi) - pw * n_u;
+        const int cf = cta_of(pi * g.kb), cl = cta_of((pi + 1) * g.kb - 1), nc = cl - cf + 1;
+        const bool all = tid != 64 || pf_wait_count(&p.counters[pi], nc, abort, p.status);
+        failed = pf_epi_or(!all);
+        if (failed) break;
+        if (tid == 64 && atomicAdd(&p.counters[g.n_sk + pi], 1) == nc - 1) {  // every contributor has seen the count
+          p.counters[pi] = 0;
+          p.counters[g.n_sk + pi] = 0;
+        }
+        const int n_units = 2 * pw + 1 < g.n_o ? 16 : 8;
+        for (int y = static_cast<int>(blockIdx.x) - cf + nc * grp; y < n_units; y += nc * kPgGroups) {
+          const int a = y >> 3, ch = y & 7;
+          const int t = 2 * pw + a, j0 = pu * 128 + ch * 16 + 4 * q;
+          PfRows<EPI> rows;
+          // two contributors' parts per round of loads, the first round before the epilogue's own loads
+          float x[4][4];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) x[i][0] = x[i][1] = x[i][2] = x[i][3] = 0.f;
+          for (int cc = cf; cc <= cl; cc += 2) {
+            float4 part2[2][4];
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+              const float* pp = p.partials + slot_of(min(cc + k, cl), pi) * kSlot + (a * 128 + ch * 16 + 4 * q) * 128 + f0;
+#pragma unroll
+              for (int i = 0; i < 4; ++i)
+                part2[k][i] = cc + k <= cl ? __ldcg(reinterpret_cast<const float4*>(pp + i * 128)) : make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+            if (cc == cf) rows.pre(p, t, j0, f0);
+#pragma unroll
+            for (int k = 0; k < 2; ++k)
+#pragma unroll
+              for (int i = 0; i < 4; ++i) {
+                x[i][0] += part2[k][i].x;
+                x[i][1] += part2[k][i].y;
+                x[i][2] += part2[k][i].z;
+                x[i][3] += part2[k][i].w;
+              }
+          }
+          rows.finish(p, t, j0, f0, x);
+        }
+      }
+      n_pend = 0;
+      if (failed) break;
     }
   }
   __syncwarp();
@@ -706,14 +861,50 @@ cudaError_t launch_pf_norm(const PfParams& p, const float* g, cudaStream_t s) {
   return launch_k(pf_norm_kernel, dim3(p.T), dim3(256), 0, s, false, p, g);
 }
 
+// The items that are split (see pf_gemm_kernel) and the CTAs sharing them.  Whole items only, where
+// the CTA with the most of them has at most kPfWhole k-blocks (about 0.55 us each) more than an
+// even share: about what storing, counting and adding the parts costs (three layers, us, with
+// 12 / 20 / 28 / 40 k-blocks: 7B 200 tokens 762 / 762 / 803 / 803, 384 tokens 970 / 925 / 925 / 925,
+// 13B 866 tokens 2556 / 2307 / 2306 / 2316).
+int pf_plan(PfGemm* g, int T, int sms) {
+  constexpr long long kPfWhole = 20;
+  const long long items = static_cast<long long>((g->n_o + 1) / 2) * ((T + 127) / 128);
+  const long long even = (items * g->kb + sms - 1) / sms, whole = (items + sms - 1) / sms * g->kb;
+  g->n_sk = 0;
+  g->geff = 1;
+  if (whole <= even + kPfWhole) return static_cast<int>(items < sms ? items : sms);
+  const long long waves = items / sms;
+  g->n_sk = static_cast<int>(items - (waves >= 2 ? (waves - 1) * sms : 0));
+  const long long blocks = static_cast<long long>(g->n_sk) * g->kb;
+  g->geff = static_cast<int>(blocks < sms ? blocks : sms);
+  return g->geff;  // (whole items follow only where every CTA has a range)
+}
+
+size_t pf_partial_floats(int sms) { return static_cast<size_t>(2) * sms * 2 * 128 * 128; }
+int pf_counters(int sms) { return 4 * sms; }
+
+template <int EPI>
+cudaError_t launch_pf_gemm_epi(const CUtensorMap& xh, const CUtensorMap& xl, const PfParams& p, PfGemm g, int sms,
+                               cudaStream_t s) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(pf_plan(&g, p.T, sms));
+  cfg.blockDim = dim3(kPgThreads);
+  cfg.dynamicSmemBytes = pf_gemm_smem();
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeCooperative;  // all CTAs resident: contributors wait for one another
+  attr[0].val.cooperative = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = g.n_sk > 0 ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, pf_gemm_kernel<EPI>, xh, xl, p, g);
+}
+
 cudaError_t launch_pf_gemm(int epi, const CUtensorMap& xh, const CUtensorMap& xl, const PfParams& p, const PfGemm& g,
-                           int grid, cudaStream_t s) {
-  const long long tiles = static_cast<long long>((g.n_o + 1) / 2) * ((p.T + 127) / 128);
-  const dim3 gr(static_cast<unsigned>(tiles < grid ? tiles : grid)), blk(kPgThreads);
+                           int sms, cudaStream_t s) {
   switch (epi) {
-    case kPfEpiQkv: return launch_k(pf_gemm_kernel<kPfEpiQkv>, gr, blk, pf_gemm_smem(), s, false, xh, xl, p, g);
-    case kPfEpiResid: return launch_k(pf_gemm_kernel<kPfEpiResid>, gr, blk, pf_gemm_smem(), s, false, xh, xl, p, g);
-    case kPfEpiSwiglu: return launch_k(pf_gemm_kernel<kPfEpiSwiglu>, gr, blk, pf_gemm_smem(), s, false, xh, xl, p, g);
+    case kPfEpiQkv: return launch_pf_gemm_epi<kPfEpiQkv>(xh, xl, p, g, sms, s);
+    case kPfEpiResid: return launch_pf_gemm_epi<kPfEpiResid>(xh, xl, p, g, sms, s);
+    case kPfEpiSwiglu: return launch_pf_gemm_epi<kPfEpiSwiglu>(xh, xl, p, g, sms, s);
     default: return cudaErrorInvalidValue;
   }
 }

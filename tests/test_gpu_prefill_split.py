@@ -1,0 +1,49 @@
+"""GPU parity of the prefill GEMMs where their work items are split between CTAs: a decoder of
+d 2048 and MLP 2880 (45 gate/up tiles, so the last pair holds one) with prompts from one token tile
+(few items, each shared by many CTAs) to a full pass (whole waves after the split items)."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import tss_oracle as O
+from paper_2609_26100_gb300 import native, synth
+from tests.conftest import oracle_weights
+from tests.parity_util import to_device_weights
+
+pytestmark = pytest.mark.gpu
+
+SEED = synth.DEFAULT_SEED
+ARCH = synth.Arch(n_layers=2, d_model=2048, n_heads=16, head_dim=128, d_mlp=2880, vocab=512)
+
+
+@pytest.fixture(scope="module")
+def weights():
+    from paper_2609_26100_gb300 import build
+    build.build()
+    w = synth.make_weights(ARCH, device="cuda")
+    return oracle_weights(to_device_weights(w, "cpu")), w
+
+
+@pytest.mark.parametrize("lengths", [[1], [128], [129, 70], [700], [1900, 1500, 300]])
+def test_split_prefill_matches_oracle(weights, lengths):
+    """K and V rows of both layers (the second layer's depend on every projection of the first),
+    twice into the same cache with the same bits."""
+    from paper_2609_26100_gb300.runner import TssRunner
+    wo, wg = weights
+    run = TssRunner(ARCH, wg, n_slots=len(lengths), kv_cap=2048, max_batch=len(lengths))
+    prompts = [synth.uniform_ints(n, ARCH.vocab, SEED, f"split.{b}").tolist() for b, n in enumerate(lengths)]
+    got = []
+    for _ in range(2):
+        run.prefill(prompts, [0] * len(lengths), [0] * len(lengths))
+        assert run.sync_status() == native.TSS_OK
+        got.append([t.clone() for t in run.kv])
+    for l in range(ARCH.n_layers):
+        assert torch.equal(got[0][l], got[1][l])
+    for b, n in enumerate(lengths):
+        ref = O.prefill(wo, ARCH, frozenset(), prompts[b])
+        for l in range(ARCH.n_layers):
+            for kind in range(2):
+                g = got[0][l][b, kind, :, :n].float().cpu().numpy()
+                np.testing.assert_allclose(g, ref[l][kind], atol=5e-2, rtol=3e-2, err_msg=f"request {b} layer {l}")
+                assert float(np.abs(g - ref[l][kind]).mean()) < 4e-3
+    run.close()
