@@ -122,8 +122,13 @@ class TssRunner:
                 stream=None) -> None:
         """Append each request's prompt tokens to its KV cache (tss_prefill) under its domain's
         skip configuration; request b's cache then holds ctx_lens[b] + len(prompts[b]) tokens."""
-        toks = torch.tensor([t for pr in prompts for t in pr] or [0], dtype=torch.int32, device=self.device)
-        s = stream if stream is not None else torch.cuda.current_stream().cuda_stream
+        current = torch.cuda.current_stream().cuda_stream
+        s = stream if stream is not None else current
+        toks = torch.tensor([t for pr in prompts for t in pr] or [0], dtype=torch.int32)
+        if s == current:  # from pinned memory in stream order: the copy waits for no earlier work
+            toks = toks.pin_memory().to(self.device, non_blocking=True)
+        else:  # on another stream than the copy's: complete before the call
+            toks = toks.to(self.device)
         self.v.prefill([len(pr) for pr in prompts], list(ctx_lens), list(domains), toks, self.kv_struct, kv_slot=slots,
                        stream=s)
         self._prefill_tokens = toks  # alive until the stream has used it
