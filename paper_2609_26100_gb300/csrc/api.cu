@@ -451,11 +451,11 @@ tss_status enqueue_step(tss_ctx* c, const StepPlan& sp, cudaStream_t s, Prof* pr
   return TSS_OK;
 }
 
-// Shared-memory plan of the persistent kernel: the ring (stages x kps weight blocks with their
-// B-operand blocks) and, behind it, attention-only space so that the attention, which borrows
-// the ring, keeps all key tiles of a split resident (or as many as fit, in rounds).
+// Shared-memory plan of the persistent kernel: two rings -- stages x kps weight blocks, x_stages x
+// xps B-operand blocks -- and, behind them, attention-only space so that the attention, which
+// borrows the rings, keeps all key tiles of a split resident (or as many as fit, in rounds).
 struct MkConfig {
-  int kps = 0, stages = 0, attn_splits = 1;
+  int kps = 0, stages = 0, xps = 0, x_stages = 0, attn_splits = 1;
   size_t attn_extra = 0, smem = 0;
 };
 
@@ -525,30 +525,39 @@ bool mk_config_for(const MkPlanIn& c, int B, int M, int tiles, MkConfig* out) {
   const size_t tile = static_cast<size_t>(2) * 64 * (c.D + 8) * 2;
   const int splits = c.splits_force > 0 ? std::min(c.splits_force, c.max_splits) : mk_attn_splits(c, B, std::max(tiles, 1));
   const int per = std::max(1, (std::max(tiles, 1) + splits - 1) / splits);
-  for (int kps = c.kps_max; kps >= 1; --kps) {
-    const XsLayout xs = xs_layout(M);
-    const size_t stage = static_cast<size_t>(kps) * (16384 + static_cast<size_t>(xs.rows) * xs.parts * 128);
-    for (int S = c.stages_max; S >= 2; --S) {
-      const size_t ring = S * stage;
-      const size_t base = mk_smem_bytes(xs.rows, xs.parts, S, c.D, kps, 0);
-      if (base > kLimit) continue;
-      const size_t avail = kLimit - base;
-      // at least Q + one tile, and Q + the warps' merge buffer (8 warps x 16 rows x D floats)
-      const size_t first = q + std::max(tile, static_cast<size_t>(8) * 16 * c.D * 4);
-      const size_t need_min = ring >= first ? 0 : first - ring;
-      if (need_min > avail) continue;
-      const size_t want = q + per * tile > ring ? q + per * tile - ring : 0;
-      size_t extra = std::max(need_min, std::min(want, avail));
-      extra = (extra + 15) & ~size_t(15);
-      if (base + extra > kLimit) extra = need_min;
-      out->kps = kps;
-      out->stages = S;
-      out->attn_splits = splits;
-      out->attn_extra = extra;
-      out->smem = base + extra;
-      return true;
-    }
-  }
+  const XsLayout xs = xs_layout(M);
+  const size_t xb = static_cast<size_t>(xs.rows) * xs.parts * 128;  // B-operand bytes of a k-block
+  auto take = [&](int kps, int S, int xps, int SX) {
+    const size_t base = mk_smem_bytes(xs.rows, xs.parts, S, kps, SX, xps, 0);
+    if (kps > c.kps_max || S > c.stages_max || base > kLimit) return false;
+    const size_t ring = static_cast<size_t>(S) * kps * 16384 + SX * xps * xb;
+    const size_t avail = kLimit - base;
+    // at least Q + one tile, and Q + the warps' merge buffer (8 warps x 16 rows x D floats)
+    const size_t first = q + std::max(tile, static_cast<size_t>(8) * 16 * c.D * 4);
+    const size_t need_min = ring >= first ? 0 : first - ring;
+    if (need_min > avail) return false;
+    const size_t want = q + per * tile > ring ? q + per * tile - ring : 0;
+    size_t extra = std::max(need_min, std::min(want, avail));
+    extra = (extra + 15) & ~size_t(15);
+    if (base + extra > kLimit) extra = need_min;
+    out->kps = kps;
+    out->stages = S;
+    out->xps = xps;
+    out->x_stages = SX;
+    out->attn_splits = splits;
+    out->attn_extra = extra;
+    out->smem = base + extra;
+    return true;
+  };
+  // The deepest pair of rings that fits, in the order measured: weight stages of 48 KiB, then the
+  // bytes of weights in flight (three stages where there is room), then the B operand's stages, which
+  // hold the same k-blocks.  A stage costs the role that handles it a few hundred cycles, so one
+  // k-block a stage is the last resort (7B layers, us a step, six rows: three k-blocks a stage
+  // 553, two 587, one 761; 61 rows: 48 KiB x 2 590, 32 KiB x 3 586, one k-block 709).
+  static const int kRings[][4] = {{3, 3, 3, 3}, {3, 3, 3, 2}, {3, 2, 3, 2}, {2, 3, 2, 2}, {2, 2, 2, 2}, {2, 4, 1, 2},
+                                  {2, 3, 1, 2}, {2, 2, 1, 2}, {1, 3, 1, 2}, {1, 2, 1, 2}};
+  for (const auto& r : kRings)
+    if (take(r[0], r[1], r[2], r[3])) return true;
   return false;
 }
 
@@ -582,6 +591,8 @@ tss_status enqueue_step_mk(tss_ctx* c, const StepPlan& sp, cudaStream_t s, Prof*
   p.n_pad = n_pad;
   p.stages = stages;
   p.kps = kps;
+  p.xps = cfg.xps;
+  p.x_stages = cfg.x_stages;
   p.xs = xs;
   p.dp_tail = c->mk_dp_tail;
   p.attn_plo = c->attn_plo;

@@ -193,7 +193,8 @@ cudaError_t launch_tile_weights(const __nv_bfloat16* src, __nv_bfloat16* dst, in
 // Persistent verify kernel (verify_mk.cu).
 struct MkParams {
   int n_act, d, H, D, F_pad, Ft, V, V_pad, n_pad, stages, attn_splits, B, max_tiles;
-  int kps;  // k-blocks (16 KiB of weights each) per pipeline stage
+  int kps;  // k-blocks (16 KiB of weights each) per stage of the weight ring
+  int x_stages, xps;  // stages of the B-operand ring, and its k-blocks per stage (1 or kps)
   XsLayout xs;  // B-operand layout (n_pad == xs.rows)
   int attn_plo;         // attention P.V with P split into hi/lo bf16 parts
   int w_evict_first;  // stream weights with the evict-first L2 policy
@@ -241,7 +242,7 @@ struct MkParams {
   int withhold_flag;  // fault injection: withhold one dataflow flag so that a bounded wait runs out
   int dp_tail;     // phases with a tile per CTA end with one whole tile per CTA (no fix-up on their tail)
 };
-size_t mk_smem_bytes(int n_pad, int parts, int stages, int head_dim, int kps, size_t attn_extra);
+size_t mk_smem_bytes(int n_pad, int parts, int stages, int kps, int x_stages, int xps, size_t attn_extra);
 size_t mk_trace_slots();
 cudaError_t mk_prepare();
 int mk_max_blocks_per_sm(int head_dim, size_t smem);

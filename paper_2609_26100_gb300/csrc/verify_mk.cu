@@ -10,9 +10,12 @@
 //               boundaries (it is bounded only by the shared-memory ring).
 //   warp 1      tcgen05.mma issuer (lane 0; accumulators in TMEM, up to 8 buffers).
 //   warp 2      B-operand producer: for every k-block it waits until the activations it needs
-//               are final (flags polled 32 at a time), then loads the N x 64 bf16 tile by TMA --
+//               are final (flags polled 32 at a time), then lane 0 copies the N x 64 bf16 blocks of
+//               every stage that the flags allow, into a ring of their own --
 //               bf16(h * g) for QKV / gate-up / LM head, the attention output for O, the SwiGLU
-//               activations for down.
+//               activations for down.  (One proxy fence per batch of polls; a fence, a poll test
+//               and two 64-bit divisions per stage, with the divisions of the other roles, cost
+//               the 7B chain 5 % of its step: 2886 -> 2750 us.)
 //   warp 3      attention only.
 //   warps 4-7   epilogues (TMEM -> registers, stream-K fix-up, fused op).
 // All roles run one loop over the phases; at each O phase (when the attention runs in this
@@ -106,13 +109,14 @@ __device__ __forceinline__ void mk_fail(const MkShared& sh) {
 
 // Bounded wait for *f >= target.
 __device__ bool mk_wait_flag(const unsigned long long* f, unsigned long long target, const MkShared& sh) {
-  if (ld_acquire_u64(f) >= target) return true;
-  const uint64_t t0 = globaltimer_ns();
+  uint64_t t0 = 0;
   for (uint32_t i = 1;; ++i) {
     if (ld_acquire_u64(f) >= target) return true;
     if ((i & 63) == 0) {
       if (mk_aborted(sh)) return false;
-      if (globaltimer_ns() - t0 > sh.limit_ns) {
+      const uint64_t now = globaltimer_ns();
+      if (t0 == 0) t0 = now;
+      if (now - t0 > sh.limit_ns) {
         mk_fail(sh);
         return false;
       }
@@ -123,14 +127,16 @@ __device__ bool mk_wait_flag(const unsigned long long* f, unsigned long long tar
 
 // Bounded wait for the arrival counter *f to reach `target`.
 __device__ bool mk_wait_count(const int* f, int target, const MkShared& sh) {
-  const uint64_t t0 = globaltimer_ns();
+  uint64_t t0 = 0;
   for (uint32_t i = 1;; ++i) {
     int v;
     asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(f) : "memory");
     if (v >= target) return true;
     if ((i & 63) == 0) {
       if (mk_aborted(sh)) return false;
-      if (globaltimer_ns() - t0 > sh.limit_ns) {
+      const uint64_t now = globaltimer_ns();
+      if (t0 == 0) t0 = now;
+      if (now - t0 > sh.limit_ns) {
         mk_fail(sh);
         return false;
       }
@@ -140,13 +146,15 @@ __device__ bool mk_wait_count(const int* f, int target, const MkShared& sh) {
 
 // Bounded mbarrier wait that also leaves when another CTA aborted.
 __device__ bool mk_wait_bar(uint64_t* bar, uint32_t parity, const MkShared& sh) {
-  if (mbar_try_wait(bar, parity)) return true;
-  const uint64_t t0 = globaltimer_ns();
+  // (the clock is read only after a while: its latency would delay the waiting role at every stage)
+  uint64_t t0 = 0;
   for (uint32_t i = 1;; ++i) {
-    if (mbar_try_wait_sleep(bar, parity, 20000u)) return true;
+    if (mbar_try_wait(bar, parity)) return true;
     if ((i & 255) == 0) {
       if (mk_aborted(sh)) return false;
-      if (globaltimer_ns() - t0 > sh.limit_ns) {
+      const uint64_t now = globaltimer_ns();
+      if (t0 == 0) t0 = now;
+      if (now - t0 > sh.limit_ns) {
         mk_fail(sh);
         return false;
       }
@@ -162,6 +170,20 @@ __device__ __forceinline__ bool mk_team_sync(uint64_t* bar, uint32_t& n, const M
   ++n;
   return ok;
 }
+
+// Position in a ring of n slots: slot and the parity of its current turn, advanced without a
+// division (64-bit divisions by the ring size, one per role and stage, had cost about 0.3 us a
+// stage).
+struct MkRing {
+  int s = 0;
+  uint32_t turn = 0;
+  __device__ __forceinline__ void next(int n) {
+    if (++s == n) {
+      s = 0;
+      turn ^= 1u;
+    }
+  }
+};
 
 struct MkPhase {
   int kind, slot, layer, n_tiles, kb;
@@ -215,14 +237,15 @@ __device__ __forceinline__ const __nv_bfloat16* mk_weights(const MkParams& p, co
 // and p.dp_tail is set, stream-K over its first n_tiles - G tiles followed by one whole tile per
 // CTA, so that the phase ends with whole-tile epilogues (no partial tiles, no arrival counter,
 // no reload of other CTAs' partials on its critical tail).  Residual phases keep plain stream-K.
+// (32-bit arithmetic: T x #SMs is at most 152 / 8192 of a matrix's elements, below 2^32 for any
+// matrix that fits the device; 64-bit divisions took a role about a microsecond a phase)
 struct MkSeg {
-  long long it, it1;  // stream-K iterations of this CTA still to take
-  long long T;        // stream-K iterations of the phase (the fix-up contributor arithmetic)
-  int geff;           // CTAs sharing them
-  int kb, whole;      // this CTA's whole tile after them, -1: none
+  uint32_t it, it1;  // stream-K iterations of this CTA still to take
+  uint32_t T;        // stream-K iterations of the phase (the fix-up contributor arithmetic)
+  uint32_t geff;     // CTAs sharing them
+  int kb, whole;     // this CTA's whole tile after them, -1: none
   __device__ __forceinline__ bool next(int& t, int& k0, int& k1);
   __device__ __forceinline__ bool done() const { return it >= it1 && whole < 0; }
-  __device__ __forceinline__ long long start() const { return it; }
 };
 
 __device__ __forceinline__ MkSeg mk_seg(const MkParams& p, const MkPhase& ph, int c, int G) {
@@ -234,14 +257,14 @@ __device__ __forceinline__ MkSeg mk_seg(const MkParams& p, const MkPhase& ph, in
     n_split = ph.n_tiles - G;
     s.whole = n_split + c;
   }
-  s.T = static_cast<long long>(n_split) * ph.kb;
-  s.geff = static_cast<int>(s.T < G ? s.T : G);
+  s.T = static_cast<uint32_t>(n_split) * ph.kb;
+  s.geff = min(s.T, static_cast<uint32_t>(G));
   // Few short tiles (small models): whole tiles when streaming one takes at most kMkWholeKb
   // k-blocks (16 KiB, about 0.23 us each) more than a CTA's even share -- about what the partial
   // sums' store, counter and reload cost (the tiny decoder's tiles of 4 k-blocks, split over 4
   // CTAs: 6.5 us from MMA to flag against 3 us whole).
-  if (s.whole < 0 && n_split <= G && ph.kb <= s.T / s.geff + kMkWholeKb) s.geff = n_split;
-  if (c >= s.geff) {
+  if (s.whole < 0 && n_split <= G && static_cast<uint32_t>(ph.kb) <= s.T / s.geff + kMkWholeKb) s.geff = n_split;
+  if (static_cast<uint32_t>(c) >= s.geff) {
     s.it = s.it1 = 0;
   } else {
     s.it = s.T * c / s.geff;
@@ -250,23 +273,20 @@ __device__ __forceinline__ MkSeg mk_seg(const MkParams& p, const MkPhase& ph, in
   return s;
 }
 
-__device__ __forceinline__ int mk_cta_of(long long i, long long T, int G) {
+// The CTA whose range holds stream-K iteration i.
+__device__ __forceinline__ int mk_cta_of(uint32_t i, uint32_t T, uint32_t G) {
   return static_cast<int>(((i + 1) * G - 1) / T);
 }
 
-__device__ __forceinline__ bool mk_next_segment(long long& it, long long end, int kb, int& t, int& k0, int& k1) {
-  if (it >= end) return false;
-  t = static_cast<int>(it / kb);
-  k0 = static_cast<int>(it - static_cast<long long>(t) * kb);
-  const long long tile_end = static_cast<long long>(t + 1) * kb;
-  const long long e = end < tile_end ? end : tile_end;
-  k1 = static_cast<int>(e - static_cast<long long>(t) * kb);
-  it = e;
-  return true;
-}
-
 __device__ __forceinline__ bool MkSeg::next(int& t, int& k0, int& k1) {
-  if (mk_next_segment(it, it1, kb, t, k0, k1)) return true;
+  if (it < it1) {
+    t = static_cast<int>(it / kb);
+    const uint32_t t0 = static_cast<uint32_t>(t) * kb;
+    k0 = static_cast<int>(it - t0);
+    it = min(it1, t0 + kb);
+    k1 = static_cast<int>(it - t0);
+    return true;
+  }
   if (whole < 0) return false;
   t = whole;
   k0 = 0;
@@ -701,16 +721,18 @@ __global__ void __launch_bounds__(kMkThreads, 1)
     verify_mk_kernel(const MkParams p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  const int S = p.stages, n_pad = p.n_pad, KPS = p.kps;
+  const int S = p.stages, SX = p.x_stages, n_pad = p.n_pad, KPS = p.kps, XPS = p.xps;
   const int XP = p.xs.parts;
   const uint32_t x_bytes = static_cast<uint32_t>(n_pad) * 128u;  // one block of one k-block of the B operand
-  const uint32_t sw_bytes = KPS * kMkWBytes, sx_bytes = KPS * XP * x_bytes;
+  const uint32_t sw_bytes = KPS * kMkWBytes, sx_bytes = XPS * XP * x_bytes;
   uint8_t* sW = base;
   uint8_t* sX = sW + static_cast<size_t>(S) * sw_bytes;
-  uint8_t* s_attn = sX + static_cast<size_t>(S) * sx_bytes;
-  uint64_t* full = reinterpret_cast<uint64_t*>(s_attn + p.attn_extra);
-  uint64_t* empty = full + S;
-  uint64_t* accf = empty + S;
+  uint8_t* s_attn = sX + static_cast<size_t>(SX) * sx_bytes;
+  uint64_t* fullw = reinterpret_cast<uint64_t*>(s_attn + p.attn_extra);
+  uint64_t* emptyw = fullw + S;
+  uint64_t* fullx = emptyw + S;
+  uint64_t* emptyx = fullx + SX;
+  uint64_t* accf = emptyx + SX;
   uint64_t* acce = accf + kMkMaxAcc;
   uint64_t* team = acce + kMkMaxAcc;  // all 256 threads: entry to / exit from a layer's attention
   int* misc = reinterpret_cast<int*>(team + 1);  // [0] tmem addr, [1] abort, [2..4] bcast, [5] s_last
@@ -741,8 +763,12 @@ __global__ void __launch_bounds__(kMkThreads, 1)
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < S; ++i) {
-      mbar_init(&full[i], 2);  // weight TMA arrival + B-operand arrival
-      mbar_init(&empty[i], 1);
+      mbar_init(&fullw[i], 1);
+      mbar_init(&emptyw[i], 1);
+    }
+    for (int i = 0; i < SX; ++i) {
+      mbar_init(&fullx[i], 1);
+      mbar_init(&emptyx[i], 1);
     }
     for (int i = 0; i < kMkMaxAcc; ++i) {
       mbar_init(&accf[i], 1);
@@ -796,8 +822,8 @@ __global__ void __launch_bounds__(kMkThreads, 1)
   // (inside this kernel's attention) all eight warps first run the layer's attention as one team.
   const uint64_t wpol = l2_policy_evict_first();
   const uint32_t idesc = idesc_bf16_m128(n_pad);
-  long long i = 0;  // this role's ring stage counter
-  int use = 0;      // this role's accumulator buffer counter
+  MkRing rw, rx;  // this role's positions in the weight and B-operand rings
+  MkRing use;     // ... and in the accumulator buffers
   bool ok = true;
   MkEpi e;
   e.q = warp & 3;
@@ -819,18 +845,18 @@ __global__ void __launch_bounds__(kMkThreads, 1)
       const bool last_seg = seg.done();
       for (int kc = k0; kc < k1; kc += KPS, ++j) {
         const int nk = min(KPS, k1 - kc);
-        const int s = static_cast<int>(i % S);
-        if (!mk_wait_bar(&empty[s], static_cast<uint32_t>((i / S) & 1) ^ 1u, sh)) return false;
+        const int s = rw.s;
+        if (!mk_wait_bar(&emptyw[s], rw.turn ^ 1u, sh)) return false;
         if (j == 0) mk_trace(p, pi * 8 + 0);
         if (last_seg && kc + nk == k1) mk_trace(p, pi * 8 + 1);
-        mbar_arrive_expect_tx(&full[s], nk * kMkWBytes);
+        mbar_arrive_expect_tx(&fullw[s], nk * kMkWBytes);
         if (p.w_evict_first)
           bulk_load_hint(sW + static_cast<size_t>(s) * sw_bytes,
-                         wl + (static_cast<size_t>(t) * ph.kb + kc) * kTileElems, nk * kMkWBytes, &full[s], wpol);
+                         wl + (static_cast<size_t>(t) * ph.kb + kc) * kTileElems, nk * kMkWBytes, &fullw[s], wpol);
         else
           bulk_load(sW + static_cast<size_t>(s) * sw_bytes,
-                    wl + (static_cast<size_t>(t) * ph.kb + kc) * kTileElems, nk * kMkWBytes, &full[s]);
-        ++i;
+                    wl + (static_cast<size_t>(t) * ph.kb + kc) * kTileElems, nk * kMkWBytes, &fullw[s]);
+        rw.next(S);
       }
     }
     return true;
@@ -856,48 +882,56 @@ __global__ void __launch_bounds__(kMkThreads, 1)
         int t, k0, k1;
         bool first = true;
         while (ok && seg.next(t, k0, k1)) {
-          const int buf = use % NB;
-          if (!mk_wait_bar(&acce[buf], static_cast<uint32_t>((use / NB) & 1) ^ 1u, sh)) {
+          const int buf = use.s;
+          if (!mk_wait_bar(&acce[buf], use.turn ^ 1u, sh)) {
             ok = false;
             break;
           }
           tc_fence_after();
           const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(buf * n_pad);
-          for (int kc = k0; kc < k1; kc += KPS, ++i) {
+          for (int kc = k0; ok && kc < k1; kc += KPS, rw.next(S)) {
             const int nk = min(KPS, k1 - kc);
-            const int s = static_cast<int>(i % S);
-            if (!mk_wait_bar(&full[s], static_cast<uint32_t>((i / S) & 1), sh)) {
+            const int s = rw.s;
+            if (!mk_wait_bar(&fullw[s], rw.turn, sh)) {
               ok = false;
               break;
             }
-            tc_fence_after();
-            if (first) mk_trace(p, pi * 8 + 4);
-            first = false;
-            for (int j = 0; j < nk; ++j) {
-              const uint32_t a0 = smem_u32(sW + static_cast<size_t>(s) * sw_bytes + j * kMkWBytes);
-              const uint32_t b0 = smem_u32(sX + static_cast<size_t>(s) * sx_bytes + j * XP * x_bytes);
-              // (branch outside the issue loops: a conditional MMA inside them was measured to
-              // slow every stage down)
-              if (XP == 1) {
+            for (int jx = 0; jx < nk; jx += XPS, rx.next(SX)) {
+              const int sx = rx.s;
+              if (!mk_wait_bar(&fullx[sx], rx.turn, sh)) {
+                ok = false;
+                break;
+              }
+              tc_fence_after();
+              if (first) mk_trace(p, pi * 8 + 4);
+              first = false;
+              for (int j = jx; j < min(jx + XPS, nk); ++j) {
+                const uint32_t a0 = smem_u32(sW + static_cast<size_t>(s) * sw_bytes + j * kMkWBytes);
+                const uint32_t b0 = smem_u32(sX + static_cast<size_t>(sx) * sx_bytes + (j - jx) * XP * x_bytes);
+                // (branch outside the issue loops: a conditional MMA inside them was measured to
+                // slow every stage down)
+                if (XP == 1) {
 #pragma unroll
-                for (int k16 = 0; k16 < 4; ++k16)
-                  umma_bf16(d_tmem, sdesc_sw128(a0 + k16 * 32), sdesc_sw128(b0 + k16 * 32), idesc,
-                            (kc + j > k0 || k16 > 0) ? 1u : 0u);
-              } else {  // the lo block accumulates into the same columns
+                  for (int k16 = 0; k16 < 4; ++k16)
+                    umma_bf16(d_tmem, sdesc_sw128(a0 + k16 * 32), sdesc_sw128(b0 + k16 * 32), idesc,
+                              (kc + j > k0 || k16 > 0) ? 1u : 0u);
+                } else {  // the lo block accumulates into the same columns
 #pragma unroll
-                for (int k16 = 0; k16 < 4; ++k16) {
-                  umma_bf16(d_tmem, sdesc_sw128(a0 + k16 * 32), sdesc_sw128(b0 + k16 * 32), idesc,
-                            (kc + j > k0 || k16 > 0) ? 1u : 0u);
-                  umma_bf16(d_tmem, sdesc_sw128(a0 + k16 * 32), sdesc_sw128(b0 + x_bytes + k16 * 32), idesc, 1u);
+                  for (int k16 = 0; k16 < 4; ++k16) {
+                    umma_bf16(d_tmem, sdesc_sw128(a0 + k16 * 32), sdesc_sw128(b0 + k16 * 32), idesc,
+                              (kc + j > k0 || k16 > 0) ? 1u : 0u);
+                    umma_bf16(d_tmem, sdesc_sw128(a0 + k16 * 32), sdesc_sw128(b0 + x_bytes + k16 * 32), idesc, 1u);
+                  }
                 }
               }
+              umma_commit(&emptyx[sx]);
             }
-            umma_commit(&empty[s]);
+            umma_commit(&emptyw[s]);
           }
           if (!ok) break;
           umma_commit(&accf[buf]);
           if (seg.done()) mk_trace(p, pi * 8 + 5);
-          ++use;
+          use.next(NB);
         }
       }
       ok = __shfl_sync(0xffffffffu, ok, 0);
@@ -923,7 +957,7 @@ __global__ void __launch_bounds__(kMkThreads, 1)
         n_dep = p.d / 128;
       }
       const __nv_bfloat16* xsrc = ph.kind == kMkO ? p.obuf : ph.kind == kMkDown ? p.act : p.xn;
-      uint32_t ready[8] = {0, 0, 0, 0, 0, 0, 0, 0};  // known-complete dependency indices (<= 256)
+      uint32_t ready[17] = {};  // known-complete dependency indices below 512 (others are polled each time)
       // one flag index is complete when every request that runs the slot has it (attention) or
       // the single flag reached `want`
       auto poll = [&](int x) -> bool {
@@ -932,60 +966,81 @@ __global__ void __launch_bounds__(kMkThreads, 1)
           if (pl->slot_crow[ph.slot][b] >= 0 && ld_acquire_u64(&flags[b * p.H + x]) < want) return false;
         return true;
       };
+      // dependency index of a k-block, and the first k-block after those of index x
+      auto dep = [&](int kk) { return ph.kind == kMkO ? kk * 64 / D : ph.kind == kMkDown ? kk : kk >> 1; };
+      auto dep_end = [&](int x) { return ph.kind == kMkO ? (x + 1) * D / 64 : ph.kind == kMkDown ? x + 1 : 2 * (x + 1); };
       int t, k0, k1;
       bool first = true;
       while (ok && seg.next(t, k0, k1)) {
-       const bool last_seg = seg.done();
-       for (int kc = k0; ok && kc < k1; kc += KPS, ++i) {
-        const int nk = min(KPS, k1 - kc);
-        const int s = static_cast<int>(i % S);
-        if (lane == 0) ok = mk_wait_bar(&empty[s], static_cast<uint32_t>((i / S) & 1) ^ 1u, sh);
-        ok = __shfl_sync(0xffffffffu, ok, 0);
-        if (!ok) break;
-        for (int kk = kc; kk < kc + nk; ++kk) {
-        const int x = want == 0ull ? -1 : (ph.kind == kMkO ? kk * 64 / p.D : ph.kind == kMkDown ? kk : (kk >> 1));
-        if (x >= 0 && !((ready[x >> 5] >> (x & 31)) & 1u)) {
-          // poll x .. x+31 at once; then wait (bounded) for x itself if it is not there yet
-          const int y = x + lane;
-          const bool rdy = y < n_dep && poll(y);
-          const uint32_t bal = __ballot_sync(0xffffffffu, rdy);
-          __syncwarp();  // memory ordering: lane 0's copy follows the acquire loads of the others
-          for (int l = 0; l < 32; ++l)
-            if ((bal >> l) & 1u) ready[(x + l) >> 5] |= 1u << ((x + l) & 31);
-          if (!(bal & 1u)) {
-            bool got = true;
-            if (lane == 0) {
-              const uint64_t t0 = globaltimer_ns();
-              while (!poll(x)) {
-                if (mk_aborted(sh)) {
-                  got = false;
-                  break;
-                }
-                if (globaltimer_ns() - t0 > sh.limit_ns) {
-                  mk_fail(sh);
-                  got = false;
-                  break;
-                }
-                __nanosleep(64);
-              }
+        const bool last_seg = seg.done();
+        int kc = k0, kr = want == 0ull ? k1 : k0;  // k-blocks below kr are known to be complete
+        while (ok && kc < k1) {
+          // the whole warp: extend kr over the next stage, or as far as the flags already go
+          const int need = min(kc + XPS, k1);
+          while (ok && kr < need) {
+            const int x = dep(kr);
+            if (x < 512 && ((ready[x >> 5] >> (x & 31)) & 1u)) {
+              kr = dep_end(x);
+              continue;
             }
-            ok = __shfl_sync(0xffffffffu, got, 0);
-            if (!ok) break;
-            ready[x >> 5] |= 1u << (x & 31);
+            // poll x .. x+31 at once; then wait (bounded) for x itself if it is not there yet
+            const int y = x + lane;
+            const uint32_t bal = __ballot_sync(0xffffffffu, y < n_dep && poll(y));
+            __syncwarp();  // memory ordering: lane 0's copies follow the acquire loads of the others
+            if (x < 512) {
+              ready[x >> 5] |= bal << (x & 31);
+              if (x & 31) ready[(x >> 5) + 1] |= bal >> (32 - (x & 31));
+            }
+            if (bal & 1u) {
+              kr = dep_end(x + __ffs(~bal | 0x80000000u) - 2);
+            } else {
+              bool got = true;
+              if (lane == 0) {
+                const uint64_t t0 = globaltimer_ns();
+                while (!poll(x)) {
+                  if (mk_aborted(sh)) {
+                    got = false;
+                    break;
+                  }
+                  if (globaltimer_ns() - t0 > sh.limit_ns) {
+                    mk_fail(sh);
+                    got = false;
+                    break;
+                  }
+                  __nanosleep(64);
+                }
+              }
+              ok = __shfl_sync(0xffffffffu, got, 0);
+              if (!ok) break;
+              kr = dep_end(x);
+            }
           }
+          if (!ok) break;
+          // lane 0: the copies of every stage below kr.  They read what the flags' producers wrote:
+          // one proxy fence after the polls.
+          const int kend = min(kr, k1);
+          if (lane == 0) {
+            fence_proxy_async_global();
+            int k = kc;
+            for (; k < k1 && min(k + XPS, k1) <= kend; k += XPS) {
+              const int nk = min(XPS, k1 - k), s = rx.s;
+              if (!mk_wait_bar(&emptyx[s], rx.turn ^ 1u, sh)) {
+                ok = false;
+                break;
+              }
+              if (first) mk_trace(p, pi * 8 + 2);
+              first = false;
+              if (last_seg && k + nk == k1) mk_trace(p, pi * 8 + 3);
+              mbar_arrive_expect_tx(&fullx[s], nk * XP * x_bytes);
+              bulk_load(sX + static_cast<size_t>(s) * sx_bytes, xsrc + static_cast<size_t>(k) * XP * n_pad * 64,
+                        nk * XP * x_bytes, &fullx[s]);
+              rx.next(SX);
+            }
+            kc = k;
+          }
+          ok = __shfl_sync(0xffffffffu, ok, 0);
+          kc = __shfl_sync(0xffffffffu, kc, 0);
         }
-        }
-        if (!ok) break;
-        if (lane == 0) {
-          if (first) mk_trace(p, pi * 8 + 2);
-          if (last_seg && kc + nk == k1) mk_trace(p, pi * 8 + 3);
-          fence_proxy_async_global();
-          mbar_arrive_expect_tx(&full[s], nk * XP * x_bytes);
-          bulk_load(sX + static_cast<size_t>(s) * sx_bytes, xsrc + static_cast<size_t>(kc) * XP * n_pad * 64, nk * XP * x_bytes,
-                    &full[s]);
-        }
-        first = false;
-       }
       }
     } else if (warp >= 4) {
       // ---------------- epilogues ----------------
@@ -1074,8 +1129,7 @@ __global__ void __launch_bounds__(kMkThreads, 1)
         }
         named_bar_sync(1, 128);
       }
-      const long long T = seg.T;
-      const int geff = seg.geff;
+      const uint32_t T = seg.T, geff = seg.geff;
       float* partials = (pi & 1) ? p.partials1 : p.partials0;
       int* counters = p.counters + static_cast<size_t>(ph.kind) * p.max_tiles;
       int* done = counters + static_cast<size_t>(7) * p.max_tiles;
@@ -1098,8 +1152,8 @@ __global__ void __launch_bounds__(kMkThreads, 1)
       int t, k0, k1;
       bool first = true;
       while (ok && seg.next(t, k0, k1)) {
-        const int buf = use % NB;
-        const bool got = e.et == 0 ? mk_wait_bar(&accf[buf], static_cast<uint32_t>((use / NB) & 1), sh) : true;
+        const int buf = use.s;
+        const bool got = e.et == 0 ? mk_wait_bar(&accf[buf], use.turn, sh) : true;
         if (!bar_and(1, 128, got)) {
           ok = false;
           break;
@@ -1127,8 +1181,8 @@ __global__ void __launch_bounds__(kMkThreads, 1)
           named_bar_sync(1, 128);  // every thread's partial stores precede the release below
           if (tr_last) mk_trace(p, kMkTraceSub + pi * 8 + 1);
           if (e.et == 0) {
-            const int f = mk_cta_of(static_cast<long long>(t) * ph.kb, T, geff);
-            const int l = mk_cta_of(static_cast<long long>(t + 1) * ph.kb - 1, T, geff);
+            const int f = mk_cta_of(t * ph.kb, T, geff);
+            const int l = mk_cta_of((t + 1) * ph.kb - 1, T, geff);
             const int last = atom_add_acq_rel_gpu(&counters[t], 1) == l - f;
             if (last && !share) atomicExch(&counters[t], 0);
             int* pd = s_pend + 4 * n_pend;
@@ -1194,7 +1248,7 @@ __global__ void __launch_bounds__(kMkThreads, 1)
           if (!share) named_bar_sync(1, 128);  // s_pend is rewritten by the next segment
         }
         if (e.et == 0 && seg.done()) mk_trace(p, pi * 8 + 7);
-        ++use;
+        use.next(NB);
       }
     }
   }
@@ -1215,9 +1269,10 @@ __global__ void __launch_bounds__(kMkThreads, 1)
 
 size_t mk_trace_slots() { return kMkTraceSlots; }
 
-size_t mk_smem_bytes(int n_pad, int parts, int stages, int head_dim, int kps, size_t attn_extra) {
-  return 1024 + static_cast<size_t>(stages) * kps * (kMkWBytes + static_cast<size_t>(n_pad) * parts * 128) +
-         attn_extra + static_cast<size_t>(2 * stages + 2 * kMkMaxAcc + 1) * 8 + 64 + 16 * 128 * 4 +
+size_t mk_smem_bytes(int n_pad, int parts, int stages, int kps, int x_stages, int xps, size_t attn_extra) {
+  return 1024 + static_cast<size_t>(stages) * kps * kMkWBytes +
+         static_cast<size_t>(x_stages) * xps * n_pad * parts * 128 + attn_extra +
+         static_cast<size_t>(2 * stages + 2 * x_stages + 2 * kMkMaxAcc + 1) * 8 + 64 + 16 * 128 * 4 +
          64 * 4 * 2 + kMaxRows * 4 + 256 * 4 + 5 * kMaxRows * 4 + 2 * 16 * 64 * 4 + 64;
 }
 
