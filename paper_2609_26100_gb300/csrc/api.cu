@@ -94,6 +94,8 @@ struct tss_ctx {
   int* counters = nullptr;
   float* amax_val = nullptr;
   int* amax_idx = nullptr;
+  float* row_stat = nullptr;  // sampling: softmax statistics of the rows
+  int* row_cnt = nullptr;
   float *attn_po = nullptr, *attn_pml = nullptr;
   int* attn_cnt = nullptr;
   int max_splits = kMaxSplits;
@@ -241,6 +243,8 @@ MiscParams misc_params(tss_ctx* c) {
   p.amax_val = c->amax_val;
   p.amax_idx = c->amax_idx;
   p.n_vtiles = c->V_pad / 128;
+  p.row_stat = c->row_stat;
+  p.row_cnt = c->row_cnt;
   p.status = c->d_status;
   return p;
 }
@@ -442,7 +446,7 @@ tss_status enqueue_step(tss_ctx* c, const StepPlan& sp, cudaStream_t s, Prof* pr
   g.w_layer_elems = 0;
   TSS_K(6, TSS_TRY(run_gemm(c, kEpiLmHead, *txn, *txn, g, c->V_pad / 128, kbd, s, pdl)));
   if (sp.mode == TSS_MODE_SAMPLE) {
-    TSS_K(7, TSS_CU(launch_accept_sample(mp, sp.B, s, pdl)));
+    TSS_K(7, TSS_CU(launch_accept_sample(mp, sp.M, s, pdl)));
   } else {
     TSS_K(7, TSS_CU(launch_accept_greedy(mp, sp.B, s, pdl)));
   }
@@ -708,7 +712,7 @@ tss_status enqueue_step_mk(tss_ctx* c, const StepPlan& sp, cudaStream_t s, Prof*
     p.ph_end = 1 << 30;
     TSS_MK(8, TSS_CU(launch_verify_mk(p, c->num_sms, smem, s)));
   }
-  TSS_MK(7, TSS_CU(launch_finish(mp, sp.B, sp.mode == TSS_MODE_SAMPLE, s, false)));
+  TSS_MK(7, TSS_CU(launch_finish(mp, sp.B, sp.M, sp.mode == TSS_MODE_SAMPLE, s, false)));
 #undef TSS_MK
   return TSS_OK;
 }
@@ -827,6 +831,9 @@ tss_status build_workspaces(tss_ctx* c) {
   TSS_CU(cudaMemset(c->counters, 0, (max_tiles + 64) * sizeof(int)));
   TSS_TRY(c->alloc(&c->amax_val, static_cast<size_t>(c->V_pad / 128) * kMaxRows));
   TSS_TRY(c->alloc(&c->amax_idx, static_cast<size_t>(c->V_pad / 128) * kMaxRows));
+  TSS_TRY(c->alloc(&c->row_stat, 2 * kMaxRows));
+  TSS_TRY(c->alloc(&c->row_cnt, kMaxBatch));
+  TSS_CU(cudaMemset(c->row_cnt, 0, kMaxBatch * sizeof(int)));
   // partials of the split attention: 64 rows per (request, head, split), 128 for wide blocks
   const size_t ph = static_cast<size_t>(c->a.max_batch) * c->H * c->max_splits *
                     (c->a.max_nodes > kNarrowNodes ? kMaxNodes : kNarrowNodes);
@@ -919,9 +926,10 @@ void destroy_ctx(tss_ctx* c) {
 }
 
 // Host-side per-step checks and the descriptor contents.  Nothing is enqueued here.
-// rng_ids (optional): the Philox request index of each request (default: its index in the batch).
+// orig_ids, orig_rows (optional): each request's index and first row in the caller's arrays (default: as
+// in the batch itself).
 tss_status prepare_step(const tss_ctx* c, const tss_verify_batch* bt, const tss_kv_cache* kv,
-                        const tss_verify_result* res, StepDesc* sd, StepPlan* sp, const int* rng_ids = nullptr) {
+                        const tss_verify_result* res, StepDesc* sd, StepPlan* sp, const int* orig_ids = nullptr, const int* orig_rows = nullptr) {
   if (!bt || !kv || !res) return fail(TSS_ERR_INVALID_ARG, "batch, kv or result is NULL");
   const int B = bt->n_req;
   if (B < 1 || B > c->a.max_batch) return fail(TSS_ERR_INVALID_ARG, "n_req must be in [1, max_batch]");
@@ -953,8 +961,8 @@ tss_status prepare_step(const tss_ctx* c, const tss_verify_batch* bt, const tss_
     sd->req_nodes[b] = n;
     sd->req_rowoff[b] = M;
     sd->req_slot[b] = slot;
-    sd->req_domain[b] = dom;
-    sd->req_rng[b] = rng_ids ? rng_ids[b] : b;
+    sd->req_orow[b] = orig_rows ? orig_rows[b] : M;
+    sd->req_rng[b] = orig_ids ? orig_ids[b] : b;
     sd->req_phi[b] = mask;
     unsigned long long anc[kMaxNodes], anc_hi[kMaxNodes];  // ancestor-or-self bits of rows 0..63, 64..127
     int depth[kMaxNodes];
@@ -1319,13 +1327,13 @@ tss_status tss_active_layer_count(const tss_ctx* c, const tss_verify_batch* bt, 
 namespace {
 
 tss_status verify_impl(tss_ctx* c, const tss_verify_batch* bt, const tss_kv_cache* kv, const tss_verify_result* res,
-                       cudaStream_t s, Prof* prof, const int* rng_ids = nullptr) {
+                       cudaStream_t s, Prof* prof, const int* orig_ids = nullptr, const int* orig_rows = nullptr) {
   if (!c) return fail(TSS_ERR_INVALID_ARG, "ctx is NULL");
   const int ri = c->ring_i;
   if (c->ring_used[ri]) TSS_CU(cudaEventSynchronize(c->ring_ev[ri]));
   StepDesc* sd = c->h_ring[ri];
   StepPlan sp;
-  TSS_TRY(prepare_step(c, bt, kv, res, sd, &sp, rng_ids));
+  TSS_TRY(prepare_step(c, bt, kv, res, sd, &sp, orig_ids, orig_rows));
   const int M = sp.M, B = sp.B;
   const bool host_io = bt->io_host != 0;
   if (host_io) {
@@ -1469,15 +1477,14 @@ tss_status tss_verify_grouped(tss_ctx* c, const tss_verify_batch* bt, const tss_
   std::stable_sort(keys.begin(), keys.end(), [&](unsigned long long x, unsigned long long y) {
     return __builtin_popcountll(all_layers & ~x) < __builtin_popcountll(all_layers & ~y);
   });
-  const size_t V = static_cast<size_t>(c->V);
   for (size_t g = 0; g < keys.size(); ++g) {
     std::vector<int32_t> nn, cl, dom, slot, par, pos;
-    std::vector<int> orig;
-    int rows = 0;
+    std::vector<int> orig, orow;
     for (int b = 0; b < B; ++b) {
       if (masks[b] != keys[g]) continue;
       const int n = bt->n_nodes[b];
       orig.push_back(b);
+      orow.push_back(off[b]);
       nn.push_back(n);
       cl.push_back(bt->ctx_len[b]);
       dom.push_back(bt->domain_id[b]);
@@ -1486,18 +1493,8 @@ tss_status tss_verify_grouped(tss_ctx* c, const tss_verify_batch* bt, const tss_
         par.push_back(bt->parent_idx[off[b] + i]);
         if (bt->positions) pos.push_back(bt->positions[off[b] + i]);
       }
-      // inputs of the group, contiguous in the context's staging buffers
-      TSS_CU(cudaMemcpyAsync(c->io_tokens + rows, bt->tokens + off[b], sizeof(int32_t) * n, cudaMemcpyDeviceToDevice, s));
-      if (bt->mode == TSS_MODE_SAMPLE) {
-        TSS_CU(cudaMemcpyAsync(c->io_probs + rows * V, bt->draft_probs + off[b] * V, sizeof(float) * n * V,
-                               cudaMemcpyDeviceToDevice, s));
-        if (bt->uniforms)
-          TSS_CU(cudaMemcpyAsync(c->io_unif + (orig.size() - 1) * bt->uniform_stride,
-                                 bt->uniforms + static_cast<size_t>(b) * bt->uniform_stride,
-                                 sizeof(float) * bt->uniform_stride, cudaMemcpyDeviceToDevice, s));
-      }
-      rows += n;
     }
+    // the group's step reads and writes the caller's arrays at each request's own place
     tss_verify_batch sub = *bt;
     sub.n_req = static_cast<int>(nn.size());
     sub.n_nodes = nn.data();
@@ -1506,32 +1503,7 @@ tss_status tss_verify_grouped(tss_ctx* c, const tss_verify_batch* bt, const tss_
     sub.kv_slot = slot.data();
     sub.parent_idx = par.data();
     sub.positions = bt->positions ? pos.data() : nullptr;
-    sub.tokens = c->io_tokens;
-    sub.draft_probs = bt->mode == TSS_MODE_SAMPLE ? c->io_probs : nullptr;
-    sub.uniforms = bt->mode == TSS_MODE_SAMPLE && bt->uniforms ? c->io_unif : nullptr;
-    tss_verify_result sr{};
-    sr.accept_len = c->io_res;
-    sr.bonus = c->io_res + kMaxBatch;
-    sr.new_ctx_len = c->io_res + 2 * kMaxBatch;
-    sr.path = c->io_res + 3 * kMaxBatch;
-    sr.path_stride = res->path_stride;
-    sr.logits = res->logits ? c->logits_ws : nullptr;
-    TSS_TRY(verify_impl(c, &sub, kv, &sr, s, nullptr, orig.data()));
-    // results back to the caller's request positions
-    int r = 0;
-    for (size_t j = 0; j < orig.size(); ++j) {
-      const int b = orig[j], n = nn[j];
-      TSS_CU(cudaMemcpyAsync(res->accept_len + b, sr.accept_len + j, sizeof(int32_t), cudaMemcpyDeviceToDevice, s));
-      TSS_CU(cudaMemcpyAsync(res->bonus + b, sr.bonus + j, sizeof(int32_t), cudaMemcpyDeviceToDevice, s));
-      TSS_CU(cudaMemcpyAsync(res->new_ctx_len + b, sr.new_ctx_len + j, sizeof(int32_t), cudaMemcpyDeviceToDevice, s));
-      TSS_CU(cudaMemcpyAsync(res->path + static_cast<size_t>(b) * res->path_stride,
-                             sr.path + j * static_cast<size_t>(res->path_stride), sizeof(int32_t) * res->path_stride,
-                             cudaMemcpyDeviceToDevice, s));
-      if (res->logits)
-        TSS_CU(cudaMemcpyAsync(res->logits + off[b] * V, c->logits_ws + r * V, sizeof(float) * n * V,
-                               cudaMemcpyDeviceToDevice, s));
-      r += n;
-    }
+    TSS_TRY(verify_impl(c, &sub, kv, res, s, nullptr, orig.data(), orow.data()));
     if (group_events && group_events[g]) TSS_CU(cudaEventRecord(static_cast<cudaEvent_t>(group_events[g]), s));
   }
   if (n_groups) *n_groups = static_cast<int>(keys.size());

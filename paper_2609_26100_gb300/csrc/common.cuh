@@ -42,12 +42,14 @@ struct StepDesc {
   int req_nodes[kMaxBatch];
   int req_rowoff[kMaxBatch];
   int req_slot[kMaxBatch];
-  int req_domain[kMaxBatch];
+  int req_orow[kMaxBatch];  // first row of the request in the caller's arrays (tokens, draft_probs, logits)
   // S(x) of every request: the domain map's entry for its domain when the step was enqueued (the
   // lookup S(x) = Phi(d(x)) runs on the host, so a later change of the map affects later steps
   // only), 0 (dense) for a domain that is not configured.
   unsigned long long req_phi[kMaxBatch];
-  int req_rng[kMaxBatch];  // request index of the Philox counter (the caller's index when a batch is split)
+  // the request's index in the caller's batch: Philox counter, uniforms and result arrays (differs from
+  // its index here when a batch is split)
+  int req_rng[kMaxBatch];
   int row_req[kMaxRows];
   int row_pos[kMaxRows];
   int row_parent[kMaxRows];  // request-local parent, -1 for the root
@@ -63,6 +65,12 @@ struct StepDesc {
   float* logits;
   __nv_bfloat16* kv_layer[kMaxLayers];
 };
+
+// Row m of the step in the caller's arrays.
+__device__ __forceinline__ int caller_row(const StepDesc* st, int m) {
+  const int b = st->row_req[m];
+  return st->req_orow[b] + (m - st->req_rowoff[b]);
+}
 
 // Written on the device by the skip controller from the descriptor and the domain table Phi.
 struct PlanDev {

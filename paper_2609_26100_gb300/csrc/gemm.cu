@@ -161,7 +161,7 @@ __device__ __forceinline__ void epilogue_chunk(const GemmParams& p, const EpiCtx
       const int j = j0 + jj;
       float val = valid ? v[jj] : -INFINITY;
       if (valid && j < e.M) {
-        if (logits) logits[static_cast<size_t>(batch_row(e, j)) * p.vocab + o] = v[jj];
+        if (logits) logits[static_cast<size_t>(caller_row(p.step, batch_row(e, j))) * p.vocab + o] = v[jj];
         if (v[jj] != v[jj]) report(p.status, kStatusCheck);
       }
       int idx = o;

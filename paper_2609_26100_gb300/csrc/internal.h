@@ -161,13 +161,15 @@ struct MiscParams {
   const float* amax_val;        // [n_vtiles][kMaxRows]
   const int* amax_idx;
   int n_vtiles;
+  float* row_stat;              // [kMaxRows][2] sampling: (max, sum of exponentials) of each row
+  int* row_cnt;                 // [kMaxBatch] rows of a request done, self-resetting
   int* status;
   XsLayout xs;  // xs.rows == 0: xn row-major; else the persistent kernel's split tiled operand
 };
 
 cudaError_t misc_prepare();
 cudaError_t launch_prologue(const MiscParams& p, float* ssp, int* zero_ints, int n_zero, int M, cudaStream_t s, bool pdl);
-cudaError_t launch_finish(const MiscParams& p, int B, bool sample, cudaStream_t s, bool pdl);
+cudaError_t launch_finish(const MiscParams& p, int B, int M, bool sample, cudaStream_t s, bool pdl);
 // Dynamic shared memory of the sampling acceptance's staged inverse CDF: the vocabulary's weights
 // with one skew word per 32 (0 when that exceeds kCdfStageMaxBytes: the unstaged pass runs).
 constexpr size_t kCdfStageMaxBytes = 200 * 1024;
@@ -180,7 +182,7 @@ cudaError_t launch_embed(const MiscParams& p, int M, cudaStream_t s, bool pdl);
 // which: 0 = attention norm of the slot's layer, 1 = MLP norm, 2 = final norm (slot ignored)
 cudaError_t launch_rmsnorm(const MiscParams& p, int slot, int which, int M, cudaStream_t s, bool pdl);
 cudaError_t launch_accept_greedy(const MiscParams& p, int B, cudaStream_t s, bool pdl);
-cudaError_t launch_accept_sample(const MiscParams& p, int B, cudaStream_t s, bool pdl);
+cudaError_t launch_accept_sample(const MiscParams& p, int M, cudaStream_t s, bool pdl);
 cudaError_t launch_compact(const MiscParams& p, int B, int n_act, cudaStream_t s, bool pdl);
 cudaError_t launch_bf16_to_f32(const __nv_bfloat16* src, float* dst, size_t n, cudaStream_t s);
 // The acceptance's Philox4x32-10 stream for one (seed, offset): words [n_req][n_slots][4] and/or

@@ -71,7 +71,7 @@ __global__ void embed_kernel(const MiscParams p) {
   const StepDesc* st = p.step;
   const int m = blockIdx.x;
   if (m >= st->M) return;
-  int tok = st->tokens[m];
+  int tok = st->tokens[caller_row(st, m)];
   if (tok < 0 || tok >= p.vocab) {
     if (threadIdx.x == 0) report(p.status, kStatusCheck);
     tok = 0;
@@ -128,8 +128,8 @@ __global__ void rmsnorm_kernel(const MiscParams p, int slot, int which) {
 __device__ void write_result(const MiscParams& p, int b, int a, int bonus, const int* path) {
   const StepDesc* st = p.step;
   PlanDev* pl = p.plan;
-  const int stride = st->path_stride;
-  int* out = st->path + static_cast<size_t>(b) * stride;
+  const int stride = st->path_stride, ob = st->req_rng[b];
+  int* out = st->path + static_cast<size_t>(ob) * stride;
   for (int i = threadIdx.x; i < stride; i += blockDim.x) out[i] = i <= a ? path[i] : -1;
   for (int i = threadIdx.x; i <= a; i += blockDim.x) pl->res_path[b][i] = path[i];
   if (threadIdx.x == 0) {
@@ -137,9 +137,9 @@ __device__ void write_result(const MiscParams& p, int b, int a, int bonus, const
     int* accept_len = st->accept_len;
     int* bonus_out = st->bonus;
     int* new_ctx = st->new_ctx;
-    accept_len[b] = a;
-    bonus_out[b] = bonus;
-    new_ctx[b] = ctx + 1 + a;
+    accept_len[ob] = a;
+    bonus_out[ob] = bonus;
+    new_ctx[ob] = ctx + 1 + a;
     pl->res_accept[b] = a;
   }
 }
@@ -154,7 +154,7 @@ __device__ int accept_greedy_body(const MiscParams& p, int b, int* path) {
   const int N = st->req_nodes[b], off = st->req_rowoff[b];
   for (int i = threadIdx.x; i < N; i += blockDim.x) {
     s_par[i] = st->row_parent[off + i];
-    s_tok[i] = st->tokens[off + i];
+    s_tok[i] = st->tokens[st->req_orow[b] + i];
   }
   // Argmax of every row over the vocabulary tiles' partials (laid out [tile][row]): thread
   // (g, r), g < G = blockDim / RP, scans row r's tiles g, g + G, ..., so that a warp's loads
@@ -258,7 +258,7 @@ __device__ __forceinline__ uint4 philox_slot(uint32_t seed_lo, uint32_t seed_hi,
 __device__ __forceinline__ float uniform24(uint32_t x) { return static_cast<float>(x >> 8) * (1.f / 16777216.f); }
 
 __device__ __forceinline__ double draw_uniform(const StepDesc* st, int b, int slot) {
-  if (st->uniforms) return static_cast<double>(st->uniforms[static_cast<size_t>(b) * st->uniform_stride + slot]);
+  if (st->uniforms) return static_cast<double>(st->uniforms[static_cast<size_t>(st->req_rng[b]) * st->uniform_stride + slot]);
   return static_cast<double>(
       uniform24(philox_slot(st->seed_lo, st->seed_hi, st->off_lo, st->off_hi, st->req_rng[b], slot).x));
 }
@@ -419,68 +419,98 @@ __device__ int inverse_cdf_staged(int V, float u, WFn w, float* scan) {
   return inverse_cdf_block(V, u, [&](int v) { return cdf_stage[v + (v >> 5)]; }, scan);
 }
 
+// Softmax statistics of row m's logits / T, (max, sum of exponentials), by the whole block.  Returns
+// true in every thread of the block that completes the last row of m's request.
+__device__ bool sample_row_stats(const MiscParams& p, int m, int b) {
+  const StepDesc* st = p.step;
+  __shared__ float redf[32];
+  __shared__ int s_last;
+  const int V = p.vocab, nt = blockDim.x;
+  const float invT = st->inv_temperature;
+  const float* lg = st->logits + static_cast<size_t>(caller_row(st, m)) * V;
+  auto fmx = [](float a, float c) { return a > c ? a : c; };
+  auto fsum = [](float a, float c) { return a + c; };
+  float mx = -INFINITY;
+  for (int b0 = threadIdx.x; b0 < V; b0 += kLoadBatch * nt) {
+    float x[kLoadBatch];
+#pragma unroll
+    for (int j = 0; j < kLoadBatch; ++j) x[j] = b0 + j * nt < V ? lg[b0 + j * nt] : -INFINITY;
+#pragma unroll
+    for (int j = 0; j < kLoadBatch; ++j) mx = fmx(mx, x[j]);
+  }
+  mx = block_reduce(mx, redf, fmx);
+  float z = 0.f;
+  for (int b0 = threadIdx.x; b0 < V; b0 += kLoadBatch * nt) {
+    float x[kLoadBatch];
+#pragma unroll
+    for (int j = 0; j < kLoadBatch; ++j) x[j] = b0 + j * nt < V ? lg[b0 + j * nt] : 0.f;
+#pragma unroll
+    for (int j = 0; j < kLoadBatch; ++j)
+      if (b0 + j * nt < V) z += expf((x[j] - mx) * invT);
+  }
+  z = block_reduce(z, redf, fsum);
+  if (threadIdx.x == 0) {
+    __stcg(&p.row_stat[2 * m], mx);
+    __stcg(&p.row_stat[2 * m + 1], z);
+    s_last = atom_add_acq_rel_gpu(&p.row_cnt[b], 1) == st->req_nodes[b] - 1;
+    if (s_last) atomicExch(&p.row_cnt[b], 0);
+  }
+  __syncthreads();
+  return s_last != 0;
+}
+
 // Speculative sampling on a chain draft (rule of the speculative-decoding works the paper cites
 // as its base methods): p_i = softmax(logits_i / T); accept draft x_i iff r_i * q_i(x_i) <
 // p_{i-1}(x_i); at the first rejection draw the bonus from normalise(max(0, p_{i-1} - q_i));
 // if every draft is accepted draw it from p_k.  Uniform slots: r_i at i-1, u_i at k+i-1.
+// A block per row computes the rows' statistics side by side, and the block that finishes a
+// request's last row runs the tests of all its drafts at once and the one inverse CDF that the walk
+// ends with.  Latency-bound: with one block per request and two passes over the vocabulary for
+// every row up to the first rejection, the acceptance of 8 requests of 5 drafts took 67 us.
 __device__ int accept_sample_body(const MiscParams& p, int b, int* path) {
   const StepDesc* st = p.step;
   __shared__ float scan[1025];
-  __shared__ float redf[32];
+  __shared__ float s_mx[kMaxNodes], s_iz[kMaxNodes];
+  __shared__ int s_stop[kMaxNodes];  // per draft: 0 accepted, 1 rejected, 2 token out of range; + 4: q(x) not positive
   const int N = st->req_nodes[b], off = st->req_rowoff[b], k = N - 1, V = p.vocab;
+  const size_t orow = static_cast<size_t>(st->req_orow[b]);
   const float invT = st->inv_temperature;
-  auto fmx = [](float a, float c) { return a > c ? a : c; };
-  auto fsum = [](float a, float c) { return a + c; };
-  int a = 0, bonus = 0;
-  for (int i = threadIdx.x; i < N; i += blockDim.x) path[i] = i;  // (read after the first barrier)
-  for (int i = 1; i <= k + 1; ++i) {
-    const float* lg = st->logits + static_cast<size_t>(off + i - 1) * V;
-    const int nt = blockDim.x;
-    float mx = -INFINITY;
-    for (int b0 = threadIdx.x; b0 < V; b0 += kLoadBatch * nt) {
-      float x[kLoadBatch];
-#pragma unroll
-      for (int j = 0; j < kLoadBatch; ++j) x[j] = b0 + j * nt < V ? lg[b0 + j * nt] : -INFINITY;
-#pragma unroll
-      for (int j = 0; j < kLoadBatch; ++j) mx = fmx(mx, x[j]);
-    }
-    mx = block_reduce(mx, redf, fmx);
-    float z = 0.f;
-    for (int b0 = threadIdx.x; b0 < V; b0 += kLoadBatch * nt) {
-      float x[kLoadBatch];
-#pragma unroll
-      for (int j = 0; j < kLoadBatch; ++j) x[j] = b0 + j * nt < V ? lg[b0 + j * nt] : 0.f;
-#pragma unroll
-      for (int j = 0; j < kLoadBatch; ++j)
-        if (b0 + j * nt < V) z += expf((x[j] - mx) * invT);
-    }
-    z = block_reduce(z, redf, fsum);
-    const float invz = 1.f / z;
-    auto pr = [&](int v) { return expf((lg[v] - mx) * invT) * invz; };
-    if (i <= k) {
-      const int x = st->tokens[off + i];
-      const float* q = st->draft_probs + static_cast<size_t>(off + i) * V;
-      if (x < 0 || x >= V) {
-        if (threadIdx.x == 0) report(p.status, kStatusCheck);
-        a = i - 1;
-        bonus = 0;
-        break;
-      }
-      const float qx = q[x];
-      if (!(qx > 0.f) && threadIdx.x == 0) report(p.status, kStatusCheck);
+  for (int i = threadIdx.x; i < N; i += blockDim.x) {
+    s_mx[i] = __ldcg(&p.row_stat[2 * (off + i)]);
+    s_iz[i] = 1.f / __ldcg(&p.row_stat[2 * (off + i) + 1]);
+    path[i] = i;
+  }
+  __syncthreads();
+  for (int i = 1 + threadIdx.x; i <= k; i += blockDim.x) {
+    const int x = st->tokens[orow + i];
+    int stop = 2;
+    if (x >= 0 && x < V) {
+      const float qx = st->draft_probs[(orow + i) * V + x];
+      const float px = expf((st->logits[(orow + i - 1) * V + x] - s_mx[i - 1]) * invT) * s_iz[i - 1];
       const float r = static_cast<float>(draw_uniform(st, b, i - 1));
-      if (r * qx < pr(x)) continue;  // accept draft i
-      const float u = static_cast<float>(draw_uniform(st, b, k + i - 1));
-      bonus = inverse_cdf_staged(V, u, [&](int v) {
-        const float d = pr(v) - q[v];
-        return d > 0.f ? d : 0.f;
-      }, scan);
-      a = i - 1;
-      break;
+      stop = (r * qx < px ? 0 : 1) + (qx > 0.f ? 0 : 4);
     }
-    const float u = static_cast<float>(draw_uniform(st, b, 2 * k));
-    bonus = inverse_cdf_staged(V, u, pr, scan);
-    a = k;
+    s_stop[i] = stop;
+  }
+  __syncthreads();
+  int i = 1;  // first draft that is not accepted, k + 1: none
+  while (i <= k && (s_stop[i] & 3) == 0) ++i;
+  if (threadIdx.x == 0)
+    for (int j = 1; j <= min(i, k); ++j)
+      if (s_stop[j] >= 2) report(p.status, kStatusCheck);
+  const int a = i - 1;
+  int bonus = 0;
+  const float* lg = st->logits + (orow + a) * V;
+  const float mx = s_mx[a], invz = s_iz[a];
+  auto pr = [&](int v) { return expf((lg[v] - mx) * invT) * invz; };
+  if (i > k) {
+    bonus = inverse_cdf_staged(V, static_cast<float>(draw_uniform(st, b, 2 * k)), pr, scan);
+  } else if ((s_stop[i] & 3) == 1) {
+    const float* q = st->draft_probs + (orow + i) * V;
+    bonus = inverse_cdf_staged(V, static_cast<float>(draw_uniform(st, b, k + i - 1)), [&](int v) {
+      const float d = pr(v) - q[v];
+      return d > 0.f ? d : 0.f;
+    }, scan);
   }
   __syncthreads();
   write_result(p, b, a, bonus, path);
@@ -490,9 +520,12 @@ __device__ int accept_sample_body(const MiscParams& p, int b, int* path) {
 __global__ void __launch_bounds__(1024) accept_sample_kernel(const MiscParams p) {
   griddep_wait();
   griddep_launch();
-  if (blockIdx.x >= p.step->B) return;
+  const int m = blockIdx.x;  // a block per row
+  if (m >= p.step->M) return;
+  const int b = p.step->row_req[m];
+  if (!sample_row_stats(p, m, b)) return;
   __shared__ int path[kMaxNodes];
-  accept_sample_body(p, blockIdx.x, path);
+  accept_sample_body(p, b, path);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -513,7 +546,7 @@ __global__ void __launch_bounds__(256) prologue_kernel(const MiscParams p, float
   const StepDesc* st = p.step;
   const int m = blockIdx.x - 1;
   if (m >= st->M) return;
-  int tok = st->tokens[m];
+  int tok = st->tokens[caller_row(st, m)];
   if (tok < 0 || tok >= p.vocab) {
     if (threadIdx.x == 0) report(p.status, kStatusCheck);
     tok = 0;
@@ -590,17 +623,25 @@ __global__ void __launch_bounds__(256) prologue_kernel(const MiscParams p, float
 
 // ------------------------------------------------------------------------------------------
 // Step finish: acceptance of request b (greedy walk or speculative sampling), then the KV
-// compaction of its accepted path in every layer it ran (one 1024-thread block per request).
+// compaction of its accepted path in every layer it ran (one 1024-thread block per request; when
+// sampling, one per row: see accept_sample_body).
 // ------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(1024) finish_kernel(const MiscParams p) {
   griddep_wait();
   griddep_launch();
   const StepDesc* st = p.step;
   const PlanDev* pl = p.plan;
+  __shared__ int path[kMaxNodes];
+  if (st->mode == TSS_MODE_SAMPLE) {  // a block per row; chains only, whose accepted rows are in place
+    const int m = blockIdx.x;
+    if (m >= st->M) return;
+    const int b = st->row_req[m];
+    if (sample_row_stats(p, m, b)) accept_sample_body(p, b, path);
+    return;
+  }
   const int b = blockIdx.x;
   if (b >= st->B) return;
-  __shared__ int path[kMaxNodes];
-  const int a = st->mode == TSS_MODE_SAMPLE ? accept_sample_body(p, b, path) : accept_greedy_body(p, b, path);
+  const int a = accept_greedy_body(p, b, path);
   if (a <= 0) return;
   // A chain's accepted rows are already in place (path[j] == j): nothing moves in any layer.
   bool moved = false;
@@ -691,8 +732,8 @@ cudaError_t launch_prologue(const MiscParams& p, float* ssp, int* zero_ints, int
                             bool pdl) {
   return launch_k(prologue_kernel, dim3(M + 1), dim3(256), 0, s, pdl, p, ssp, zero_ints, n_zero);
 }
-cudaError_t launch_finish(const MiscParams& p, int B, bool sample, cudaStream_t s, bool pdl) {
-  return launch_k(finish_kernel, dim3(B), dim3(1024), sample ? cdf_stage_bytes(p.vocab) : 0, s, pdl, p);
+cudaError_t launch_finish(const MiscParams& p, int B, int M, bool sample, cudaStream_t s, bool pdl) {
+  return launch_k(finish_kernel, dim3(sample ? M : B), dim3(1024), sample ? cdf_stage_bytes(p.vocab) : 0, s, pdl, p);
 }
 
 cudaError_t launch_controller(const MiscParams& p, cudaStream_t s, bool pdl) {
@@ -707,8 +748,8 @@ cudaError_t launch_rmsnorm(const MiscParams& p, int slot, int which, int M, cuda
 cudaError_t launch_accept_greedy(const MiscParams& p, int B, cudaStream_t s, bool pdl) {
   return launch_k(accept_greedy_kernel, dim3(B), dim3(256), 0, s, pdl, p);
 }
-cudaError_t launch_accept_sample(const MiscParams& p, int B, cudaStream_t s, bool pdl) {
-  return launch_k(accept_sample_kernel, dim3(B), dim3(1024), cdf_stage_bytes(p.vocab), s, pdl, p);
+cudaError_t launch_accept_sample(const MiscParams& p, int M, cudaStream_t s, bool pdl) {
+  return launch_k(accept_sample_kernel, dim3(M), dim3(1024), cdf_stage_bytes(p.vocab), s, pdl, p);
 }
 cudaError_t launch_compact(const MiscParams& p, int B, int n_act, cudaStream_t s, bool pdl) {
   if (n_act <= 0) n_act = 1;

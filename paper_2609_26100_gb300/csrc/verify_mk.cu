@@ -331,7 +331,7 @@ __device__ __forceinline__ void mk_acc_tokens(uint32_t tb, int ch, const XsLayou
 struct MkEpi {
   int M;
   const int* rows;  // shared-memory copy of the phase's compacted row list
-  int* pos;         // [kMaxRows] RoPE position of each compacted row (QKV)
+  int* pos;         // [kMaxRows] RoPE position of each compacted row (QKV); LM head: its row in the caller's logits
   int* kvslot;      // [kMaxRows] KV-cache slot and row of each compacted row (QKV)
   int* kvrow;
   // residual phases: the next norm phase's B operand bf16(h * g_next) is written by the epilogue
@@ -609,7 +609,7 @@ __device__ void mk_finish_rows(const MkParams& p, const MkPhase& ph, const MkEpi
           }
         }
         if (e.logits && in) {
-          float* lg = e.logits + static_cast<size_t>(e.rows[j]) * p.V + o0;
+          float* lg = e.logits + static_cast<size_t>(e.pos[j]) * p.V + o0;
           if (e.logits_vec) {  // (V is a multiple of 4: all four features exist, or none)
             if (o0 < p.V) *reinterpret_cast<float4*>(lg) = make_float4(val[0], val[1], val[2], val[3]);
           } else {
@@ -1061,6 +1061,7 @@ __global__ void __launch_bounds__(kMkThreads, 1)
           s_kvslot[j] = p.step->req_slot[b];
           s_kvrow[j] = p.step->req_ctx[b] + (m - p.step->req_rowoff[b]);
         }
+        if (ph.kind == kMkLm) s_pos[j] = caller_row(p.step, m);
       }
       e.n_extra = 0;
       if (mk_resid(ph)) {
