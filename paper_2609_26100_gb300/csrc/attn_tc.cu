@@ -18,8 +18,8 @@
 // sums and O are rescaled then), so a typical tile needs no reduction across keys.
 //
 // Work split: the (request, head) items of the requests that run this layer, each cut into
-// 128-key tiles, are laid end to end and cut into min(grid, tiles) equal ranges, one per CTA
-// (one CTA per SM).  A CTA streams its range through two three-slot TMA rings -- keys, released
+// 128-key tiles and led by kTcItem units for what an item costs beside its tiles, are laid end to
+// end and cut into min(grid, units) equal ranges, one per CTA (one CTA per SM).  A CTA streams its range through two three-slot TMA rings -- keys, released
 // as soon as their score product completes, and values, released after P.V -- and produces one
 // result per item it covers: the output itself when it holds the whole item, else a partial
 // (O, max, sum) that the last CTA to finish the item merges with the others in CTA order.
@@ -46,6 +46,13 @@ constexpr uint32_t kQBytes = 2 * kOpBytes;    // Q operand: 128 columns
 constexpr uint32_t kPBytes = 2 * kOpBytes;    // P operand: 128 keys
 constexpr uint32_t kTmemCols = 128;           // S^T x 2 (cols 0-63), O^T x 2 (cols 64-127), 32 each
 constexpr uint32_t kOCol = 64;
+// An item's fixed cost in tiles: the first tile's column maxima, the last tile's mask and sums, Q and
+// the output.  With tiles alone in the balance the CTA that got 33 one-tile items of a batch of
+// ragged contexts (24 requests of 33-2047 tokens) took 159 us and the mean 86.  Units 0 / 2 / 3 / 5,
+// us a launch: that batch (average over its layers) 126 / 87 / 85 / 85, five requests of 50-16000
+// tokens 159 / 82 / 79 / 79, 13B of 8 requests 71 / 66 / 66 / 67, 16 x 16384 tokens (HBM-bound)
+// 616 at any.
+constexpr int kTcItem = 3;
 constexpr float kRaise = 8.f;                 // log2 headroom before the running max is raised
 
 struct TcShared {
@@ -55,7 +62,7 @@ struct TcShared {
   uint32_t tmem;
   int abort;
   int last;
-  int cum[kMaxBatch + 1];   // prefix sums of the (request, head) tiles over the requests
+  int cum[kMaxBatch + 1];   // prefix sums over the requests of their items' units (tiles + kTcItem each)
   float red[4][kTcRows];    // softmax: per-warp column maxima
   float hm[2][kTcRows];     // softmax -> epilogue: running maxima of an item's part
   float hl[2][4][kTcRows];  // ... and the per-warp sums of its weights
@@ -125,16 +132,17 @@ __device__ __forceinline__ int tc_cta_of(long long g, long long T, int C) {
   return static_cast<int>(((g + 1) * C - 1) / T);
 }
 
-// Cursor over a CTA's tiles in the global order (request, head, key tile).
+// Cursor over a CTA's tiles in the global order (request, head, key tile).  An item's units are its
+// kTcItem leading ones and then its tiles; start(g) is the first tile at unit g or later.
 struct TcCursor {
   int b, h, kt, nt;  // nt: tiles of each head of request b
   __device__ void start(const TcShared& sh, int B, int H, long long g) {
     b = 0;
     while (b + 1 < B && sh.cum[b + 1] <= g) ++b;
-    nt = (sh.cum[b + 1] - sh.cum[b]) / H;
-    const int r = static_cast<int>(g - sh.cum[b]);
-    h = r / nt;
-    kt = r - h * nt;
+    const int L = (sh.cum[b + 1] - sh.cum[b]) / H, r = static_cast<int>(g - sh.cum[b]);
+    nt = L - kTcItem;
+    h = r / L;
+    kt = max(r - h * L - kTcItem, 0);
   }
   __device__ void next(const TcShared& sh, int B, int H) {
     if (++kt < nt) return;
@@ -144,7 +152,7 @@ struct TcCursor {
     do {
       ++b;
     } while (b < B && sh.cum[b + 1] == sh.cum[b]);
-    if (b < B) nt = (sh.cum[b + 1] - sh.cum[b]) / H;
+    if (b < B) nt = (sh.cum[b + 1] - sh.cum[b]) / H - kTcItem;
   }
 };
 
@@ -430,7 +438,7 @@ __device__ __forceinline__ void tc_epilogue(const AttnTcParams& p, TcShared& sh,
       mbar_arrive(&sh.h_free[j & 1]);
     }
     const int item = b * H + h;
-    const long long gi0 = sh.cum[b] + static_cast<long long>(h) * nt;
+    const long long gi0 = sh.cum[b] + static_cast<long long>(h) * (nt + kTcItem) + kTcItem;  // its first tile
     const int cf = tc_cta_of(gi0, T, C), cl = tc_cta_of(gi0 + nt - 1, T, C);
     const int col = h * kTcD + e;
     if (cf == cl) {
@@ -521,13 +529,15 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_tc_kernel(const AttnTcPara
   griddep_wait();
   if (p.slot >= pl->n_act) return;
   const int B = st->B, H = p.n_heads;
+  // (the requests' lengths by a thread each: one round of loads instead of one per request)
+  for (int b = tid; b < B; b += kTcThreads)
+    sh.cum[b + 1] = pl->slot_crow[p.slot][b] < 0
+                        ? 0
+                        : H * ((st->req_ctx[b] + st->req_nodes[b] + kTcKeys - 1) / kTcKeys + kTcItem);
+  __syncthreads();
   if (tid == 0) {
-    int acc = 0;
     sh.cum[0] = 0;
-    for (int b = 0; b < B; ++b) {
-      if (pl->slot_crow[p.slot][b] >= 0) acc += H * ((st->req_ctx[b] + st->req_nodes[b] + kTcKeys - 1) / kTcKeys);
-      sh.cum[b + 1] = acc;
-    }
+    for (int b = 0; b < B; ++b) sh.cum[b + 1] += sh.cum[b];
     sh.abort = 0;
     for (int i = 0; i < kTcStages; ++i) {
       mbar_init(&sh.kfull[i], 1);
@@ -550,13 +560,23 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_tc_kernel(const AttnTcPara
     fence_mbar_init();
   }
   __syncthreads();
-  // ranges for C = min(grid, T) CTAs, so that every range holds at least one tile (an item's
-  // partials then come from every CTA between the ones holding its first and last tiles)
+  // ranges for C = min(grid, T) CTAs, so that no range is empty and an item's partials come from
+  // every CTA between the ones holding its first and last tiles
   const long long T = sh.cum[B];
   const int C = static_cast<int>(T < gridDim.x ? T : gridDim.x), c = blockIdx.x;
   if (c >= C) return;  // (the whole CTA)
   const long long g0 = c * T / C, g1 = (c + 1) * T / C;
-  const int n = static_cast<int>(g1 - g0);
+  // tiles in [g0, g1): a position's tiles are those of the items before it and, in its own item, of
+  // the units past the leading ones
+  auto tiles_before = [&](long long g) -> int {
+    int b = 0, before = 0;
+    for (; b + 1 < B && sh.cum[b + 1] <= g; ++b) before += sh.cum[b + 1] > sh.cum[b] ? H * kTcItem : 0;
+    if (g >= sh.cum[B]) return sh.cum[B] - before - (sh.cum[b + 1] > sh.cum[b] ? H * kTcItem : 0);
+    const int L = (sh.cum[b + 1] - sh.cum[b]) / H, r = static_cast<int>(g - sh.cum[b]), h = r / L;
+    return sh.cum[b] - before + h * (L - kTcItem) + max(r - h * L - kTcItem, 0);
+  };
+  const int n = tiles_before(g1) - tiles_before(g0);
+  if (n == 0) return;  // (only leading units: no tile, no partial)
   if (warp == 0) {
     tmem_alloc(&sh.tmem, kTmemCols);
     tmem_relinquish();
@@ -618,8 +638,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_tc_kernel(const AttnTcPara
       cur.start(sh, B, H, g0);
       int seg_s = -1, pv_seg = 0;
       bool pv_first = false, pv_last = false;
-      // fault injection: CTA 0 issues no MMA, so its softmax's first wait runs out
-      const int n_issue = p.withhold && blockIdx.x == 0 ? -1 : n;
+      // fault injection: the CTA of the first tile issues no MMA, so its softmax's first wait runs out
+      const int n_issue = p.withhold && c == tc_cta_of(kTcItem, T, C) ? -1 : n;
       for (int t = 0; t <= n_issue; ++t) {
         bool first = false, last = false;
         if (t < n) {

@@ -93,7 +93,7 @@ struct AttnTcParams {
   float* part_ml;                // [attn_tc_partial_rows][2]
   int* counters;                 // [B][H], self-resetting
   int* status;
-  int withhold;                  // fault injection: CTA 0 issues no MMA (its first wait runs out)
+  int withhold;                  // fault injection: the first tile's CTA issues no MMA (its first wait runs out)
 };
 // Compute-bound prefill (prefill.cu; head_dim 128): one pass = T rows holding the prompt chunks
 // of requests with the same skip set, each chunk starting at a multiple of 128 rows (rows in the
