@@ -252,6 +252,8 @@ MiscParams misc_params(tss_ctx* c) {
 GemmParams gemm_base(tss_ctx* c, int n_pad) {
   GemmParams g{};
   g.n_pad = n_pad;
+  g.kps = 1;
+  g.n_acc = 1;
   g.plan = c->d_plan;
   g.step = c->d_step;
   g.partials = c->partials;

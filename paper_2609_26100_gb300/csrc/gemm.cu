@@ -36,19 +36,42 @@ size_t gemm_smem_bytes(int n_pad, int stages) {
          + 2 * 4 * 16 * 4;                              // argmax reduction
 }
 
-__device__ __forceinline__ int cta_of(long long i, long long T, int G) {
+// (32-bit: T x CTAs is a few hundred times a matrix's 16 KiB blocks, below 2^32 on any device)
+__device__ __forceinline__ int cta_of(uint32_t i, uint32_t T, uint32_t G) {
   return static_cast<int>(((i + 1) * G - 1) / T);
 }
 
-__device__ __forceinline__ bool next_segment(long long& it, long long end, int kb, int& t, int& k0, int& k1) {
+__device__ __forceinline__ bool next_segment(uint32_t& it, uint32_t end, uint32_t kb, int& t, int& k0, int& k1) {
   if (it >= end) return false;
-  t = static_cast<int>(it / kb);
-  k0 = static_cast<int>(it - static_cast<long long>(t) * kb);
-  const long long tile_end = static_cast<long long>(t + 1) * kb;
-  const long long e = end < tile_end ? end : tile_end;
-  k1 = static_cast<int>(e - static_cast<long long>(t) * kb);
-  it = e;
+  const uint32_t tile = it / kb, t0 = tile * kb;
+  t = static_cast<int>(tile);
+  k0 = static_cast<int>(it - t0);
+  it = min(end, t0 + kb);
+  k1 = static_cast<int>(it - t0);
   return true;
+}
+
+// Position in the pipeline ring: slot and the parity of its turn.
+struct GemmRing {
+  int s = 0;
+  uint32_t turn = 0;
+  __device__ __forceinline__ void next(int n) {
+    if (++s == n) {
+      s = 0;
+      turn ^= 1u;
+    }
+  }
+};
+
+// 16 columns of a tile's accumulators, added in fp32.
+__device__ __forceinline__ void acc_chunk(uint32_t taddr, int n_acc, int n_pad, float* v) {
+  tmem_ld16(taddr, v);
+  for (int a = 1; a < n_acc; ++a) {
+    float x[16];
+    tmem_ld16(taddr + a * n_pad, x);
+#pragma unroll
+    for (int jj = 0; jj < 16; ++jj) v[jj] += x[jj];
+  }
 }
 
 struct EpiCtx {
@@ -207,12 +230,12 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
     gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmX, const GemmParams p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  const int S = p.stages;
+  const int S = p.stages, KPS = p.kps;
   const int n_pad = p.n_pad;
   const uint32_t x_bytes = static_cast<uint32_t>(n_pad) * 128u;
   uint8_t* sW = base;
-  uint8_t* sX = base + static_cast<size_t>(S) * kWTileBytes;
-  uint64_t* full = reinterpret_cast<uint64_t*>(sX + static_cast<size_t>(S) * x_bytes);
+  uint8_t* sX = base + static_cast<size_t>(S) * KPS * kWTileBytes;
+  uint64_t* full = reinterpret_cast<uint64_t*>(sX + static_cast<size_t>(S) * KPS * x_bytes);
   uint64_t* empty = full + S;
   uint64_t* accf = empty + S;
   uint64_t* acce = accf + 2;
@@ -224,7 +247,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
   int* redi = reinterpret_cast<int*>(redv + 64);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t ncols = gemm_tmem_cols(n_pad, p.n_acc_bufs);
+  const int NA = p.n_acc;  // accumulators of a tile: the MMAs of a k-block go round them
+  const uint32_t ncols = gemm_tmem_cols(n_pad * NA, p.n_acc_bufs);
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < S; ++i) {
@@ -249,9 +273,9 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
 
-  const long long T = static_cast<long long>(p.n_tiles) * p.kb;
-  const int G = gridDim.x, c = blockIdx.x;
-  const long long it0 = T * c / G, it1 = T * (c + 1) / G;
+  const uint32_t T = static_cast<uint32_t>(p.n_tiles) * p.kb;
+  const uint32_t G = gridDim.x, c = blockIdx.x;
+  const uint32_t it0 = T * c / G, it1 = T * (c + 1) / G;
 
   if (warp == 0) {
     if (lane == 0) {
@@ -260,39 +284,50 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
       // dependents only after its own griddepcontrol.wait, so that kernel has completed here.
       int layer = p.layer_fixed;
       if (layer < 0) layer = p.slot < p.plan->n_act ? p.plan->act_layer[p.slot] : 0;
-      const long long n_it = it1 - it0;
-      const int pre = static_cast<int>(n_it < S ? n_it : S);
-      for (int i = 0; i < pre; ++i) {
-        const long long it = it0 + i;
-        const int t = static_cast<int>(it / p.kb), kk = static_cast<int>(it % p.kb);
-        mbar_arrive_expect_tx(&full[i], kWTileBytes + x_bytes);
-        if (p.w_tiled)
-          bulk_load(sW + static_cast<size_t>(i) * kWTileBytes,
-                    p.w_tiled + layer * p.w_layer_elems + (static_cast<size_t>(t) * p.kb + kk) * kTileElems, kWTileBytes,
-                    &full[i]);
-        else
-          tma_load_3d(sW + static_cast<size_t>(i) * kWTileBytes, &tmW, &full[i], kk * 64, t * 128, layer);
-      }
+      // a stage: the next KPS k-blocks of one tile (fewer at the end of a segment)
+      auto load_w = [&](int s, int t, int kk, int nk) {
+        for (int j = 0; j < nk; ++j) {
+          uint8_t* dst = sW + static_cast<size_t>(s * KPS + j) * kWTileBytes;
+          if (p.w_tiled)
+            bulk_load(dst, p.w_tiled + layer * p.w_layer_elems + (static_cast<size_t>(t) * p.kb + kk + j) * kTileElems,
+                      kWTileBytes, &full[s]);
+          else
+            tma_load_3d(dst, &tmW, &full[s], (kk + j) * 64, t * 128, layer);
+        }
+      };
+      auto load_x = [&](int s, int kk, int nk) {
+        for (int j = 0; j < nk; ++j)
+          tma_load_2d(sX + static_cast<size_t>(s * KPS + j) * x_bytes, &tmX, &full[s], (kk + j) * 64, 0);
+      };
+      // the first stages' weights before the previous kernel's results are waited for
+      uint32_t it = it0;
+      int t, k0, k1, pre = 0;
+      while (pre < S && next_segment(it, it1, p.kb, t, k0, k1))
+        for (int kk = k0; kk < k1 && pre < S; kk += KPS, ++pre) {
+          const int nk = min(KPS, k1 - kk);
+          mbar_arrive_expect_tx(&full[pre], nk * (kWTileBytes + x_bytes));
+          load_w(pre, t, kk, nk);
+        }
       griddep_wait();
       griddep_launch();
-      for (int i = 0; i < pre; ++i) {
-        const int kk = static_cast<int>((it0 + i) % p.kb);
-        tma_load_2d(sX + static_cast<size_t>(i) * x_bytes, &tmX, &full[i], kk * 64, 0);
-      }
-      for (long long i = pre; i < n_it; ++i) {
-        const int s = static_cast<int>(i % S);
-        const uint32_t ph = static_cast<uint32_t>((i / S) & 1) ^ 1u;
-        if (!mbar_wait(&empty[s], ph, abort_flag, p.status)) break;
-        const long long it = it0 + i;
-        const int t = static_cast<int>(it / p.kb), kk = static_cast<int>(it % p.kb);
-        mbar_arrive_expect_tx(&full[s], kWTileBytes + x_bytes);
-        if (p.w_tiled)
-          bulk_load(sW + static_cast<size_t>(s) * kWTileBytes,
-                    p.w_tiled + layer * p.w_layer_elems + (static_cast<size_t>(t) * p.kb + kk) * kTileElems, kWTileBytes,
-                    &full[s]);
-        else
-          tma_load_3d(sW + static_cast<size_t>(s) * kWTileBytes, &tmW, &full[s], kk * 64, t * 128, layer);
-        tma_load_2d(sX + static_cast<size_t>(s) * x_bytes, &tmX, &full[s], kk * 64, 0);
+      GemmRing ring;
+      it = it0;
+      int i = 0;
+      bool ok = true;
+      while (ok && next_segment(it, it1, p.kb, t, k0, k1)) {
+        for (int kk = k0; kk < k1; kk += KPS, ++i) {
+          const int nk = min(KPS, k1 - kk), s = ring.s;
+          if (i >= pre) {
+            if (!mbar_wait(&empty[s], ring.turn ^ 1u, abort_flag, p.status)) {
+              ok = false;
+              break;
+            }
+            mbar_arrive_expect_tx(&full[s], nk * (kWTileBytes + x_bytes));
+            load_w(s, t, kk, nk);
+          }
+          load_x(s, kk, nk);
+          ring.next(S);
+        }
       }
     }
   } else if (warp == 1) {
@@ -301,30 +336,35 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
       griddep_wait();
       griddep_launch();
       const uint32_t idesc = idesc_bf16_m128(n_pad);
-      long long it = it0, i = 0;
+      uint32_t it = it0;
       int t, k0, k1, use = 0;
       bool ok = true;
+      GemmRing ring;
       while (ok && next_segment(it, it1, p.kb, t, k0, k1)) {
         const int buf = p.n_acc_bufs == 2 ? (use & 1) : 0;
         const int ub = p.n_acc_bufs == 2 ? (use >> 1) : use;
         if (!mbar_wait(&acce[buf], static_cast<uint32_t>(ub & 1) ^ 1u, abort_flag, p.status)) break;
         tc_fence_after();
-        const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(buf * n_pad);
-        for (int kk = k0; kk < k1; ++kk, ++i) {
-          const int s = static_cast<int>(i % S);
-          if (!mbar_wait(&full[s], static_cast<uint32_t>((i / S) & 1), abort_flag, p.status)) {
+        const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(buf * NA * n_pad);
+        const uint32_t d_step = NA == 4 ? n_pad : 0;
+        for (int kk = k0; kk < k1; kk += KPS) {
+          const int nk = min(KPS, k1 - kk), s = ring.s;
+          if (!mbar_wait(&full[s], ring.turn, abort_flag, p.status)) {
             ok = false;
             break;
           }
           tc_fence_after();
-          const uint32_t a0 = smem_u32(sW + static_cast<size_t>(s) * kWTileBytes);
-          const uint32_t b0 = smem_u32(sX + static_cast<size_t>(s) * x_bytes);
+          for (int j = 0; j < nk; ++j) {
+            const uint32_t a0 = smem_u32(sW + static_cast<size_t>(s * KPS + j) * kWTileBytes);
+            const uint32_t b0 = smem_u32(sX + static_cast<size_t>(s * KPS + j) * x_bytes);
 #pragma unroll
-          for (int k16 = 0; k16 < 4; ++k16) {
-            umma_bf16(d_tmem, sdesc_sw128(a0 + k16 * 32), sdesc_sw128(b0 + k16 * 32), idesc,
-                      (kk > k0 || k16 > 0) ? 1u : 0u);
+            for (int k16 = 0; k16 < 4; ++k16) {
+              umma_bf16(d_tmem + k16 * d_step, sdesc_sw128(a0 + k16 * 32), sdesc_sw128(b0 + k16 * 32), idesc,
+                        (kk + j > k0 || (k16 > 0 && NA == 1)) ? 1u : 0u);
+            }
           }
           umma_commit(&empty[s]);
+          ring.next(S);
         }
         if (!ok) break;
         umma_commit(&accf[buf]);
@@ -355,19 +395,19 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
       e.layer = p.layer_fixed;
     }
     const int r = e.q * 32 + lane;
-    long long it = it0;
+    uint32_t it = it0;
     int t, k0, k1, use = 0;
     while (next_segment(it, it1, p.kb, t, k0, k1)) {
       const int buf = p.n_acc_bufs == 2 ? (use & 1) : 0;
       const int ub = p.n_acc_bufs == 2 ? (use >> 1) : use;
       if (!mbar_wait(&accf[buf], static_cast<uint32_t>(ub & 1), abort_flag, p.status)) break;
       tc_fence_after();
-      const uint32_t tb = tmem_base + (static_cast<uint32_t>(e.q * 32) << 16) + static_cast<uint32_t>(buf * n_pad);
+      const uint32_t tb = tmem_base + (static_cast<uint32_t>(e.q * 32) << 16) + static_cast<uint32_t>(buf * NA * n_pad);
       const int n_ch = n_pad >> 4;
       if (k0 == 0 && k1 == p.kb) {
         for (int ch = 0; ch < n_ch; ++ch) {
           float v[16];
-          tmem_ld16(tb + ch * 16, v);
+          acc_chunk(tb + ch * 16, NA, n_pad, v);
           epilogue_chunk<EPI>(p, e, t, r, ch, v);
         }
         tc_fence_before();
@@ -376,16 +416,16 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
         float* part = p.partials + static_cast<size_t>(c + t) * 128 * n_pad;
         for (int ch = 0; ch < n_ch; ++ch) {
           float v[16];
-          tmem_ld16(tb + ch * 16, v);
+          acc_chunk(tb + ch * 16, NA, n_pad, v);
 #pragma unroll
-          for (int jj = 0; jj < 16; ++jj) __stcg(&part[(ch * 16 + jj) * 128 + r], v[jj]);
+          for (int jj = 0; jj < 16; ++jj)
+            if (ch * 16 + jj < e.M) __stcg(&part[(ch * 16 + jj) * 128 + r], v[jj]);
         }
         tc_fence_before();
         mbar_arrive(&acce[buf]);
         named_bar_sync(1, 128);  // every thread's partial stores precede the release below
         if (e.et == 0) {
-          const int cf = cta_of(static_cast<long long>(t) * p.kb, T, G);
-          const int cl = cta_of(static_cast<long long>(t + 1) * p.kb - 1, T, G);
+          const int cf = cta_of(t * p.kb, T, G), cl = cta_of((t + 1) * p.kb - 1, T, G);
           const int old = atom_add_acq_rel_gpu(&p.counters[t], 1);
           const int last = old == cl - cf;
           if (last) atomicExch(&p.counters[t], 0);
@@ -400,10 +440,20 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
             float v[16];
 #pragma unroll
             for (int jj = 0; jj < 16; ++jj) v[jj] = 0.f;
-            for (int cc = cf; cc <= cl; ++cc) {
-              const float* pp = p.partials + static_cast<size_t>(cc + t) * 128 * n_pad;
+            // contributors in order, four of them per round of loads
+            for (int c0 = cf; c0 <= cl; c0 += 4) {
+              float x[4][16];
 #pragma unroll
-              for (int jj = 0; jj < 16; ++jj) v[jj] += __ldcg(&pp[(ch * 16 + jj) * 128 + r]);
+              for (int q = 0; q < 4; ++q) {
+                const float* pp = p.partials + static_cast<size_t>(c0 + q + t) * 128 * n_pad;
+#pragma unroll
+                for (int jj = 0; jj < 16; ++jj)
+                  x[q][jj] = c0 + q <= cl && ch * 16 + jj < e.M ? __ldcg(&pp[(ch * 16 + jj) * 128 + r]) : 0.f;
+              }
+#pragma unroll
+              for (int q = 0; q < 4; ++q)
+#pragma unroll
+                for (int jj = 0; jj < 16; ++jj) v[jj] += x[q][jj];
             }
             epilogue_chunk<EPI>(p, e, t, r, ch, v);
           }
@@ -419,6 +469,13 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc(tmem_base, ncols);
+  }
+  // (callers without a clearing pass of their own) The last CTA to leave clears the arrival counters
+  // where a wait has run out in this or an earlier launch, so that the next launch starts at zero.
+  if (p.exits && threadIdx.x == 0 && atom_add_acq_rel_gpu(p.exits, 1) == static_cast<int>(G) - 1) {
+    *p.exits = 0;
+    if (*reinterpret_cast<volatile int*>(p.status) != 0)
+      for (int t = 0; t < p.n_tiles; ++t) p.counters[t] = 0;
   }
 }
 

@@ -22,6 +22,8 @@ struct GemmParams {
   int kb;           // k-blocks of 64 per tile
   int n_pad;        // MMA N = token rows padded to a multiple of 16 (<= 256)
   int stages;       // smem pipeline depth
+  int kps;          // k-blocks per stage
+  int n_acc;        // accumulators of a tile (1, or 4 with n_pad <= 64)
   int n_acc_bufs;   // TMEM accumulator buffers (1 or 2)
   int slot;         // plan slot whose compacted rows feed the GEMM; -1: plain rows [0, m_raw)
   int m_raw;
@@ -32,6 +34,7 @@ struct GemmParams {
   const StepDesc* step;
   float* partials;  // stream-K partial tiles [(grid + n_tiles) * 128 * n_pad]
   int* counters;    // per-tile arrival counters (self-resetting)
+  int* exits;       // optional: CTAs that have left (self-resetting); the last clears counters after a timeout
   int* status;
   float* out;       // kEpiStore
   int out_ld;

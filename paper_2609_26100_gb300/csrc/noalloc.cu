@@ -30,7 +30,7 @@ constexpr int kStaticMaxRows = 64;
 constexpr int kMaxDevices = 64;
 
 static __device__ __align__(256) float g_static_partials[kStaticPartialFloats];
-static __device__ __align__(256) int g_static_counters[kStaticCounters];
+static __device__ __align__(256) int g_static_counters[kStaticCounters + 1];  // ... and the CTAs that have left
 // First failure of a device-side check or bounded wait since the last tss_linear_static_status
 // (0: none); the GEMM kernel records it and never traps.
 static __device__ __align__(256) int g_static_status;
@@ -120,36 +120,44 @@ extern "C" tss_status tss_linear_static(const void* x, const void* w, float* y, 
   const int n_pad = (m_rows + 15) / 16 * 16;
   const int n_tiles = n_out / 128, kb = k_dim / 64;
   const long long T = static_cast<long long>(n_tiles) * kb;
-  const int grid = static_cast<int>(T < ds->num_sms ? T : ds->num_sms);  // one CTA per SM
+  int grid = static_cast<int>(T < ds->num_sms ? T : ds->num_sms);  // one CTA per SM
   const size_t need = static_cast<size_t>(grid + n_tiles) * 128 * n_pad;
   if (need > kStaticPartialFloats)
     return reject(TSS_ERR_INVALID_ARG, "problem needs " + std::to_string(need * 4) +
                                            " bytes of stream-K scratch; the static limit is 8 MiB");
+  // One CTA per tile where that streams a CTA at most 31 k-blocks (about 0.23 us each) more than an even
+  // share -- about what storing, counting and adding partial sums costs (6 rows, k 4096, n 8192 /
+  // 10240 / 12288 / 14336: split 20.5 / 23.6 / 27.1 / 29.4 us, whole 22.6 / 22.7 / 24.7 / 26.9) -- and sums
+  // no accumulator longer than a split one was (four accumulators share a whole tile's k-blocks).
+  if (n_tiles <= grid && kb <= T / grid + 31 && static_cast<long long>(kb) * grid <= 4 * T) grid = n_tiles;
+  // Stages of three k-blocks (48 KiB of weights): a stage's fixed cost is that of one barrier round
+  // trip and its issue, whatever its size (6 x 4096 x 12288: 28.6 us with one k-block a stage).
+  const int kps = kb < 3 ? 1 : 3;
   int stages = 2;
-  while (stages < 12 && tss::gemm_smem_bytes(n_pad, stages + 1) <= 220 * 1024) ++stages;
+  while (stages < 12 / kps && tss::gemm_smem_bytes(n_pad, (stages + 1) * kps) <= 228 * 1024) ++stages;
   CUtensorMap tx, tw;
   if (!encode(&tx, x, k_dim, m_rows, n_pad, 2) || !encode(&tw, w, k_dim, n_out, 128, 3))
     return reject(TSS_ERR_CUDA, "cuTensorMapEncodeTiled failed");
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  // The counters must start at zero; a call cut short by a device timeout could leave them set.
-  e = cudaMemsetAsync(ds->counters, 0, sizeof(int) * n_tiles, s);
-  if (e != cudaSuccess) return reject(TSS_ERR_CUDA, std::string("cudaMemsetAsync: ") + cudaGetErrorString(e));
   tss::GemmParams g{};
   g.n_tiles = n_tiles;
   g.kb = kb;
   g.n_pad = n_pad;
   g.stages = stages;
+  g.kps = kps;
+  g.n_acc = 4;  // (error against 64 bits of a k of 4096: 5e-7 to 1e-6, with one accumulator 2e-6 to 4e-6)
   g.n_acc_bufs = 2;
   g.slot = -1;
   g.m_raw = m_rows;
   g.layer_fixed = 0;
   g.partials = ds->partials;
-  g.counters = ds->counters;
+  g.counters = ds->counters;  // (zero between launches: the kernel sees to it)
+  g.exits = ds->counters + kStaticCounters;
   g.status = ds->status;
   g.out = y;
   g.out_ld = n_out;
   g.o_real = n_out;
-  e = tss::launch_gemm(tss::kEpiStore, tw, tx, g, grid, tss::gemm_smem_bytes(n_pad, stages), s, false);
+  e = tss::launch_gemm(tss::kEpiStore, tw, tx, g, grid, tss::gemm_smem_bytes(n_pad, stages * kps), s, false);
   if (e != cudaSuccess) return reject(TSS_ERR_CUDA, std::string("launch: ") + cudaGetErrorString(e));
   return TSS_OK;
 }
