@@ -538,8 +538,8 @@ bool mk_config_for(const MkPlanIn& c, int B, int M, int tiles, MkConfig* out) {
     if (kps > c.kps_max || S > c.stages_max || base > kLimit) return false;
     const size_t ring = static_cast<size_t>(S) * kps * 16384 + SX * xps * xb;
     const size_t avail = kLimit - base;
-    // at least Q + one tile, and Q + the warps' merge buffer (8 warps x 16 rows x D floats)
-    const size_t first = q + std::max(tile, static_cast<size_t>(8) * 16 * c.D * 4);
+    // at least Q + one tile, and Q + the warps' merge buffer (8 warps x 16 rows x (D + 8) floats)
+    const size_t first = q + std::max(tile, static_cast<size_t>(8) * 16 * (c.D + 8) * 4);
     const size_t need_min = ring >= first ? 0 : first - ring;
     if (need_min > avail) return false;
     const size_t want = q + per * tile > ring ? q + per * tile - ring : 0;

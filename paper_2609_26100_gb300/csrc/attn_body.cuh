@@ -14,6 +14,12 @@ constexpr int attn_ld() {
   return D + 8;  // padded smem row (bf16 elements): conflict-free ldmatrix
 }
 
+// Row stride, in floats, of the warps' O in attn_finish_team's merge buffer.
+template <int D>
+constexpr int attn_ldo() {
+  return D + 8;
+}
+
 __host__ __device__ inline size_t attn_qlo_bytes(int head_dim) {
   return static_cast<size_t>(kNarrowNodes) * (head_dim + 8) * 2;  // lo parts of q
 }
@@ -326,49 +332,13 @@ __device__ __forceinline__ void attn_tile_step(const AttnItem<D>& it, int tile, 
   attn_blocks_step<D, QK16, PLO, QLO, WIDE>(it, kp, vp, key0, it.kpw / 16, scale_log2, a);
 }
 
-// Weighted sum over the splits of every output element of a (request, head): each thread takes
-// kU elements per round with the partial outputs of all (<= kS) splits loaded together; the first
-// round's loads are issued before `weights()` (which computes wgt) so that they overlap.
-template <int D, int NT, int kU, int kS, typename Weights, typename Put, int NB = kNarrowNodes>
-__device__ __forceinline__ void attn_merge_rounds(const AttnParams& p, size_t ph, int N, int ns, int tid,
-                                                  const float* wgt, Weights weights, Put put) {
-  float po[kU][kS];
-  auto load = [&](int idx0) {
-#pragma unroll
-    for (int u = 0; u < kU; ++u) {
-      const int idx = idx0 + u * NT;
-      const int i = idx / D, dd = idx - i * D;
-#pragma unroll
-      for (int sp = 0; sp < kS; ++sp)
-        po[u][sp] = idx < N * D && sp < ns ? __ldcg(&p.part_o[((ph + sp) * NB + i) * D + dd]) : 0.f;
-    }
-  };
-  load(tid);
-  weights();
-  for (int idx0 = tid; idx0 < N * D; idx0 += kU * NT) {
-    if (idx0 != tid) load(idx0);
-#pragma unroll
-    for (int u = 0; u < kU; ++u) {
-      const int idx = idx0 + u * NT;
-      if (idx >= N * D) continue;
-      const float* w = wgt + (idx / D) * ns;
-      float o = 0.f;
-#pragma unroll
-      for (int sp = 0; sp < kS; ++sp)
-        if (sp < ns) o += w[sp] * po[u][sp];
-      put(idx, o);
-    }
-  }
-}
-
 // Merge the warps that share a query tile through shared memory (sO: [NT / 32][16][D] floats, any
 // free 16-byte-aligned buffer of NT / 4 KiB for D = 128; sM, sL: [NT / 32][16]), then write this split's result: the
 // normalised output when there is one split, else the partial, and the last split of
 // (request, head) merges all partials in split order.  Returns true on the call that wrote the
 // final output rows.  `stamp(k)` records diagnostics (k = 9, 2, 3, 4 in that order).
-// kFastMerge: the merge's loads in one round (attn_merge_rounds), used by the persistent
-// kernel; the standalone kernel keeps the plain loop, which measured faster there.
-template <int D, int BAR, int NT, bool kFastMerge, typename Stamp, int NB = kNarrowNodes>
+// Used by the separate kernel; the persistent kernel's items end in attn_finish_team.
+template <int D, int BAR, int NT, typename Stamp, int NB = kNarrowNodes>
 __device__ __forceinline__ bool attn_finish(const AttnParams& p, const AttnItem<D>& it, AttnAcc<D>& a, int split,
                                             int head, int b, int tid, float* sO, float (*sM)[16], float (*sL)[16],
                                             int* s_last, Stamp stamp) {
@@ -454,103 +424,204 @@ __device__ __forceinline__ bool attn_finish(const AttnParams& p, const AttnItem<
   named_bar_sync(BAR, NT);
   stamp(3);
   if (!*s_last) return false;  // (the counter's acquire, then the barrier: the partials are visible)
-  if (kFastMerge) {
-    // Merge weights per (row, split) -- w = 2^(m_s - M) / L with L = sum 2^(m_s - M) l_s, in split
-    // order -- and the weighted sum of the splits' O for every output element.  The (m, l) pairs go
-    // to shared memory (sO is free again) while the first elements' partial outputs are already in
-    // flight, so that the merge of a small block costs one round of loads.
-    const int ns = p.n_splits;
-    float* wgt = sO;                          // [N][ns]
-    float* sml = sO + NB * kMaxSplits;  // [N][ns] x (m, l)
-    for (int x = tid; x < N * ns; x += NT) {
-      const int i = x / ns, sp = x - i * ns;
+  // Merge weights per (row, split) first -- w = 2^(m_s - M) / L with L = sum 2^(m_s - M) l_s, in
+  // split order -- into shared memory (sO is free again), then every output element is a
+  // weighted sum of the splits' O, several elements' loads in flight per thread.
+  float* wgt = sO;  // [N][n_splits]
+  const int ns = p.n_splits;
+  for (int i = tid; i < N; i += NT) {
+    float M = -INFINITY;
+    for (int sp = 0; sp < ns; ++sp) M = fmaxf(M, __ldcg(&p.part_ml[((ph + sp) * NB + i) * 2]));
+    const float base = M == -INFINITY ? 0.f : M;
+    float L = 0.f;
+    for (int sp = 0; sp < ns; ++sp) {
       const size_t pi = (ph + sp) * NB + i;
-      sml[2 * x] = __ldcg(&p.part_ml[pi * 2]);
-      sml[2 * x + 1] = __ldcg(&p.part_ml[pi * 2 + 1]);
+      const float f = exp2f(__ldcg(&p.part_ml[pi * 2]) - base);
+      L += f * __ldcg(&p.part_ml[pi * 2 + 1]);
+      wgt[i * ns + sp] = f;
     }
-    auto weights = [&]() {
-      named_bar_sync(BAR, NT);
-      for (int i = tid; i < N; i += NT) {
-        float M = -INFINITY;
-        for (int sp = 0; sp < ns; ++sp) M = fmaxf(M, sml[2 * (i * ns + sp)]);
-        const float base = M == -INFINITY ? 0.f : M;
-        float L = 0.f;
-        for (int sp = 0; sp < ns; ++sp) {
-          const float f = exp2f(sml[2 * (i * ns + sp)] - base);
-          L += f * sml[2 * (i * ns + sp) + 1];
-          wgt[i * ns + sp] = f;
-        }
-        if (!(L > 0.f)) report(p.status, kStatusCheck);
-        const float inv = L > 0.f ? 1.f / L : 0.f;
-        for (int sp = 0; sp < ns; ++sp) wgt[i * ns + sp] *= inv;
-      }
-      named_bar_sync(BAR, NT);
-    };
-    auto put = [&](int idx, float val) {
-      const int i = idx / D, dd = idx - i * D;
-      if (p.o_xs.rows)
-        store_split(p.o, p.o_xs, crow + i, head * D + dd, val);
-      else
-        p.o[static_cast<size_t>(crow + i) * d + head * D + dd] = __float2bfloat16_rn(val);
-    };
-    if (ns <= 4)
-      attn_merge_rounds<D, NT, 8, 4, decltype(weights), decltype(put), NB>(p, ph, N, ns, tid, wgt, weights, put);
-    else if (ns <= 8)
-      attn_merge_rounds<D, NT, 4, 8, decltype(weights), decltype(put), NB>(p, ph, N, ns, tid, wgt, weights, put);
-    else
-      attn_merge_rounds<D, NT, 2, 16, decltype(weights), decltype(put), NB>(p, ph, N, ns, tid, wgt, weights, put);
-  } else {
-    // Merge weights per (row, split) first -- w = 2^(m_s - M) / L with L = sum 2^(m_s - M) l_s, in
-    // split order -- into shared memory (sO is free again), then every output element is a
-    // weighted sum of the splits' O, several elements' loads in flight per thread.
-    float* wgt = sO;  // [N][n_splits]
-    const int ns = p.n_splits;
-    for (int i = tid; i < N; i += NT) {
-      float M = -INFINITY;
-      for (int sp = 0; sp < ns; ++sp) M = fmaxf(M, __ldcg(&p.part_ml[((ph + sp) * NB + i) * 2]));
-      const float base = M == -INFINITY ? 0.f : M;
-      float L = 0.f;
-      for (int sp = 0; sp < ns; ++sp) {
-        const size_t pi = (ph + sp) * NB + i;
-        const float f = exp2f(__ldcg(&p.part_ml[pi * 2]) - base);
-        L += f * __ldcg(&p.part_ml[pi * 2 + 1]);
-        wgt[i * ns + sp] = f;
-      }
-      if (!(L > 0.f)) report(p.status, kStatusCheck);
-      const float inv = L > 0.f ? 1.f / L : 0.f;
-      for (int sp = 0; sp < ns; ++sp) wgt[i * ns + sp] *= inv;
-    }
-    named_bar_sync(BAR, NT);
-    constexpr int kU = 4;  // output elements per thread with their loads in flight together
-    for (int idx0 = tid; idx0 < N * D; idx0 += kU * NT) {
-      float O[kU];
-  #pragma unroll
-      for (int u = 0; u < kU; ++u) O[u] = 0.f;
-      for (int sp = 0; sp < ns; ++sp) {
-        float po[kU];
-  #pragma unroll
-        for (int u = 0; u < kU; ++u) {
-          const int idx = idx0 + u * NT;
-          const int i = idx / D, dd = idx - i * D;
-          po[u] = idx < N * D ? __ldcg(&p.part_o[((ph + sp) * NB + i) * D + dd]) : 0.f;
-        }
-  #pragma unroll
-        for (int u = 0; u < kU; ++u) {
-          const int idx = idx0 + u * NT;
-          if (idx < N * D) O[u] += wgt[(idx / D) * ns + sp] * po[u];
-        }
-      }
-  #pragma unroll
+    if (!(L > 0.f)) report(p.status, kStatusCheck);
+    const float inv = L > 0.f ? 1.f / L : 0.f;
+    for (int sp = 0; sp < ns; ++sp) wgt[i * ns + sp] *= inv;
+  }
+  named_bar_sync(BAR, NT);
+  constexpr int kU = 4;  // output elements per thread with their loads in flight together
+  for (int idx0 = tid; idx0 < N * D; idx0 += kU * NT) {
+    float O[kU];
+#pragma unroll
+    for (int u = 0; u < kU; ++u) O[u] = 0.f;
+    for (int sp = 0; sp < ns; ++sp) {
+      float po[kU];
+#pragma unroll
       for (int u = 0; u < kU; ++u) {
         const int idx = idx0 + u * NT;
-        if (idx >= N * D) continue;
         const int i = idx / D, dd = idx - i * D;
-        if (p.o_xs.rows)
-          store_split(p.o, p.o_xs, crow + i, head * D + dd, O[u]);
-        else
-          p.o[static_cast<size_t>(crow + i) * d + head * D + dd] = __float2bfloat16_rn(O[u]);
+        po[u] = idx < N * D ? __ldcg(&p.part_o[((ph + sp) * NB + i) * D + dd]) : 0.f;
+      }
+#pragma unroll
+      for (int u = 0; u < kU; ++u) {
+        const int idx = idx0 + u * NT;
+        if (idx < N * D) O[u] += wgt[(idx / D) * ns + sp] * po[u];
       }
     }
+#pragma unroll
+    for (int u = 0; u < kU; ++u) {
+      const int idx = idx0 + u * NT;
+      if (idx >= N * D) continue;
+      const int i = idx / D, dd = idx - i * D;
+      if (p.o_xs.rows)
+        store_split(p.o, p.o_xs, crow + i, head * D + dd, O[u]);
+      else
+        p.o[static_cast<size_t>(crow + i) * d + head * D + dd] = __float2bfloat16_rn(O[u]);
+    }
+  }
+  stamp(4);
+  return true;
+}
+
+// The same end of an item for a team of NT = 256 threads (the persistent kernel; blocks of up to 64
+// rows), which every layer of a short step waits for.  Bound by its chain of latencies: the warps'
+// O through shared memory in rows of D + 8 floats (8-byte stores of a fragment then touch every bank
+// once; rows of D had put the eight rows of a store in the same banks), the row weights by a lane per
+// (row, warp) or (row, split), the sums and stores by 16-byte vectors.  The caller's barrier has
+// freed the key tiles that sO overlays ([8][16][D + 8] floats).
+template <int D, int BAR, int NT, typename Stamp>
+__device__ __forceinline__ bool attn_finish_team(const AttnParams& p, const AttnItem<D>& it, AttnAcc<D>& a, int split,
+                                                 int head, int b, int tid, float* sO, float (*sM)[16], float (*sL)[16],
+                                                 int* s_last, Stamp stamp) {
+  constexpr int NW = NT / 32, LDO = attn_ldo<D>(), C4 = D / 4;
+  static_assert(NT == 256, "128 threads cover the (row, warp) pairs of eight warps");
+  const int H = p.n_heads, d = p.d_model;
+  const int N = it.N, crow = it.crow, mt = it.mt, warp = it.warp, g = it.g, tq = it.tq;
+  a.l0 += __shfl_xor_sync(0xffffffffu, a.l0, 1);
+  a.l0 += __shfl_xor_sync(0xffffffffu, a.l0, 2);
+  a.l1 += __shfl_xor_sync(0xffffffffu, a.l1, 1);
+  a.l1 += __shfl_xor_sync(0xffffffffu, a.l1, 2);
+  float* o0 = sO + (warp * 16 + g) * LDO + tq * 2;
+#pragma unroll
+  for (int dt = 0; dt < D / 8; ++dt) *reinterpret_cast<float2*>(o0 + dt * 8) = make_float2(a.o[dt][0], a.o[dt][1]);
+  if (N - it.wm * 16 > 8) {
+#pragma unroll
+    for (int dt = 0; dt < D / 8; ++dt)
+      *reinterpret_cast<float2*>(o0 + 8 * LDO + dt * 8) = make_float2(a.o[dt][2], a.o[dt][3]);
+  }
+  if (tq == 0) {
+    sM[warp][g] = a.m0;
+    sM[warp][g + 8] = a.m1;
+    sL[warp][g] = a.l0;
+    sL[warp][g + 8] = a.l1;
+  }
+  named_bar_sync(BAR, NT);
+  stamp(9);
+  const size_t ph = (static_cast<size_t>(b) * H + head) * p.n_splits;
+  // per query row: the warps' common max M, their weights 2^(m_w - M) (over sM) and the merged sum L
+  // (over sL of the row's first warp), a lane per warp
+  if (tid < 128) {
+    const int R = NW / mt, i = tid / R, wt = i >> 4, rr = i & 15, wi = wt + mt * (tid & (R - 1));
+    const float m = sM[wi][rr];
+    float M = m;
+    for (int o = R >> 1; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
+    const float f = exp2f(m - (M == -INFINITY ? 0.f : M));
+    float L = f * sL[wi][rr];
+    for (int o = R >> 1; o > 0; o >>= 1) L += __shfl_xor_sync(0xffffffffu, L, o);
+    sM[wi][rr] = f;
+    __syncwarp();  // (sL of the row is read by its other lanes above)
+    if ((tid & (R - 1)) == 0 && i < N) {
+      sL[wt][rr] = L;
+      if (p.n_splits == 1) {
+        if (!(L > 0.f)) report(p.status, kStatusCheck);
+      } else {
+        __stcg(reinterpret_cast<float2*>(p.part_ml) + (ph + split) * kNarrowNodes + i, make_float2(M, L));
+      }
+    }
+  }
+  named_bar_sync(BAR, NT);
+  auto put = [&](int i, int c4, float4 v) {
+    const float x[4] = {v.x, v.y, v.z, v.w};
+    if (p.o_xs.rows)
+      store_split4(split_at(p.o, p.o_xs, head * D + c4), crow + i, x);
+    else
+      *reinterpret_cast<uint2*>(p.o + static_cast<size_t>(crow + i) * d + head * D + c4) =
+          make_uint2(pack_bf16(x[0], x[1]), pack_bf16(x[2], x[3]));
+  };
+  for (int u = tid; u < N * C4; u += NT) {
+    const int i = u / C4, c4 = (u % C4) * 4, wt = i >> 4, rr = i & 15;
+    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int w = wt; w < NW; w += mt) {
+      const float f = sM[w][rr];
+      const float4 x = *reinterpret_cast<const float4*>(sO + (w * 16 + rr) * LDO + c4);
+      s.x += f * x.x;
+      s.y += f * x.y;
+      s.z += f * x.z;
+      s.w += f * x.w;
+    }
+    if (p.n_splits == 1) {
+      const float L = sL[wt][rr], inv = L > 0.f ? 1.f / L : 0.f;
+      put(i, c4, make_float4(s.x * inv, s.y * inv, s.z * inv, s.w * inv));
+    } else {
+      __stcg(reinterpret_cast<float4*>(p.part_o + ((ph + split) * kNarrowNodes + i) * D + c4), s);
+    }
+  }
+  if (p.n_splits == 1) return true;
+  stamp(2);
+  // the last CTA of (request, head) merges the splits in order
+  named_bar_sync(BAR, NT);  // every thread's partial stores precede the release below
+  if (tid == 0) {
+    int* cnt = p.counters + static_cast<size_t>(b) * H + head;
+    const int old = atom_add_acq_rel_gpu(cnt, 1);
+    *s_last = old == p.n_splits - 1;
+    if (*s_last) atomicExch(cnt, 0);
+  }
+  named_bar_sync(BAR, NT);
+  stamp(3);
+  if (!*s_last) return false;  // (the counter's acquire, then the barrier: the partials are visible)
+  const int ns = p.n_splits;
+  constexpr int kS = 4;  // splits per round of loads
+  auto load = [&](int u, int s0, float4 (&x)[kS]) {
+    const int i = u / C4, c4 = (u % C4) * 4;
+#pragma unroll
+    for (int q = 0; q < kS; ++q)
+      x[q] = u < N * C4 && s0 + q < ns
+                 ? __ldcg(reinterpret_cast<const float4*>(p.part_o + ((ph + s0 + q) * kNarrowNodes + i) * D + c4))
+                 : make_float4(0.f, 0.f, 0.f, 0.f);
+  };
+  float4 x[kS];
+  load(tid, 0, x);  // in flight while the weights are computed
+  // weights w = 2^(m_s - M) / L with L = sum 2^(m_s - M) l_s, a lane per (row, split)
+  float* wgt = sO;  // [N][ns] (sO is free again)
+  int P = 1;
+  while (P < ns) P <<= 1;
+  for (int i0 = 0; i0 < N; i0 += NT / P) {
+    const int i = i0 + tid / P, sp = tid & (P - 1);
+    float2 ml = make_float2(-INFINITY, 0.f);
+    if (i < N && sp < ns) ml = __ldcg(reinterpret_cast<const float2*>(p.part_ml) + (ph + sp) * kNarrowNodes + i);
+    float M = ml.x;
+    for (int o = P >> 1; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
+    const float f = exp2f(ml.x - (M == -INFINITY ? 0.f : M));
+    float L = f * ml.y;
+    for (int o = P >> 1; o > 0; o >>= 1) L += __shfl_xor_sync(0xffffffffu, L, o);
+    if (i < N && sp < ns) {
+      if (sp == 0 && !(L > 0.f)) report(p.status, kStatusCheck);
+      wgt[i * ns + sp] = L > 0.f ? f / L : 0.f;
+    }
+  }
+  named_bar_sync(BAR, NT);
+  for (int u = tid; u < N * C4; u += NT) {
+    const float* w = wgt + (u / C4) * ns;
+    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int s0 = 0; s0 < ns; s0 += kS) {
+      if (u != tid || s0 > 0) load(u, s0, x);
+#pragma unroll
+      for (int q = 0; q < kS; ++q)
+        if (s0 + q < ns) {
+          const float f = w[s0 + q];
+          s.x += f * x[q].x;
+          s.y += f * x[q].y;
+          s.z += f * x[q].z;
+          s.w += f * x[q].w;
+        }
+    }
+    put(u / C4, (u % C4) * 4, s);
   }
   stamp(4);
   return true;
@@ -603,7 +674,7 @@ __device__ bool attention_item(const AttnParams& p, int split, int head, int b, 
   }
   cp_async_wait<0>();
   auto no_stamp = [](int) {};
-  return attn_finish<D, BAR, NT, false, decltype(no_stamp), NB>(p, it, a, split, head, b, tid, reinterpret_cast<float*>(sK),
+  return attn_finish<D, BAR, NT, decltype(no_stamp), NB>(p, it, a, split, head, b, tid, reinterpret_cast<float*>(sK),
                                                              sM, sL, s_last, no_stamp);
 }
 
@@ -620,7 +691,7 @@ __host__ __device__ inline int attn_resident_tiles(int head_dim, size_t smem_byt
 // round trip per round instead of one per tile.  The scores are fp16 MMAs (q arrives in fp16, the
 // keys are converted in registers).  Run by a team of NT threads (tid < NT); each warp scores
 // every (NT / 32 / query tiles)-th 16-key block of a round.  Needs smem_bytes >= the Q buffer +
-// 1 tile and the NT / 4 KiB merge buffer (D = 128) to fit behind Q.  If wait_inputs() fails,
+// 1 tile and the merge buffer of attn_finish_team to fit behind Q.  If wait_inputs() fails,
 // drains its copies and returns false without output.
 template <int D, int BAR, int NT, typename Wait>
 __device__ bool attention_item_resident(const AttnParams& p, int split, int head, int b, int tid, uint8_t* smem,
@@ -736,7 +807,7 @@ __device__ bool attention_item_resident(const AttnParams& p, int split, int head
   }
   stamp(1);
   if (trace && it.lane == 0 && it.warp < 4) trace[5 + it.warp] = globaltimer_ns();
-  return attn_finish<D, BAR, NT, true>(p, it, a, split, head, b, tid, reinterpret_cast<float*>(sKV), sM, sL, s_last, stamp);
+  return attn_finish_team<D, BAR, NT>(p, it, a, split, head, b, tid, reinterpret_cast<float*>(sKV), sM, sL, s_last, stamp);
 }
 
 }  // namespace tss

@@ -371,33 +371,6 @@ __device__ bool mk_prepare_rs(const MkParams& p, const MkEpi& e, unsigned long l
   return true;
 }
 
-// Stores of 4 consecutive features (k % 4 == 0) into the split hi/lo layout: they are adjacent in
-// the swizzled 64-element rows, so each part is one 8-byte store.  The part of the address that does
-// not depend on the row is kept per lane, and the lo part lies at a constant distance (half is a
-// multiple of 8, so both parts' rows are swizzled alike).
-struct SplitAt {
-  __nv_bfloat16* base;  // of feature k's k-block, plus k & 7
-  uint32_t c8, lo;      // 16-byte chunk within the 64-element row; elements from a hi to its lo part
-};
-__device__ __forceinline__ SplitAt split_at(__nv_bfloat16* buf, const XsLayout& L, int k) {
-  const uint32_t kb = static_cast<uint32_t>(k) >> 6, kc = static_cast<uint32_t>(k) & 63u;
-  return SplitAt{buf + kb * static_cast<uint32_t>(L.parts * L.rows * 64) + (kc & 7u), kc >> 3,
-                 static_cast<uint32_t>(L.parts == 1 ? L.half : L.rows) * 64u};
-}
-__device__ __forceinline__ void store_split4(const SplitAt& s, int j, const float* x) {
-  uint32_t hi[2], lo[2];
-#pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    hi[i] = pack_bf16(x[2 * i], x[2 * i + 1]);
-    const float h0 = __uint_as_float(hi[i] << 16), h1 = __uint_as_float(hi[i] & 0xffff0000u);
-    lo[i] = pack_bf16(x[2 * i] - h0, x[2 * i + 1] - h1);
-  }
-  const uint32_t row = static_cast<uint32_t>(j);
-  __nv_bfloat16* d = s.base + row * 64u + ((s.c8 ^ (row & 7u)) << 3);
-  *reinterpret_cast<uint2*>(d) = make_uint2(hi[0], hi[1]);
-  *reinterpret_cast<uint2*>(d + s.lo) = make_uint2(lo[0], lo[1]);
-}
-
 // Sums of G values per lane over the warp's 32 lanes, G a power of two: the values are halved
 // between lane pairs first (G - 1 shuffles), then one value each remains to be summed.  Lane l ends
 // with the sum of value l & (G - 1).
