@@ -231,7 +231,8 @@ tss_status tss_persistent_plan(const tss_arch* arch, int n_req, int n_rows, int 
  * not overlap on different streams (they share workspaces).
  * Default path: three launches -- a prologue (controller, embedding), one persistent cooperative
  * kernel for every active layer and the LM head, and a finish kernel (acceptance, compaction).
- * When a step's context KV outweighs half a layer's weights (long contexts), the persistent kernel
+ * When a step's context KV outweighs half a layer's weights (long contexts), its (request, head)
+ * pairs outnumber the SMs or a tree block meets many keys, the persistent kernel
  * is launched once per span of GEMM phases between two attentions and each layer's attention
  * runs as its own kernel (2 + 2 x active layers + 1 launches).
  * A step that does not fit the persistent kernel's shared-memory plan (tss_persistent_plan) is
@@ -244,11 +245,12 @@ tss_status tss_verify(tss_ctx* ctx, const tss_verify_batch* batch, const tss_kv_
 
 /* The attention kernel of the last step enqueued on ctx (tss_verify, tss_verify_grouped's last
  * group, tss_verify_profiled):
- *   0  the separate split-KV attention kernel (warp-level MMA; blocks of up to 64 rows),
+ *   0  the separate split-KV attention kernel for blocks of up to 64 rows (head_dim 128 on the
+ *      persistent path: tcgen05, the rows on the MMA's 128-row side; else warp-level MMA),
  *   1  the tcgen05 attention kernel: blocks of at most 16 rows and head_dim 128, the keys on the
  *      MMA's 128-row side, K/V tiles by TMA, scores and outputs in tensor memory (the default for
  *      such steps; the environment variable TSS_ATTN_TC=0 at tss_create turns it off),
- *   2  the separate kernel's variant for blocks of more than 64 rows,
+ *   2  the same for blocks of more than 64 rows,
  *   3  the attention inside the persistent verify kernel;
  * -1 before the first step or for a NULL ctx.  Host state only: no CUDA call. */
 int tss_attention_kernel(const tss_ctx* ctx);

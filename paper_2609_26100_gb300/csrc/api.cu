@@ -134,7 +134,7 @@ struct tss_ctx {
   // tcgen05 attention of blocks of at most 16 rows (head_dim 128; TSS_ATTN_TC=0 turns it off)
   int attn_tc = 1;
   int last_attn = -1;                    // attention kernel of the last step (tss_attention_kernel)
-  CUtensorMap* d_kvmaps = nullptr;       // [L] each layer's KV cache as a 2-D tensor
+  CUtensorMap* d_kvmaps = nullptr;       // [2][L] each layer's KV cache as a 2-D tensor, boxes of 128 and of 64 rows
   std::vector<CUtensorMap> h_kvmaps;     // host copy of the last maps uploaded
   std::vector<const void*> kvmap_ptr;    // the layer pointers they were made for
   int kvmap_slots = -1, kvmap_cap = -1;  // ... and the cache shape
@@ -292,6 +292,7 @@ tss_status run_gemm(tss_ctx* c, int epi, const CUtensorMap& tmW, const CUtensorM
 
 struct StepPlan {
   int B, M, n_act, mode, splits, n_pad;
+  int rows_splits;    // key splits of attn_rows_kernel
   int max_nodes;      // rows of the largest request's block
   int tiles;          // 64-key tiles of the longest request (context + block)
   long long ctx_sum;  // context tokens over the batch
@@ -304,6 +305,12 @@ int attn_variant(const tss_ctx* c, const StepPlan& sp) {
   if (sp.max_nodes > kNarrowNodes) return 2;
   if (c->attn_tc && c->D == 128 && sp.max_nodes <= kTcMaxNodes && c->kvmap_ok) return 1;
   return 0;
+}
+
+// Whether a separate attention launch of the persistent path runs on attn_rows_kernel: blocks of more
+// than kTcMaxNodes rows (attn_variant 0 or 2 otherwise the warp-level kernel).
+bool attn_rows(const tss_ctx* c, const StepPlan& sp) {
+  return c->attn_tc && c->D == 128 && sp.max_nodes > kTcMaxNodes && c->kvmap_ok;
 }
 
 AttnTcParams tc_params(const tss_ctx* c, float scale_log2) {
@@ -340,10 +347,12 @@ tss_status sync_kv_maps(tss_ctx* c, const tss_kv_cache* kv, cudaStream_t s) {
   if (rows == 0 || rows + kTcMaxKeyTile > 0x7fffffffull) return TSS_OK;  // (row coordinates are 32-bit)
   for (int l = 0; l < c->L; ++l) {
     std::memset(&c->h_kvmaps[l], 0, sizeof(CUtensorMap));
-    if (kv->layer[l] && !make_tmap(&c->h_kvmaps[l], kv->layer[l], 128, rows, 1, 128, 2))
+    std::memset(&c->h_kvmaps[c->L + l], 0, sizeof(CUtensorMap));
+    if (kv->layer[l] && (!make_tmap(&c->h_kvmaps[l], kv->layer[l], 128, rows, 1, 128, 2) ||
+                         !make_tmap(&c->h_kvmaps[c->L + l], kv->layer[l], 128, rows, 1, 64, 2)))
       return fail(TSS_ERR_CUDA, "cuTensorMapEncodeTiled failed for a KV cache layer");
   }
-  TSS_CU(cudaMemcpyAsync(c->d_kvmaps, c->h_kvmaps.data(), sizeof(CUtensorMap) * c->L, cudaMemcpyHostToDevice, s));
+  TSS_CU(cudaMemcpyAsync(c->d_kvmaps, c->h_kvmaps.data(), sizeof(CUtensorMap) * 2 * c->L, cudaMemcpyHostToDevice, s));
   c->kvmap_ok = true;
   return TSS_OK;
 }
@@ -524,6 +533,30 @@ int ext_attn_splits(const tss_ctx* c, const StepDesc* sd, int B) {
   return best;
 }
 
+// Key splits per (request, head) for attn_rows_kernel (one CTA per SM): an item costs about six tiles
+// beside its own (Q, output), a merge about four more; the launch takes the longest item where all
+// items run at once, else about the mean load of an SM plus half an item.  The fewest splits on ties.
+int rows_splits(const tss_ctx* c, const StepDesc* sd, int B) {
+  constexpr long long kItem = 6, kMerge = 4;
+  int best = 1;
+  long long best_cost = -1;
+  for (int sl = 1; sl <= c->max_splits; ++sl) {
+    long long work = 0, longest = 0, items = 0;
+    for (int b = 0; b < B; ++b) {
+      const long long t = (sd->req_ctx[b] + sd->req_nodes[b] + 63) / 64, per = (t + sl - 1) / sl, n = (t + per - 1) / per;
+      items += c->H * n;
+      work += c->H * (t + n * kItem + (n > 1 ? kMerge : 0));
+      longest = std::max(longest, per + kItem + (n > 1 ? kMerge : 0));
+    }
+    const long long cost = items <= c->num_sms ? longest : std::max(longest, work / c->num_sms + longest / 2);
+    if (best_cost < 0 || cost < best_cost) {
+      best_cost = cost;
+      best = sl;
+    }
+  }
+  return best;
+}
+
 // B requests with M rows in all, the longest one spanning `tiles` 64-key tiles.
 bool mk_config_for(const MkPlanIn& c, int B, int M, int tiles, MkConfig* out) {
   constexpr size_t kLimit = 232448;  // per-block shared-memory maximum of sm_103 (227 KiB)
@@ -662,8 +695,13 @@ tss_status enqueue_step_mk(tss_ctx* c, const StepPlan& sp, cudaStream_t s, Prof*
   // Also when the (request, head) items outnumber the CTAs: inside the persistent kernel they
   // would run in more than one wave, one CTA per SM (13B, 4 requests x 40 heads, contexts ~2000:
   // 7.6 ms with separate kernels vs 11.2 ms inside).
+  // And when a block of more than 16 rows meets many keys (head_dim 128): the attention inside scores
+  // with mma.sync, in time with key tiles x 16-row query tiles, the separate kernel on tcgen05.  4 layers of
+  // 7B, us a step inside / separate: 60 drafts at 1000, 2048, 4000 tokens 639 / 655, 713 / 688, 814 / 760;
+  // 30 drafts at 1000, 2048, 4000 535 / 571, 591 / 602, 667 / 664.
+  const bool long_block = attn_rows(c, sp) && sp.tiles * (sp.max_nodes > 32 ? 4 : 2) >= 96;
   const bool ext = sp.max_nodes > kNarrowNodes || c->attn_mode == 2 ||
-                   (c->attn_mode == 0 && (kv_bytes >= 0.5 * layer_bytes || sp.B * c->H > c->num_sms));
+                   (c->attn_mode == 0 && (kv_bytes >= 0.5 * layer_bytes || sp.B * c->H > c->num_sms || long_block));
   p.attn_external = ext ? 1 : 0;
   c->last_attn = ext ? attn_variant(c, sp) : 3;
   TSS_MK(0, TSS_CU(launch_prologue(mp, c->ssp, c->mk_zero, c->mk_n_zero, sp.M, s, false)));
@@ -691,6 +729,23 @@ tss_status enqueue_step_mk(tss_ctx* c, const StepPlan& sp, cudaStream_t s, Prof*
     const bool tc = attn_variant(c, sp) == 1;
     AttnTcParams tp = tc_params(c, p.scale_log2);
     tp.o_xs = xs;
+    const bool rows = attn_rows(c, sp);
+    AttnRowsParams rp{};
+    rp.n_heads = c->H;
+    rp.d_model = c->d;
+    rp.n_splits = sp.rows_splits;
+    rp.nb = c->a.max_nodes > kNarrowNodes ? kMaxNodes : kNarrowNodes;
+    rp.scale_log2 = p.scale_log2;
+    rp.plan = c->d_plan;
+    rp.step = c->d_step;
+    rp.kv_maps = c->d_kvmaps ? c->d_kvmaps + c->L : nullptr;
+    rp.q = c->qbuf;
+    rp.o = c->obuf;
+    rp.o_xs = xs;
+    rp.part_o = c->attn_po;
+    rp.part_ml = c->attn_pml;
+    rp.counters = c->attn_cnt;
+    rp.status = c->d_status;
     // fault injection: with the tcgen05 attention the first attention launch withholds the signal
     // (the persistent launches then withhold nothing)
     const int inject_attn = tc ? p.withhold_flag : 0;
@@ -704,6 +759,9 @@ tss_status enqueue_step_mk(tss_ctx* c, const StepPlan& sp, cudaStream_t s, Prof*
         tp.slot = j;
         tp.withhold = j == 0 ? inject_attn : 0;
         TSS_MK(2, TSS_CU(launch_attention_tc(tp, c->num_sms, s, prof == nullptr)));
+      } else if (rows) {
+        rp.slot = j;
+        TSS_MK(2, TSS_CU(launch_attention_rows(rp, sp.B, s, prof == nullptr)));
       } else {
         ap.slot = j;
         TSS_MK(2, TSS_CU(launch_attention(ap, sp.B, s, false)));
@@ -842,8 +900,8 @@ tss_status build_workspaces(tss_ctx* c) {
   TSS_TRY(c->alloc(&c->attn_po, ph * c->D));
   TSS_TRY(c->alloc(&c->attn_pml, ph * 2));
   if (c->D == 128 && c->attn_tc) {
-    TSS_TRY(c->alloc(&c->d_kvmaps, c->L));
-    c->h_kvmaps.assign(c->L, CUtensorMap{});
+    TSS_TRY(c->alloc(&c->d_kvmaps, 2 * c->L));
+    c->h_kvmaps.assign(2 * c->L, CUtensorMap{});
     c->kvmap_ptr.assign(c->L, nullptr);
     const size_t tr = attn_tc_partial_rows(c->a.max_batch, c->H, c->num_sms);
     TSS_TRY(c->alloc(&c->tc_po, tr * 128));
@@ -887,6 +945,7 @@ tss_status build_workspaces(tss_ctx* c) {
   TSS_CU(gemm_prepare(max_smem));
   TSS_CU(attn_prepare());
   TSS_CU(attn_tc_prepare());
+  TSS_CU(attn_rows_prepare());
   TSS_CU(pf_prepare());
   TSS_CU(mk_prepare());
   {
@@ -1032,6 +1091,7 @@ tss_status prepare_step(const tss_ctx* c, const tss_verify_batch* bt, const tss_
   sp->n_act = n_act;
   sp->mode = bt->mode;
   sp->splits = splits;
+  sp->rows_splits = c->attn_splits_force > 0 ? splits : rows_splits(c, sd, B);
   sp->n_pad = pad_to(M, 16);
   sp->max_nodes = 1;
   for (int b = 0; b < B; ++b) sp->max_nodes = std::max(sp->max_nodes, bt->n_nodes[b]);

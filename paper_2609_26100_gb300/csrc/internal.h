@@ -143,6 +143,26 @@ cudaError_t launch_pf_gemm(int epi, const CUtensorMap& xh, const CUtensorMap& xl
 cudaError_t launch_pf_attn(const CUtensorMap& qh, const CUtensorMap& ql, const CUtensorMap& kv, const PfParams& p,
                            cudaStream_t s);
 
+// The tcgen05 attention for blocks of 17 to 128 rows and head_dim 128 (attn_rows.cu): a CTA per
+// (split, head, request).
+struct AttnRowsParams {
+  int slot, n_heads, d_model, n_splits;
+  int nb;                        // rows that the partials are strided by (64 or 128)
+  float scale_log2;              // log2(e) / sqrt(head_dim)
+  const PlanDev* plan;
+  const StepDesc* step;
+  const CUtensorMap* kv_maps;    // [n_layers] as AttnTcParams' but boxes of 64 rows
+  const __nv_bfloat16* q;        // [kMaxRows][d_model] compacted rows (fp16 bits)
+  __nv_bfloat16* o;              // the split tiled operand o_xs
+  XsLayout o_xs;
+  float* part_o;                 // [B][H][n_splits][nb][128]
+  float* part_ml;                // [B][H][n_splits][nb][2]
+  int* counters;                 // [B][H], self-resetting
+  int* status;
+};
+cudaError_t attn_rows_prepare();
+cudaError_t launch_attention_rows(const AttnRowsParams& p, int B, cudaStream_t s, bool pdl);
+
 size_t attn_tc_smem_bytes();
 size_t attn_tc_partial_rows(int max_batch, int n_heads, int grid);
 cudaError_t attn_tc_prepare();
