@@ -153,10 +153,11 @@ KERNEL_SOURCES = {
     "verify_persistent": ("verify_mk.cu", "attn_body.cuh", "common.cuh", "internal.h"),
     "attention": ("attention.cu", "attn_body.cuh", "common.cuh", "internal.h"),
     "attention_tc": ("attn_tc.cu", "common.cuh", "internal.h"),
+    "attention_rows": ("attn_rows.cu", "common.cuh", "internal.h"),
 }
 
 # tss_attention_kernel -> the KERNEL_SOURCES entry of the separate attention kernel that ran
-ATTENTION_IMPL = {0: "attention", 1: "attention_tc", 2: "attention"}
+ATTENTION_IMPL = {0: "attention_rows", 1: "attention_tc", 2: "attention_rows"}
 
 
 def kernel_sources_hash(kernel="verify_persistent"):

@@ -81,7 +81,10 @@ __device__ __forceinline__ bool attn_item_setup(const AttnParams& p, int split, 
   it.Vg = it.Kg + static_cast<size_t>(H) * cap * D;
   it.warp = tid >> 5;
   it.lane = tid & 31;
-  it.mt = it.N <= 16 ? 1 : (it.N <= 32 ? 2 : (NB > kNarrowNodes && it.N > kNarrowNodes ? 8 : 4));  // 16-row query tiles
+  // 16-row query tiles (in the wide variant at least two: its eight warps cut a 64-key tile into
+  // 16-key blocks, so that at most four of them share a query tile)
+  constexpr bool kWide = NB > kNarrowNodes;
+  it.mt = it.N <= (kWide ? 0 : 16) ? 1 : (it.N <= 32 ? 2 : (kWide && it.N > kNarrowNodes ? 8 : 4));
   it.ksplit = NT / 32 / it.mt;  // warps sharing one query tile
   it.wm = it.warp % it.mt;
   it.wk = it.warp / it.mt;

@@ -1,6 +1,6 @@
 """GPU parity of the speculative-sampling acceptance over block sizes: the rows' statistics are
 computed by one block each and the walk by the block that finishes a request's last row, for blocks
-of one to 64 rows, rejected at the first, a middle and no draft, alone and as
+of one to 128 rows, also very different ones in one step, rejected at the first, a middle and no draft, alone and as
 a group of a split batch (results and inputs at the caller's places)."""
 import numpy as np
 import pytest
@@ -17,15 +17,15 @@ ARCH = synth.TINY
 SEED = synth.DEFAULT_SEED
 
 
+@pytest.mark.parametrize("sizes", [[1, 64, 2, 33], [1, 128, 2, 16]])
 @pytest.mark.parametrize("grouped", [False, True])
 @pytest.mark.parametrize("stop", ["first", "middle", "none"])
-def test_sampling_block_sizes(grouped, stop):
+def test_sampling_block_sizes(grouped, stop, sizes):
     from paper_2609_26100_gb300 import build
     from paper_2609_26100_gb300.runner import TssRunner
     build.build()
     w = synth.make_weights(ARCH)
     wo = oracle_weights(w)
-    sizes = [1, 64, 2, 33]
     run = TssRunner(ARCH, to_device_weights(w), n_slots=4, kv_cap=256, max_batch=4, max_nodes=128)
     phi = {0: 0b0010, 1: 0}
     run.set_phi(phi)
