@@ -12,49 +12,71 @@ namespace tss {
 // layers that at least one request runs (the only layers that get launches) and, per layer, the
 // compacted list of rows of the requests that run it.
 // ------------------------------------------------------------------------------------------
+// A warp builds a slot's lists: lanes over the requests for their first compacted rows (a scan of
+// the running requests' row counts), then over the rows.
 __device__ void controller_body(const MiscParams& p) {
   const StepDesc* st = p.step;
   PlanDev* pl = p.plan;
   __shared__ unsigned long long smask[kMaxBatch];
+  __shared__ int snodes[kMaxBatch], soff[kMaxBatch];
   __shared__ int sact[kMaxLayers];
-  __shared__ int s_n;
+  __shared__ unsigned long long s_all;  // layers that every request skips
   const int B = st->B, L = p.n_layers;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
   for (int b = threadIdx.x; b < B; b += blockDim.x) {
     const unsigned long long m = st->req_phi[b];
     smask[b] = m;
+    snodes[b] = st->req_nodes[b];
+    soff[b] = st->req_rowoff[b];
     pl->req_mask[b] = m;
   }
   __syncthreads();
+  if (warp == 0) {
+    unsigned long long all = ~0ull;
+    for (int b = lane; b < B; b += 32) all &= smask[b];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) all &= __shfl_xor_sync(0xffffffffu, all, o);
+    if (lane == 0) s_all = all;
+  }
+  __syncthreads();
+  const unsigned long long runs = ~s_all & (L == 64 ? ~0ull : (1ull << L) - 1);
+  const int n = __popcll(runs);
+  if (threadIdx.x < L && ((runs >> threadIdx.x) & 1ull)) {
+    const int j = __popcll(runs & ((1ull << threadIdx.x) - 1));
+    sact[j] = threadIdx.x;
+    pl->act_layer[j] = threadIdx.x;
+  }
   if (threadIdx.x == 0) {
-    int n = 0;
-    for (int l = 0; l < L; ++l) {
-      bool any = false;
-      for (int b = 0; b < B; ++b) any = any || !((smask[b] >> l) & 1ull);
-      if (any) sact[n++] = l;
-    }
-    s_n = n;
     pl->n_act = n;
-    for (int j = 0; j < n; ++j) pl->act_layer[j] = sact[j];
     if (n != st->n_act_host) report(p.status, kStatusCheck);
   }
   __syncthreads();
-  for (int j = threadIdx.x; j <= s_n; j += blockDim.x) {
-    const bool final_slot = j == s_n;
-    const int slot = final_slot ? kFinalSlot : j;
-    const int l = final_slot ? -1 : sact[j];
-    int crow = 0;
-    for (int b = 0; b < B; ++b) {
-      const bool runs = final_slot || !((smask[b] >> l) & 1ull);
-      if (runs) {
-        pl->slot_crow[slot][b] = crow;
-        const int n = st->req_nodes[b], r0 = st->req_rowoff[b];
-        for (int i = 0; i < n; ++i) pl->slot_rows[slot][crow + i] = r0 + i;
-        crow += n;
-      } else {
-        pl->slot_crow[slot][b] = -1;
+  for (int j = warp; j <= n; j += nw) {
+    const int slot = j == n ? kFinalSlot : j, l = j == n ? 0 : sact[j];
+    int base = 0;
+    for (int b0 = 0; b0 < B; b0 += 32) {
+      const int b = b0 + lane;
+      const bool run = b < B && (j == n || !((smask[b] >> l) & 1ull));
+      const int c = run ? snodes[b] : 0;
+      int incl = c;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
       }
+      const int first = base + incl - c;
+      if (b < B) pl->slot_crow[slot][b] = run ? first : -1;
+      // the rows of each running request, by the whole warp
+      unsigned todo = __ballot_sync(0xffffffffu, run);
+      while (todo) {
+        const int k = __ffs(todo) - 1;
+        todo &= todo - 1;
+        const int f = __shfl_sync(0xffffffffu, first, k), cnt = __shfl_sync(0xffffffffu, c, k), r0 = soff[b0 + k];
+        for (int i = lane; i < cnt; i += 32) pl->slot_rows[slot][f + i] = r0 + i;
+      }
+      base += __shfl_sync(0xffffffffu, incl, 31);
     }
-    pl->slot_M[slot] = crow;
+    if (lane == 0) pl->slot_M[slot] = base;
   }
 }
 
@@ -200,24 +222,27 @@ __device__ int accept_greedy_body(const MiscParams& p, int b, int* path) {
     am[threadIdx.x] = ix;
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
+  if (threadIdx.x < 32) {  // one warp walks, its lanes over the nodes of each level's search
+    const int lane = threadIdx.x;
     int cur = 0, a = 0;
-    path[0] = 0;
+    if (lane == 0) path[0] = 0;
     while (true) {
       const int want = am[cur];
       int nxt = -1;
-      for (int c = cur + 1; c < N; ++c) {
-        if (s_par[c] == cur && s_tok[c] == want) {
-          nxt = c;
-          break;
-        }
+      for (int c0 = cur + 1; c0 < N && nxt < 0; c0 += 32) {
+        const int c = c0 + lane;
+        const unsigned hit = __ballot_sync(0xffffffffu, c < N && s_par[c] == cur && s_tok[c] == want);
+        if (hit) nxt = c0 + __ffs(hit) - 1;
       }
       if (nxt < 0) break;
       cur = nxt;
-      path[++a] = cur;
+      ++a;
+      if (lane == 0) path[a] = cur;
     }
-    s_a = a;
-    s_bonus = am[cur];
+    if (lane == 0) {
+      s_a = a;
+      s_bonus = am[cur];
+    }
   }
   __syncthreads();
   const int a = s_a;
@@ -551,7 +576,6 @@ __global__ void __launch_bounds__(256) prologue_kernel(const MiscParams p, float
     if (threadIdx.x == 0) report(p.status, kStatusCheck);
     tok = 0;
   }
-  __shared__ float red[16];
   __shared__ unsigned long long smask[kMaxBatch];
   __shared__ int s_l0, s_crow;
   // The first norm phase is the QKV of the union's first layer (or the LM head when every layer
@@ -580,44 +604,60 @@ __global__ void __launch_bounds__(256) prologue_kernel(const MiscParams p, float
   }
   __syncthreads();
   const float* gain = s_l0 >= 0 ? p.g_attn + static_cast<size_t>(s_l0) * p.d_model : p.g_final;
-  const int xrow = s_crow;
-  const __nv_bfloat16* e = p.embed + static_cast<size_t>(tok) * p.d_model;
-  float* h = p.h + static_cast<size_t>(m) * p.d_model;
-  const int half = threadIdx.x >> 7, r = threadIdx.x & 127;
-  const int n_t = p.d_model / 128;
-  // every load of the row first (one memory round trip), then the per-tile work
-  constexpr int kPer = 32;  // 128-feature tiles per thread half: d_model <= 8192
-  float xe[kPer], xg[kPer];
+  const int xrow = s_crow, d = p.d_model;
+  const __nv_bfloat16* e = p.embed + static_cast<size_t>(tok) * d;
+  float* h = p.h + static_cast<size_t>(m) * d;
+  // 8 consecutive features per thread and turn, every load of the row first (one round trip); 16 lanes
+  // hold a 128-feature tile.  (One feature per thread with a barrier per tile pair took 6 us of a
+  // 4096-wide row: the instructions of its address arithmetic and stores.)
+  constexpr int kPer = 4;  // d_model <= 8192 = 256 threads x 8 x kPer
+  uint4 xe[kPer];
+  float4 xg[kPer][2];
 #pragma unroll
   for (int q = 0; q < kPer; ++q) {
-    const int t = 2 * q + half;
-    xe[q] = t < n_t ? __bfloat162float(e[t * 128 + r]) : 0.f;
-    xg[q] = t < n_t && xrow >= 0 ? gain[t * 128 + r] : 0.f;
+    const int c = (q * 256 + static_cast<int>(threadIdx.x)) * 8;
+    xe[q] = make_uint4(0, 0, 0, 0);
+    xg[q][0] = xg[q][1] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (c < d) {
+      xe[q] = *reinterpret_cast<const uint4*>(e + c);
+      if (xrow >= 0) {
+        xg[q][0] = *reinterpret_cast<const float4*>(gain + c);
+        xg[q][1] = *reinterpret_cast<const float4*>(gain + c + 4);
+      }
+    }
   }
 #pragma unroll
   for (int q = 0; q < kPer; ++q) {
-    if (2 * q >= n_t) break;
-    const int t = 2 * q + half;
-    float sq = 0.f;
-    if (t < n_t) {
-      const float x = xe[q];
-      h[t * 128 + r] = x;
-      if (xrow >= 0) {
-        const float xv = x * xg[q];
-        if (p.xs.rows)
-          store_split(p.xn, p.xs, xrow, t * 128 + r, xv);
-        else
-          p.xn[static_cast<size_t>(xrow) * p.d_model + t * 128 + r] = __float2bfloat16_rn(xv);
-      }
-      sq = x * x;
-    }
+    if (q * 2048 >= d) break;  // (uniform)
+    const int c = (q * 256 + static_cast<int>(threadIdx.x)) * 8;
+    const uint32_t w[4] = {xe[q].x, xe[q].y, xe[q].z, xe[q].w};
+    float x[8];
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, off);
-    if ((threadIdx.x & 31) == 0) red[(q & 1) * 8 + (threadIdx.x >> 5)] = sq;
-    __syncthreads();  // red is double-buffered by q parity, so one barrier per tile pair
-    if (r == 0 && t < n_t)
-      ssp[static_cast<size_t>(t) * kMaxRows + m] = (red[(q & 1) * 8 + half * 4] + red[(q & 1) * 8 + half * 4 + 1]) +
-                                                   (red[(q & 1) * 8 + half * 4 + 2] + red[(q & 1) * 8 + half * 4 + 3]);
+    for (int i = 0; i < 4; ++i) {
+      x[2 * i] = __uint_as_float(w[i] << 16);
+      x[2 * i + 1] = __uint_as_float(w[i] & 0xffff0000u);
+    }
+    float sq = 0.f;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) sq += x[i] * x[i];
+#pragma unroll
+    for (int off = 8; off > 0; off >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, off);
+    if (c < d) {
+      *reinterpret_cast<float4*>(h + c) = make_float4(x[0], x[1], x[2], x[3]);
+      *reinterpret_cast<float4*>(h + c + 4) = make_float4(x[4], x[5], x[6], x[7]);
+      if (xrow >= 0) {
+        const float y[8] = {x[0] * xg[q][0].x, x[1] * xg[q][0].y, x[2] * xg[q][0].z, x[3] * xg[q][0].w,
+                            x[4] * xg[q][1].x, x[5] * xg[q][1].y, x[6] * xg[q][1].z, x[7] * xg[q][1].w};
+        if (p.xs.rows) {
+          store_split4(split_at(p.xn, p.xs, c), xrow, y);
+          store_split4(split_at(p.xn, p.xs, c + 4), xrow, y + 4);
+        } else {
+          *reinterpret_cast<uint4*>(p.xn + static_cast<size_t>(xrow) * d + c) =
+              make_uint4(pack_bf16(y[0], y[1]), pack_bf16(y[2], y[3]), pack_bf16(y[4], y[5]), pack_bf16(y[6], y[7]));
+        }
+      }
+      if ((threadIdx.x & 15) == 0) ssp[static_cast<size_t>(c >> 7) * kMaxRows + m] = sq;
+    }
   }
 }
 
@@ -658,20 +698,25 @@ __global__ void __launch_bounds__(1024) finish_kernel(const MiscParams p) {
   for (int j = threadIdx.x; j < n_act; j += blockDim.x)
     s_base[j] = pl->slot_crow[j][b] < 0 ? nullptr : st->kv_layer[pl->act_layer[j]] + slot_off;
   __syncthreads();
-  // 16-byte units (head_dim is 64 or 128): unit e = (kind, head, 8 dims) stays with one thread
-  // across the path steps, and a later step never reads a row an earlier step wrote, so the
-  // in-order copy needs no barrier.
+  // 16-byte units (head_dim is 64 or 128): unit e = (kind, head, 8 dims) of a layer stays with one
+  // thread.  No step of the path reads a row that an earlier one wrote (path[jj] >= jj, increasing), so
+  // the loads of kMove steps go out before their stores: one round trip a layer.
   const int vec = D / 8;
-  for (int j = 0; j < n_act; ++j) {
-    __nv_bfloat16* base = s_base[j];
-    if (!base) continue;
-    for (int jj = 1; jj <= a; ++jj) {
-      const int src = path[jj];
-      if (src == jj) continue;
-      for (int e = threadIdx.x; e < 2 * H * vec; e += blockDim.x) {
-        const int kind_head = e / vec, u = e - kind_head * vec;
-        uint4* row = reinterpret_cast<uint4*>(base + static_cast<size_t>(kind_head) * cap * D);
-        row[(ctx + jj) * vec + u] = row[(ctx + src) * vec + u];
+  constexpr int kMove = 8;
+  for (int e = threadIdx.x; e < 2 * H * vec; e += blockDim.x) {
+    const int kind_head = e / vec, u = e - kind_head * vec;
+    const size_t off = static_cast<size_t>(kind_head) * cap * D;
+    for (int j = 0; j < n_act; ++j) {
+      if (!s_base[j]) continue;
+      uint4* rows = reinterpret_cast<uint4*>(s_base[j] + off) + ctx * vec + u;
+      for (int j0 = 1; j0 <= a; j0 += kMove) {
+        uint4 x[kMove];
+#pragma unroll
+        for (int k = 0; k < kMove; ++k)
+          if (j0 + k <= a) x[k] = rows[path[j0 + k] * vec];
+#pragma unroll
+        for (int k = 0; k < kMove; ++k)
+          if (j0 + k <= a) rows[(j0 + k) * vec] = x[k];
       }
     }
   }
