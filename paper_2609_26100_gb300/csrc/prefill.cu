@@ -77,6 +77,7 @@ __global__ void pf_embed_kernel(const PfParams p) {
 // (d_model <= 256 threads x 8 x kPfNormV).
 constexpr int kPfNormV = 4;
 __global__ void __launch_bounds__(256) pf_norm_kernel(const PfParams p, const float* g) {
+  griddep_wait();
   const int j = blockIdx.x;
   if (j >= p.T) return;
   const float* h = p.h + static_cast<size_t>(j) * p.d_model;
@@ -593,6 +594,7 @@ __global__ void __launch_bounds__(kPfThreads, 1) pf_attn_kernel(const __grid_con
   __shared__ uint32_t tslot;
   __shared__ int abort_s;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  griddep_wait();
   const int h = blockIdx.x;
   const int4 qi = p.qtiles[blockIdx.y];  // (first row, slot, position of the first row, rows)
   const int H = p.n_heads, D = 128;
@@ -857,8 +859,9 @@ cudaError_t launch_pf_embed(const PfParams& p, cudaStream_t s) {
   return launch_k(pf_embed_kernel, dim3(p.T), dim3(256), 0, s, false, p);
 }
 
+// (the norm and the attention start while the GEMM before them drains: a launch's set-up, about 2 us)
 cudaError_t launch_pf_norm(const PfParams& p, const float* g, cudaStream_t s) {
-  return launch_k(pf_norm_kernel, dim3(p.T), dim3(256), 0, s, false, p, g);
+  return launch_k(pf_norm_kernel, dim3(p.T), dim3(256), 0, s, true, p, g);
 }
 
 // The items that are split (see pf_gemm_kernel) and the CTAs sharing them.  Whole items only, where
@@ -912,7 +915,7 @@ cudaError_t launch_pf_gemm(int epi, const CUtensorMap& xh, const CUtensorMap& xl
 cudaError_t launch_pf_attn(const CUtensorMap& qh, const CUtensorMap& ql, const CUtensorMap& kv, const PfParams& p,
                            cudaStream_t s) {
   const dim3 gr(p.n_heads, p.n_qtiles), blk(kPfThreads);
-  return launch_k(pf_attn_kernel, gr, blk, pf_attn_smem(), s, false, qh, ql, kv, p);
+  return launch_k(pf_attn_kernel, gr, blk, pf_attn_smem(), s, true, qh, ql, kv, p);
 }
 
 }  // namespace tss
