@@ -11,9 +11,9 @@
 // GEMMs (pf_gemm_kernel): out[t][o] = sum_k X[t][k] W[o][k] with the weights on the MMA's M side
 // (128-row tiles, the pre-tiled 128-byte-swizzled images the verification kernels stream) and
 // 128 tokens on the N side; a CTA takes two weight tiles against one token tile at a time (two
-// accumulators sharing the token operand) through its whole K loop (no split); items are taken
-// weight-pair-major by a persistent grid so that the CTAs working at the same time share weight
-// tiles through L2; three groups of epilogue warps keep up with the MMAs.  X is held as two bf16
+// accumulators sharing the token operand) through its whole K loop, or through a share of it where
+// whole items would leave most of the last wave idle (pf_plan); items are taken weight-pair-major by
+// a persistent grid so that the CTAs working at the same time share weight tiles through L2; three groups of epilogue warps keep up with the MMAs.  X is held as two bf16
 // parts (hi = bf16(x), lo = bf16(x - hi)), both multiplied by the weights into one fp32
 // accumulator in tensor memory, as on the verification path.  Attention (pf_attn_kernel): one CTA
 // per (head, 128-query tile of one request), queries on the MMA's M side, 64-key tiles of the
@@ -289,6 +289,20 @@ __device__ bool pf_wait_count(const int* f, int target, volatile int* abort, int
   }
 }
 
+// Position in the GEMM's ring: slot, and the parity of its current turn, advanced without the 64-bit
+// remainder of a running stage number, which the copy and MMA threads had on each stage's path (us,
+// 3 layers: 7B, 600 tokens 1316 -> 1288; 13B, 866 tokens 2262 -> 2235; 7B, 200 tokens 741 -> 738).
+struct PfRing {
+  int s = 0;
+  uint32_t turn = 0;
+  __device__ __forceinline__ void next() {
+    if (++s == kPfStages) {
+      s = 0;
+      turn ^= 1u;
+    }
+  }
+};
+
 template <int EPI>
 __global__ void __launch_bounds__(kPgThreads, 1) pf_gemm_kernel(const __grid_constant__ CUtensorMap tm_xh,
                                                                  const __grid_constant__ CUtensorMap tm_xl,
@@ -332,7 +346,7 @@ __global__ void __launch_bounds__(kPgThreads, 1) pf_gemm_kernel(const __grid_con
     if (lane == 0) {
       prefetch_tmap(&tm_xh);
       prefetch_tmap(&tm_xl);
-      long long it = 0;
+      PfRing ring;
       uint32_t item;
       bool ok = true;
       int k0, k1;
@@ -342,9 +356,9 @@ __global__ void __launch_bounds__(kPgThreads, 1) pf_gemm_kernel(const __grid_con
         const int w = static_cast<int>(item / n_u), u = static_cast<int>(item) - w * n_u;
         const int t0 = 2 * w;
         const bool two = t0 + 1 < g.n_o;
-        for (int k = k0; k < k1; ++k, ++it) {
-          const int s = static_cast<int>(it % kPfStages);
-          if (it >= kPfStages && !mbar_wait(&empty[s], static_cast<uint32_t>((it / kPfStages) - 1) & 1u, abort, p.status)) {
+        for (int k = k0; k < k1; ++k, ring.next()) {
+          const int s = ring.s;
+          if (!mbar_wait(&empty[s], ring.turn ^ 1u, abort, p.status)) {  // (the first turn: free at once)
             ok = false;
             break;
           }
@@ -356,9 +370,10 @@ __global__ void __launch_bounds__(kPgThreads, 1) pf_gemm_kernel(const __grid_con
           tma_load_2d(st + 2 * kPfA + kPfB, &tm_xl, &full[s], k * 64, u * 128);
         }
       }
-      for (long long v = it - 1; v >= 0 && v >= it - kPfStages; --v) {
+      // every copy issued has landed before the kernel returns: the last turn of each slot
+      for (int i = 0; i < kPfStages; ++i, ring.next()) {
         const uint64_t t0 = globaltimer_ns();
-        while (!mbar_try_wait(&full[v % kPfStages], static_cast<uint32_t>(v / kPfStages) & 1u))
+        while (!mbar_try_wait(&full[ring.s], ring.turn ^ 1u))  // (a slot never used: passes at once)
           if (globaltimer_ns() - t0 > kWaitLimitNs) break;
       }
     }
@@ -366,7 +381,7 @@ __global__ void __launch_bounds__(kPgThreads, 1) pf_gemm_kernel(const __grid_con
     // ---------------- MMA issuer: per k16 step, (A0, A1) x (hi, lo) into two accumulators ----------------
     if (lane == 0) {
       const uint32_t idesc = idesc_bf16_m128(128);
-      long long it = 0;
+      PfRing ring;
       uint32_t item;
       int n = 0, k0, k1;
       // fault injection: CTA 0 issues no MMA, so its epilogue's first wait runs out
@@ -380,9 +395,9 @@ __global__ void __launch_bounds__(kPgThreads, 1) pf_gemm_kernel(const __grid_con
         if (n >= 2 && !mbar_wait(&acc_empty[buf], static_cast<uint32_t>((n >> 1) - 1) & 1u, abort, p.status)) break;
         tc_fence_after();
         const uint32_t d0 = tm + buf * 2 * kPfAccCols, d1 = d0 + kPfAccCols;
-        for (int k = k0; k < k1; ++k, ++it) {
-          const int s = static_cast<int>(it % kPfStages);
-          if (!mbar_wait(&full[s], static_cast<uint32_t>(it / kPfStages) & 1u, abort, p.status)) {
+        for (int k = k0; k < k1; ++k, ring.next()) {
+          const int s = ring.s;
+          if (!mbar_wait(&full[s], ring.turn, abort, p.status)) {
             ok = false;
             break;
           }
