@@ -270,7 +270,7 @@ int tss_attention_kernel(const tss_ctx* ctx);
  *   group_events (optional, HOST array of cudaEvent_t passed as void*, one per request, entries
  *   may be NULL): event g is recorded on `stream` when group g's results are in place, so a caller
  *   can time or wait for each group.
- * Uses the context's staging buffers: do not overlap with another call on the same context.
+ * Uses the context's workspaces: do not overlap with another call on the same context.
  * Errors: those of tss_verify (all checked for the whole batch before anything is enqueued);
  * INVALID_ARG for io_host != 0 or a uniform_stride above 512. */
 tss_status tss_verify_grouped(tss_ctx* ctx, const tss_verify_batch* batch, const tss_kv_cache* kv,
@@ -288,7 +288,7 @@ tss_status tss_verify_grouped(tss_ctx* ctx, const tss_verify_batch* batch, const
  * TSS_PREFILL=steps at tss_create selects the other path); otherwise the prompt runs in chains of
  * up to max_nodes tokens, each chain one verification step on the same kernels, whose acceptance
  * outputs are discarded.  The first call on the tcgen05 path allocates its workspaces (about
- * 0.45 GB at d_model 4096).
+ * 0.5 GB at d_model 4096).
  *   n_tokens, ctx_len, domain_id, kv_slot: HOST arrays of n_req entries (n_tokens[b] >= 0;
  *     kv_slot NULL means slot b).
  *   tokens: the requests' tokens concatenated (sum(n_tokens) int32), DEVICE memory, or HOST
@@ -311,8 +311,8 @@ tss_status tss_sync_status(tss_ctx* ctx, void* stream);
  * That step's outputs are undefined.  The context stays usable: every step starts with fresh
  * counters and a clear abort word, so the next step runs normally.  A step with no active layer
  * withholds nothing.  n_steps = 0 cancels.  When the step's attention runs in the tcgen05 kernel
- * (tss_attention_kernel = 1), the first CTA of the step's first attention launch issues no MMA
- * instead, so that kernel's waits run out (after its fixed 2 s bound) and it takes the same
+ * (tss_attention_kernel = 1), the CTA of the first tile of the step's first attention launch issues no
+ * MMA instead, so that kernel's waits run out (after its fixed 2 s bound) and it takes the same
  * abort path; the next step's prologue resets its counters.  A tss_prefill call on the tcgen05
  * path also counts as a step: the first CTA of its first GEMM launch issues no MMA (2 s bound);
  * that call's cache rows are undefined. */

@@ -131,7 +131,7 @@ struct tss_ctx {
   int attn_plo = 1;
   int attn_splits_force = 0;  // > 0: key splits of the separate attention kernel (TSS_ATTN_SPLITS)
   int mk_splits_force = 0;    // > 0: key splits of the persistent kernel's attention (TSS_MK_ATTN_SPLITS)
-  // tcgen05 attention of blocks of at most 16 rows (head_dim 128; TSS_ATTN_TC=0 turns it off)
+  // tcgen05 attention in separate launches (head_dim 128; TSS_ATTN_TC=0 turns it off)
   int attn_tc = 1;
   int last_attn = -1;                    // attention kernel of the last step (tss_attention_kernel)
   CUtensorMap* d_kvmaps = nullptr;       // [2][L] each layer's KV cache as a 2-D tensor, boxes of 128 and of 64 rows

@@ -3,11 +3,12 @@
 //
 // The step is a fixed sequence of GEMM phases -- for each layer of the union (ascending):
 // QKV, O, gate/up, down; then the LM head -- with the attention of a layer between its QKV and
-// O phases.  Each phase is split stream-K over the grid exactly as in gemm.cu.  Per CTA:
+// O phases.  Each phase is split stream-K over the grid (mk_seg: with whole tiles at the end of a
+// phase that has a tile per CTA, and throughout one of few short tiles).  Per CTA:
 //
 //   warp 0      TMA producer of weight tiles (lane 0).  It walks the whole phase sequence and
 //               never waits for activations, so the weight stream does not stop at phase
-//               boundaries (it is bounded only by the shared-memory ring).
+//               boundaries (it is bounded only by its ring in shared memory).
 //   warp 1      tcgen05.mma issuer (lane 0; accumulators in TMEM, up to 8 buffers).
 //   warp 2      B-operand producer: for every k-block it waits until the activations it needs
 //               are final (flags polled 32 at a time), then lane 0 copies the N x 64 bf16 blocks of
