@@ -1145,7 +1145,7 @@ tss_status pf_workspaces(tss_ctx* c) {
 
 // One pass: T rows (the row tables and tokens already in place) through every layer the skip set
 // keeps (Sec. "Domain-Aware Skip Controller": h_{l+1} = h_l for a skipped layer, which writes no KV).
-tss_status pf_pass(tss_ctx* c, int T, int n_qtiles, unsigned long long skip, const tss_kv_cache* kv, cudaStream_t s,
+tss_status pf_pass(tss_ctx* c, int T, int n_qtiles, int max_keys, unsigned long long skip, const tss_kv_cache* kv, cudaStream_t s,
                    bool inject) {
   PfParams p{};
   p.T = T;
@@ -1175,6 +1175,8 @@ tss_status pf_pass(tss_ctx* c, int T, int n_qtiles, unsigned long long skip, con
   p.partials = c->pf_part;
   p.counters = c->pf_cnt;
   p.n_counters = pf_counters(c->num_sms);
+  p.n_splits = pf_attn_splits(c->H * n_qtiles, max_keys, c->num_sms);
+  p.attn_counters = c->pf_cnt + 4 * c->num_sms;
   p.rope_cos = c->rope_cos;
   p.rope_sin = c->rope_sin;
   p.status = c->d_status;
@@ -1650,7 +1652,7 @@ tss_status tss_prefill(tss_ctx* c, int n_req, const int32_t* n_tokens, const int
         TSS_CU(cudaMemcpyAsync(c->pf_pos, pos.data(), sizeof(int) * T, cudaMemcpyHostToDevice, s));
         TSS_CU(cudaMemcpyAsync(c->pf_slot, slt.data(), sizeof(int) * T, cudaMemcpyHostToDevice, s));
         TSS_CU(cudaMemcpyAsync(c->pf_qt, qt.data(), sizeof(int4) * qt.size(), cudaMemcpyHostToDevice, s));
-        TSS_TRY(pf_pass(c, T, static_cast<int>(qt.size()), skip[b0], kv, s, inject));
+        TSS_TRY(pf_pass(c, T, static_cast<int>(qt.size()), qt[0].z + qt[0].w, skip[b0], kv, s, inject));
         inject = false;
       }
     }

@@ -121,9 +121,12 @@ struct PfParams {
   __nv_bfloat16* kv;               // this layer's cache [n_slots][2][H][cap][D]
   const float* rope_cos;           // [max_positions][D / 2]
   const float* rope_sin;
-  float* partials;                 // parts of split GEMM items: [CTA][2][weight tile][token][weight row]
+  float* partials;                 // parts of split GEMM items: [CTA][2][weight tile][token][weight row];
+                                   // of split attention items: O [item][split][row][dim], then (max, sum) alike
   int* counters;                   // [n_counters] arrivals per split item (zero between launches)
   int n_counters;
+  int n_splits;                    // key splits of an attention item
+  int* attn_counters;              // [query tiles x heads] arrivals of a split item (zero between launches)
   int* status;
 };
 struct PfGemm {
@@ -135,6 +138,7 @@ struct PfGemm {
 };
 size_t pf_partial_floats(int sms);
 int pf_counters(int sms);
+int pf_attn_splits(int items, int max_keys, int sms);
 cudaError_t pf_prepare();
 cudaError_t launch_pf_embed(const PfParams& p, cudaStream_t s);
 cudaError_t launch_pf_norm(const PfParams& p, const float* g, cudaStream_t s);

@@ -589,10 +589,90 @@ __device__ __forceinline__ bool pa_or(bool v) {
   return r != 0;
 }
 
+// A split item's end, by the softmax threads: this CTA's part of O (raw sums, tensor memory at tm) and
+// its rows' (max, sum) go to p.partials; the last CTA of the item to arrive adds the parts in split
+// order and writes the outputs.  wgt: [split][128] floats of shared memory.
+__device__ __noinline__ void pa_merge(const PfParams& p, float* wgt, int* s_last, uint32_t tm, int st, int qr, int q0,
+                                      int nrow, int used, float m, float l) {
+  constexpr int D = 128;
+  const int h = blockIdx.x, item = blockIdx.y * p.n_heads + h;
+  const bool valid = qr < nrow;
+  float* po = p.partials + static_cast<size_t>(item) * p.n_splits * 128 * D;
+  float2* ml = reinterpret_cast<float2*>(p.partials + static_cast<size_t>(p.n_heads) * p.n_qtiles * p.n_splits * 128 * D) +
+               static_cast<size_t>(item) * p.n_splits * 128 + qr;
+  tc_fence_after();
+  if (valid) __stcg(ml + blockIdx.z * 128, make_float2(m, l));
+#pragma unroll 2
+  for (int c = 0; c < D / 16; ++c) {
+    float o[16];
+    tmem_ld16(tm + 128 + c * 16, o);
+    if (valid) {
+      float4* d = reinterpret_cast<float4*>(po + (static_cast<size_t>(blockIdx.z) * 128 + qr) * D + c * 16);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) __stcg(d + i, make_float4(o[4 * i], o[4 * i + 1], o[4 * i + 2], o[4 * i + 3]));
+    }
+  }
+  tc_fence_before();
+  named_bar_sync(1, 128);  // every thread's part precedes the release below
+  if (st == 0) {
+    *s_last = atom_add_acq_rel_gpu(&p.attn_counters[item], 1) == used - 1;
+    if (*s_last) atomicExch(&p.attn_counters[item], 0);
+  }
+  named_bar_sync(1, 128);
+  if (!*s_last) return;  // (else: the counter's acquire, then the barrier: the other parts are visible)
+  if (valid) {
+    float M = -INFINITY, L = 0.f;
+    for (int x = 0; x < used; ++x) M = fmaxf(M, __ldcg(ml + x * 128).x);
+    const float mb = M == -INFINITY ? 0.f : M;
+    for (int x = 0; x < used; ++x) {
+      const float2 v = __ldcg(ml + x * 128);
+      const float f = exp2f(v.x - mb);
+      L += f * v.y;
+      wgt[x * 128 + qr] = f;
+    }
+    if (!(L > 0.f)) report(p.status, kStatusCheck);
+    const float inv = L > 0.f ? 1.f / L : 0.f;
+    for (int x = 0; x < used; ++x) wgt[x * 128 + qr] *= inv;
+  }
+  named_bar_sync(1, 128);
+  // units (4 columns of a row): the loads of kU units and two splits in flight together
+  constexpr int kU = 4;
+  const int n_u = nrow * (D / 4);
+  for (int u0 = st; u0 < n_u; u0 += kU * 128) {
+    float4 a[kU];
+#pragma unroll
+    for (int k = 0; k < kU; ++k) a[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 2
+    for (int x = 0; x < used; ++x) {
+      float4 v[kU];
+#pragma unroll
+      for (int k = 0; k < kU; ++k)
+        v[k] = u0 + k * 128 < n_u ? __ldcg(reinterpret_cast<const float4*>(po + static_cast<size_t>(x) * 128 * D) + u0 + k * 128)
+                                  : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int k = 0; k < kU; ++k) {
+        const float f = wgt[x * 128 + min((u0 + k * 128) / (D / 4), 127)];
+        a[k].x += f * v[k].x;
+        a[k].y += f * v[k].y;
+        a[k].z += f * v[k].z;
+        a[k].w += f * v[k].w;
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < kU; ++k) {
+      const int u = u0 + k * 128;
+      if (u < n_u) {
+        const float o[4] = {a[k].x, a[k].y, a[k].z, a[k].w};
+        pf_split_store4(p.ah, p.al, static_cast<size_t>(q0 + u / (D / 4)) * p.d_model + h * D + (u % (D / 4)) * 4, o);
+      }
+    }
+  }
+}
+
 }  // namespace
 
 // Grid (heads, query tiles of p.qtiles, which the host orders heaviest first, so that the CTAs
-// with the most keys start first); the KV map has 64-row boxes; tm_q: q hi / lo maps over
+// with the most keys start first, key splits: pf_attn_splits); the KV map has 64-row boxes; tm_q: q hi / lo maps over
 // [T_max][d].
 __global__ void __launch_bounds__(kPfThreads, 1) pf_attn_kernel(const __grid_constant__ CUtensorMap tm_qh,
                                                                 const __grid_constant__ CUtensorMap tm_ql,
@@ -607,7 +687,7 @@ __global__ void __launch_bounds__(kPfThreads, 1) pf_attn_kernel(const __grid_con
   __shared__ uint64_t qfull, kfull[kPaSlots], kempty[kPaSlots], vfull[kPaSlots], vempty[kPaSlots];
   __shared__ uint64_t s_full[2], s_free[2], p_full[2], p_free[2], o_full, drain;
   __shared__ uint32_t tslot;
-  __shared__ int abort_s;
+  __shared__ int abort_s, s_last;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   griddep_wait();
   const int h = blockIdx.x;
@@ -615,7 +695,11 @@ __global__ void __launch_bounds__(kPfThreads, 1) pf_attn_kernel(const __grid_con
   const int H = p.n_heads, D = 128;
   const int q0 = qi.x, slot = qi.y, pos_t0 = qi.z, nrow = qi.w;
   const int key_end = pos_t0 + nrow;  // keys any query of the tile may see
-  const int n = (key_end + kPaKeys - 1) / kPaKeys;
+  const int n_tiles = (key_end + kPaKeys - 1) / kPaKeys, per = (n_tiles + p.n_splits - 1) / p.n_splits;
+  const int used = (n_tiles + per - 1) / per;  // splits that hold tiles
+  const int k0 = static_cast<int>(blockIdx.z) * per * kPaKeys;  // this CTA's first key, and its key tiles
+  const int n = min(n_tiles - static_cast<int>(blockIdx.z) * per, per);
+  if (n <= 0) return;  // (the whole CTA)
   if (tid == 0) {
     mbar_init(&qfull, 1);
     for (int i = 0; i < kPaSlots; ++i) {
@@ -645,7 +729,7 @@ __global__ void __launch_bounds__(kPfThreads, 1) pf_attn_kernel(const __grid_con
   const uint32_t tm = tslot;
   volatile int* abort = &abort_s;
   const size_t cap = static_cast<size_t>(p.kv_cap);
-  const int rowK = static_cast<int>(((static_cast<size_t>(slot) * 2) * H + h) * cap);
+  const int rowK = static_cast<int>(((static_cast<size_t>(slot) * 2) * H + h) * cap) + k0;
   const int rowV = rowK + static_cast<int>(static_cast<size_t>(H) * cap);
 
   if (warp == 0) {
@@ -732,7 +816,7 @@ __global__ void __launch_bounds__(kPfThreads, 1) pf_attn_kernel(const __grid_con
     const uint32_t lanes = static_cast<uint32_t>(qg * 32) << 16;
     const int j = q0 + qr;                  // row of this query
     const bool valid = qr < nrow;
-    const int pq = pos_t0 + qr;             // its position: keys <= pq are visible
+    const int pq = pos_t0 + qr - k0;        // its position, from this CTA's first key: keys <= pq are visible
     const float scale = 1.4426950408889634f / sqrtf(static_cast<float>(D));
     float m = -INFINITY, l = 0.f;
     bool ok = true;
@@ -767,7 +851,7 @@ __global__ void __launch_bounds__(kPfThreads, 1) pf_attn_kernel(const __grid_con
         ok = mbar_wait(&p_free[(t - 1) & 1], ((t - 1) >> 1) & 1, abort, p.status);
       // in the last tile, the V rows past the keys (stale or unwritten cache rows) are zeroed
       if (ok && t == n - 1) {
-        const int s_ = t % kPaSlots, r0 = key_end - t * kPaKeys;
+        const int s_ = t % kPaSlots, r0 = key_end - k0 - t * kPaKeys;
         ok = mbar_wait(&vfull[s_], (t / kPaSlots) & 1, abort, p.status);
         if (ok && st >= r0 && st < kPaKeys) {
           uint4* v0 = reinterpret_cast<uint4*>(sv + s_ * kPaKV + st * 128);
@@ -814,7 +898,10 @@ __global__ void __launch_bounds__(kPfThreads, 1) pf_attn_kernel(const __grid_con
     }
     if (ok) {
       ok = mbar_wait(&o_full, 0, abort, p.status);
-      if (!pa_or(!ok)) {
+      const bool fail = pa_or(!ok);
+      if (!fail && used > 1) {
+        pa_merge(p, reinterpret_cast<float*>(sp), &s_last, tm + lanes, st, qr, q0, nrow, used, m, l);
+      } else if (!fail) {
         tc_fence_after();
         const float inv = l > 0.f ? 1.f / l : 0.f;
         if (valid && !(l > 0.f)) report(p.status, kStatusCheck);
@@ -899,7 +986,26 @@ int pf_plan(PfGemm* g, int T, int sms) {
 }
 
 size_t pf_partial_floats(int sms) { return static_cast<size_t>(2) * sms * 2 * 128 * 128; }
-int pf_counters(int sms) { return 4 * sms; }
+int pf_counters(int sms) { return 5 * sms; }  // (split GEMM items: up to 4 sms, split attention items: up to sms)
+
+// Key splits of an attention item: where the items leave SMs idle, the fewest key tiles in a row plus
+// what a merge costs, in halves of a key tile (about 0.8 us each).  Three layers, us, with 1 / 2 / 3 / 4
+// splits (4: or as many as fit): 7B, 100 tokens after 1400: 646 / 610 / 602 / 594; 64 after 600: 576 / 569 /
+// 567 / 563; 250 after 900: 798 / 780 (two fit); 200 after 333: 738 / 748 (not split); 107 alone: 533 / 557
+// (not split); 13B, 100 after 800: 726 / 713 / 708 (three fit).  (At most `sms` CTAs then, whose parts
+// p.partials holds four times over.)
+int pf_attn_splits(int items, int max_keys, int sms) {
+  const int n = (max_keys + kPaKeys - 1) / kPaKeys;
+  int best = 1, cost = 2 * n;
+  for (int x = 2; x <= 8 && x * items <= sms; ++x) {
+    const int y = 2 * ((n + x - 1) / x) + 6 + x;
+    if (y < cost) {
+      cost = y;
+      best = x;
+    }
+  }
+  return best;
+}
 
 template <int EPI>
 cudaError_t launch_pf_gemm_epi(const CUtensorMap& xh, const CUtensorMap& xl, const PfParams& p, PfGemm g, int sms,
@@ -929,7 +1035,7 @@ cudaError_t launch_pf_gemm(int epi, const CUtensorMap& xh, const CUtensorMap& xl
 
 cudaError_t launch_pf_attn(const CUtensorMap& qh, const CUtensorMap& ql, const CUtensorMap& kv, const PfParams& p,
                            cudaStream_t s) {
-  const dim3 gr(p.n_heads, p.n_qtiles), blk(kPfThreads);
+  const dim3 gr(p.n_heads, p.n_qtiles, p.n_splits), blk(kPfThreads);
   return launch_k(pf_attn_kernel, gr, blk, pf_attn_smem(), s, true, qh, ql, kv, p);
 }
 

@@ -47,3 +47,30 @@ def test_split_prefill_matches_oracle(weights, lengths):
                 np.testing.assert_allclose(g, ref[l][kind], atol=5e-2, rtol=3e-2, err_msg=f"request {b} layer {l}")
                 assert float(np.abs(g - ref[l][kind]).mean()) < 4e-3
     run.close()
+
+
+@pytest.mark.parametrize("context,lengths", [(900, [1]), (900, [70]), (1023, [130]), (640, [3, 128, 61]), (1921, [128])])
+def test_split_attention_matches_oracle(weights, context, lengths):
+    """Short prompts appended to a context: the keys of each (head, query tile) split between CTAs, with
+    splits that some rows of a tile do not see, and a last split of a few keys."""
+    from paper_2609_26100_gb300.runner import TssRunner
+    wo, wg = weights
+    run = TssRunner(ARCH, wg, n_slots=len(lengths), kv_cap=2080, max_batch=len(lengths))
+    prompts = [synth.uniform_ints(context + n, ARCH.vocab, SEED, f"attn.{b}").tolist() for b, n in enumerate(lengths)]
+    run.prefill([p[:context] for p in prompts], [0] * len(lengths), [0] * len(lengths))
+    got = []
+    for _ in range(2):
+        run.prefill([p[context:] for p in prompts], [context] * len(lengths), [0] * len(lengths))
+        assert run.sync_status() == native.TSS_OK
+        got.append([t.clone() for t in run.kv])
+    for l in range(ARCH.n_layers):
+        assert torch.equal(got[0][l], got[1][l])
+    for b, n in enumerate(lengths):
+        ref = O.prefill(wo, ARCH, frozenset(), prompts[b])
+        for l in range(ARCH.n_layers):
+            for kind in range(2):
+                g = got[0][l][b, kind, :, context:context + n].float().cpu().numpy()
+                r = ref[l][kind][:, context:]
+                np.testing.assert_allclose(g, r, atol=5e-2, rtol=3e-2, err_msg=f"request {b} layer {l}")
+                assert float(np.abs(g - r).mean()) < 4e-3
+    run.close()
