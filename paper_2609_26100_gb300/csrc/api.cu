@@ -595,6 +595,14 @@ bool mk_config_for(const MkPlanIn& c, int B, int M, int tiles, MkConfig* out) {
   // 553, two 587, one 761; 61 rows: 48 KiB x 2 590, 32 KiB x 3 586, one k-block 709).
   static const int kRings[][4] = {{3, 3, 3, 3}, {3, 3, 3, 2}, {3, 2, 3, 2}, {2, 3, 2, 2}, {2, 2, 2, 2}, {2, 4, 1, 2},
                                   {2, 3, 1, 2}, {2, 2, 1, 2}, {1, 3, 1, 2}, {1, 2, 1, 2}};
+  // From 113 rows on the B operand's k-block is 32 KiB or more, twice the weights' and the larger share
+  // of the copies: three stages of one k-block keep its copies going where two stages of two left gaps
+  // (us a step: 128 rows 489 -> 481 and 764 -> 755, 144 rows 1148 -> 1139, 176 rows 925 -> 912, 13B 144 rows
+  // 1135 -> 1127; with smaller blocks the fewer, larger stages win: 96 rows 629 against 681).
+  static const int kWideRings[][4] = {{2, 3, 1, 3}, {2, 2, 1, 3}};
+  if (xb >= 2 * 16384)
+    for (const auto& r : kWideRings)
+      if (take(r[0], r[1], r[2], r[3])) return true;
   for (const auto& r : kRings)
     if (take(r[0], r[1], r[2], r[3])) return true;
   return false;
