@@ -301,6 +301,23 @@ __device__ __forceinline__ void store_split4(const SplitAt& s, int j, const floa
   *reinterpret_cast<uint2*>(d + s.lo) = make_uint2(lo[0], lo[1]);
 }
 
+// SwiGLU's gate: g / (1 + exp(-g)), rounded as by IEEE division: the same bits for every fp32 g (but
+// for the sign of the zero at g = -0; all 2^32 values compared).  Markstein's division (IBM J. Res.
+// Dev. 34, 1990): a quotient by the approximate reciprocal, corrected by its exact remainder; a large
+// divisor is scaled, so that its reciprocal stays normal.  The division operator's call for special
+// operands stands in the middle of the persistent kernel's epilogues, and __fdividef is off by up to
+// 2 ulp and 0 where the divisor exceeds 2^126 (gates below -87.3).  us a step with the operator / this /
+// __fdividef: tiny decoder's chain 131 / 124 / 124, 7B chain 2667 / 2655 / 2650, 61-row tree 536 / 531 / 527.
+__device__ __forceinline__ float silu(float g) {
+  const float e = 1.f + expf(-g);
+  const float s = e > 0x1p100f ? 0x1p-32f : 1.f;
+  const float x = g * s, d = e * s;
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d));
+  const float q0 = x * r, q = fmaf(fmaf(-d, q0, x), r, q0);
+  return e < INFINITY && g < INFINITY ? q : g > 0.f ? g : g * 0.f;  // (infinities and NaN as in IEEE)
+}
+
 // ------------------------------------------------------------------------------------------
 // tcgen05: tensor memory and the 5th-generation MMA
 // ------------------------------------------------------------------------------------------

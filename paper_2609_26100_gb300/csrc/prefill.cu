@@ -215,7 +215,7 @@ struct PfRows {
         for (int k = 0; k < 4; ++k) {
           const float y = __shfl_xor_sync(0xffffffffu, upper ? v[i][k] : v[i + 1][k], 16);
           const float gt = upper ? y : v[i][k], up = upper ? v[i + 1][k] : y;
-          a[k] = __fdividef(gt, 1.f + expf(-gt)) * up;
+          a[k] = silu(gt) * up;
         }
         pf_split_store4(p.uh, p.ul, static_cast<size_t>(j0 + i + (upper ? 1 : 0)) * p.u_ld + t * 64 + (f0 & 63), a);
       }

@@ -558,7 +558,7 @@ __device__ void mk_finish_rows(const MkParams& p, const MkPhase& ph, const MkEpi
           const float xa = v[jj][i] * ra, xb = v[jj + 1][i] * rb;
           const float y = __shfl_xor_sync(0xffffffffu, upper ? xa : xb, 16);
           const float g = upper ? y : xa, u = upper ? xb : y;
-          act[i] = __fdividef(g, 1.f + expf(-g)) * u;
+          act[i] = silu(g) * u;
         }
         if (j < e.M) store_split4(xat, j, act);
       }
