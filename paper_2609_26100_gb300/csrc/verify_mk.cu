@@ -4,7 +4,7 @@
 // The step is a fixed sequence of GEMM phases -- for each layer of the union (ascending):
 // QKV, O, gate/up, down; then the LM head -- with the attention of a layer between its QKV and
 // O phases.  Each phase is split stream-K over the grid (mk_seg: with whole tiles at the end of a
-// phase that has a tile per CTA, and throughout one of few short tiles).  Per CTA:
+// phase that has a tile per CTA).  Per CTA:
 //
 //   warp 0      TMA producer of weight tiles (lane 0).  It walks the whole phase sequence and
 //               never waits for activations, so the weight stream does not stop at phase
@@ -49,7 +49,6 @@ __host__ __device__ inline int mk_acc_bufs(int n_pad) {
   return nb;
 }
 constexpr uint32_t kMkWBytes = 128 * 64 * 2;
-constexpr int kMkWholeKb = 20;  // mk_seg: extra k-blocks for which a tile is left whole
 
 enum MkKind : int { kMkQkv = 1, kMkAtt = 2, kMkO = 3, kMkGu = 4, kMkDown = 5, kMkLm = 6 };
 
@@ -238,6 +237,10 @@ __device__ __forceinline__ const __nv_bfloat16* mk_weights(const MkParams& p, co
 // and p.dp_tail is set, stream-K over its first n_tiles - G tiles followed by one whole tile per
 // CTA, so that the phase ends with whole-tile epilogues (no partial tiles, no arrival counter,
 // no reload of other CTAs' partials on its critical tail).  Residual phases keep plain stream-K.
+// So do phases of fewer tiles than CTAs, even where a whole tile per CTA is short: it saved the tiny
+// decoder's chain 10 of 134 us and four layers of 13B 4 of 955, but one accumulator then sums more
+// k-blocks than a split tile's did and loses more low bits (error of the logits against 64 bits 0.4 %
+// and 2 % larger), and as many accumulators as parts took longer than splitting (145 us).
 // (32-bit arithmetic: T x #SMs is at most 152 / 8192 of a matrix's elements, below 2^32 for any
 // matrix that fits the device; 64-bit divisions took a role about a microsecond a phase)
 struct MkSeg {
@@ -260,11 +263,6 @@ __device__ __forceinline__ MkSeg mk_seg(const MkParams& p, const MkPhase& ph, in
   }
   s.T = static_cast<uint32_t>(n_split) * ph.kb;
   s.geff = min(s.T, static_cast<uint32_t>(G));
-  // Few short tiles (small models): whole tiles when streaming one takes at most kMkWholeKb
-  // k-blocks (16 KiB, about 0.23 us each) more than a CTA's even share -- about what the partial
-  // sums' store, counter and reload cost (the tiny decoder's tiles of 4 k-blocks, split over 4
-  // CTAs: 6.5 us from MMA to flag against 3 us whole).
-  if (s.whole < 0 && n_split <= G && static_cast<uint32_t>(ph.kb) <= s.T / s.geff + kMkWholeKb) s.geff = n_split;
   if (static_cast<uint32_t>(c) >= s.geff) {
     s.it = s.it1 = 0;
   } else {

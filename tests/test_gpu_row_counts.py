@@ -1,8 +1,8 @@
 """GPU parity of the persistent kernel's epilogues over the row counts of a step, on a decoder wide
 enough that every projection's tiles are split between CTAs (3 layers, d 2048, MLP 2816) and a
 vocabulary whose rows are not a multiple of 16 bytes: the two ways a split tile is finished (last
-arriver up to 8 rows, every contributor beyond), the edges of its row groups, whole tiles of the
-tiny decoder, and batches whose requests skip different layers (rows that join or leave between
+arriver up to 8 rows, every contributor beyond), the edges of its row groups, the tiny decoder's
+tiles of a few k-blocks, and batches whose requests skip different layers (rows that join or leave between
 two layers)."""
 import numpy as np
 import pytest
