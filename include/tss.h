@@ -377,8 +377,10 @@ tss_status tss_verify_profiled(tss_ctx* ctx, const tss_verify_batch* batch, cons
  * 8 MiB; a caller that later gives the rest of the device memory to its own pool should make that
  * first call before, and before any stream capture (it also looks up the arrays' device addresses
  * and sets the kernel's shared-memory limit).  Later calls allocate and reserve nothing.  Every
- * call on a device shares the one array and the next call overwrites it (each call leaves the
- * counters at zero, also after a timeout): calls that overlap on the GPU race, so serialise them on one stream.
+ * call on a device shares the one array and the next call overwrites it: calls that overlap on the
+ * GPU race and may return wrong results, so serialise them on one stream.  A call whose tiles are
+ * shared between CTAs clears their arrival counters on `stream` first, so a race or a timeout does
+ * not reach later calls.
  * Asynchronous on `stream`.  A device-side failure (a bounded wait that ran out) is recorded in
  * the status word that tss_linear_static_status reports; the result is then undefined. */
 tss_status tss_linear_static(const void* x, const void* w, float* y, int m_rows, int k_dim, int n_out, void* stream);

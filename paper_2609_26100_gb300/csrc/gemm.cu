@@ -470,13 +470,6 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
     tc_fence_after();
     tmem_dealloc(tmem_base, ncols);
   }
-  // (callers without a clearing pass of their own) The last CTA to leave clears the arrival counters
-  // where a wait has run out in this or an earlier launch, so that the next launch starts at zero.
-  if (p.exits && threadIdx.x == 0 && atom_add_acq_rel_gpu(p.exits, 1) == static_cast<int>(G) - 1) {
-    *p.exits = 0;
-    if (*reinterpret_cast<volatile int*>(p.status) != 0)
-      for (int t = 0; t < p.n_tiles; ++t) p.counters[t] = 0;
-  }
 }
 
 template <int EPI>

@@ -34,7 +34,6 @@ struct GemmParams {
   const StepDesc* step;
   float* partials;  // stream-K partial tiles [(grid + n_tiles) * 128 * n_pad]
   int* counters;    // per-tile arrival counters (self-resetting)
-  int* exits;       // optional: CTAs that have left (self-resetting); the last clears counters after a timeout
   int* status;
   float* out;       // kEpiStore
   int out_ld;

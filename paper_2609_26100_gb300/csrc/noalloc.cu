@@ -30,7 +30,7 @@ constexpr int kStaticMaxRows = 64;
 constexpr int kMaxDevices = 64;
 
 static __device__ __align__(256) float g_static_partials[kStaticPartialFloats];
-static __device__ __align__(256) int g_static_counters[kStaticCounters + 1];  // ... and the CTAs that have left
+static __device__ __align__(256) int g_static_counters[kStaticCounters];
 // First failure of a device-side check or bounded wait since the last tss_linear_static_status
 // (0: none); the GEMM kernel records it and never traps.
 static __device__ __align__(256) int g_static_status;
@@ -127,7 +127,9 @@ extern "C" tss_status tss_linear_static(const void* x, const void* w, float* y, 
                                            " bytes of stream-K scratch; the static limit is 8 MiB");
   // One CTA per tile where that streams a CTA at most 31 k-blocks (about 0.23 us each) more than an even
   // share -- about what storing, counting and adding partial sums costs (6 rows, k 4096, n 8192 /
-  // 10240 / 12288 / 14336: split 20.5 / 23.6 / 27.1 / 29.4 us, whole 22.6 / 22.7 / 24.7 / 26.9) -- and sums
+  // 10240 / 12288 / 14336: split 20.5 / 23.6 / 27.1 / 29.4 us, whole 22.6 / 22.7 / 24.7 / 26.9; since then a
+  // split call clears its counters, which takes 0.1 to 0.4 us, and a whole one counts nothing: 20.8 split,
+  // 22.5 / 23.6 / 26.3 whole) -- and sums
   // no accumulator longer than a split one was (four accumulators share a whole tile's k-blocks).
   if (n_tiles <= grid && kb <= T / grid + 31 && static_cast<long long>(kb) * grid <= 4 * T) grid = n_tiles;
   // Stages of three k-blocks (48 KiB of weights): a stage's fixed cost is that of one barrier round
@@ -139,6 +141,13 @@ extern "C" tss_status tss_linear_static(const void* x, const void* w, float* y, 
   if (!encode(&tx, x, k_dim, m_rows, n_pad, 2) || !encode(&tw, w, k_dim, n_out, 128, 3))
     return reject(TSS_ERR_CUDA, "cuTensorMapEncodeTiled failed");
   cudaStream_t s = static_cast<cudaStream_t>(stream);
+  if (grid != n_tiles) {
+    // Tiles are shared between CTAs, whose arrival counters must start at zero.  A call leaves them at zero,
+    // but one cut short by a device timeout, or calls that overlapped against the rule above, may not have:
+    // cleared in stream order, so that no such call spoils later ones.  (Whole tiles use no counter.)
+    e = cudaMemsetAsync(ds->counters, 0, sizeof(int) * n_tiles, s);
+    if (e != cudaSuccess) return reject(TSS_ERR_CUDA, std::string("cudaMemsetAsync: ") + cudaGetErrorString(e));
+  }
   tss::GemmParams g{};
   g.n_tiles = n_tiles;
   g.kb = kb;
@@ -151,8 +160,7 @@ extern "C" tss_status tss_linear_static(const void* x, const void* w, float* y, 
   g.m_raw = m_rows;
   g.layer_fixed = 0;
   g.partials = ds->partials;
-  g.counters = ds->counters;  // (zero between launches: the kernel sees to it)
-  g.exits = ds->counters + kStaticCounters;
+  g.counters = ds->counters;
   g.status = ds->status;
   g.out = y;
   g.out_ld = n_out;

@@ -1,6 +1,8 @@
 """The linear layer's GEMM at the edges of its stages and splits: k-blocks that do not fill a
 three-block stage, whole tiles per CTA and tiles split over many, row counts around the 16-row
 chunks; against float64 and, for the context's entry point, the same values."""
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -27,3 +29,36 @@ def test_linear_static_edges(m, k, n):
     assert np.array_equal(got[0], got[1]) and np.array_equal(got[0], got[2])
     # fp32 sums of k products of bf16 values: relative to the largest output
     assert np.abs(got[0] - exact).max() <= 2 ** -24 * k * np.abs(exact).max()
+
+
+def captured_nodes(call):
+    """The kinds of the graph nodes (0 kernel, 2 memset), sorted, that call(stream) enqueues."""
+    rt = ctypes.CDLL("libcudart.so.13")
+    stream = torch.cuda.Stream()
+    s, graph, n = ctypes.c_void_p(stream.cuda_stream), ctypes.c_void_p(), ctypes.c_size_t()
+    assert rt.cudaStreamBeginCapture(s, 1) == 0  # (thread-local)
+    try:
+        call(stream.cuda_stream)
+    finally:
+        assert rt.cudaStreamEndCapture(s, ctypes.byref(graph)) == 0
+    assert rt.cudaGraphGetNodes(graph, None, ctypes.byref(n)) == 0
+    nodes, kinds = (ctypes.c_void_p * n.value)(), []
+    assert rt.cudaGraphGetNodes(graph, nodes, ctypes.byref(n)) == 0
+    for node in nodes:
+        kind = ctypes.c_int()
+        assert rt.cudaGraphNodeGetType(ctypes.c_void_p(node), ctypes.byref(kind)) == 0
+        kinds.append(kind.value)
+    assert rt.cudaGraphDestroy(graph) == 0
+    return sorted(kinds)
+
+
+@pytest.mark.parametrize("k,n,kinds", [(4160, 256, [0, 2]), (1920, 12288, [0])])
+def test_static_counters_are_cleared_by_every_call_that_uses_them(k, n, kinds):
+    """What an earlier call left in the arrival counters (overlapping calls may leave anything) does not
+    reach a later one: shared tiles' counters are cleared in stream order, whole tiles use none."""
+    x = torch.ones((4, k), dtype=torch.bfloat16, device="cuda")
+    w = torch.ones((n, k), dtype=torch.bfloat16, device="cuda")
+    y = torch.empty((4, n), dtype=torch.float32, device="cuda")
+    native.linear_static(x, w, y)  # (the first call on a device sets it up)
+    assert native.linear_static_status() == native.TSS_OK
+    assert captured_nodes(lambda s: native.linear_static(x, w, y, s)) == kinds
