@@ -754,10 +754,10 @@ tss_status enqueue_step_mk(tss_ctx* c, const StepPlan& sp, cudaStream_t s, Prof*
     rp.part_ml = c->attn_pml;
     rp.counters = c->attn_cnt;
     rp.status = c->d_status;
-    // fault injection: with the tcgen05 attention the first attention launch withholds the signal
-    // (the persistent launches then withhold nothing)
-    const int inject_attn = tc ? p.withhold_flag : 0;
-    if (tc) p.withhold_flag = 0;
+    // fault injection: with a tcgen05 attention its first launch withholds the signal (the persistent
+    // launches then withhold nothing)
+    const int inject_attn = tc || rows ? p.withhold_flag : 0;
+    if (inject_attn) p.withhold_flag = 0;
     int pb = 0;
     for (int j = 0; j < sp.n_act; ++j) {
       p.ph_begin = pb;  // phases 4j .. 4j+3 are QKV, O, gate/up, down of slot j; 4 n_act the LM head
@@ -769,6 +769,7 @@ tss_status enqueue_step_mk(tss_ctx* c, const StepPlan& sp, cudaStream_t s, Prof*
         TSS_MK(2, TSS_CU(launch_attention_tc(tp, c->num_sms, s, prof == nullptr)));
       } else if (rows) {
         rp.slot = j;
+        rp.withhold = j == 0 ? inject_attn : 0;
         TSS_MK(2, TSS_CU(launch_attention_rows(rp, sp.B, s, prof == nullptr)));
       } else {
         ap.slot = j;

@@ -161,7 +161,9 @@ __global__ void __launch_bounds__(kArThreads, 1) attn_rows_kernel(const AttnRows
     if (lane == 0) {
       const uint32_t idS = idesc_bf16_m128(kArKeys), idPV = idesc_bf16_m128(kArD) | (1u << 16);  // (B MN-major)
       const uint32_t q_a = smem_u32(sq), k_a = smem_u32(sk), v_a = smem_u32(sv), p_a = smem_u32(sp);
-      const bool ok = mbar_wait(&qfull, 0, abort, p.status);
+      // fault injection: the first CTA at work issues no MMA, so its softmax's first wait runs out
+      const bool withheld = p.withhold && crow == 0 && h == 0 && split == 0;
+      const bool ok = mbar_wait(&qfull, 0, abort, p.status) && !withheld;
       for (int t = 0; ok && t <= n; ++t) {
         if (t < n) {
           const int s = t % kArSlots;

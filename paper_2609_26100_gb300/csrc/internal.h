@@ -162,6 +162,7 @@ struct AttnRowsParams {
   float* part_ml;                // [B][H][n_splits][nb][2]
   int* counters;                 // [B][H], self-resetting
   int* status;
+  int withhold;                  // fault injection: the first CTA at work issues no MMA (its waits run out)
 };
 cudaError_t attn_rows_prepare();
 cudaError_t launch_attention_rows(const AttnRowsParams& p, int B, cudaStream_t s, bool pdl);

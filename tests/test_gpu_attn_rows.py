@@ -3,12 +3,13 @@ attention launches): blocks of 17 rows to the largest, ends of blocks and contex
 boundaries, one split and many (merged partials), requests of very different size in one step and
 ones that skip a layer, NaN cache rows past the keys; and against the warp-level kernel."""
 import os
+import time
 
 import numpy as np
 import pytest
 import torch
 
-from paper_2609_26100_gb300 import synth
+from paper_2609_26100_gb300 import native, synth
 from tests.test_gpu_tc_attention import ARCH, SEED, Case, chain, weights  # noqa: F401 (fixture)
 
 pytestmark = pytest.mark.gpu
@@ -62,3 +63,28 @@ def test_rows_attention_close_to_warp_kernel(weights):  # noqa: F811
         out.append(Case(run, CASES["largest"](), {0: 0, 1: 0b010}).step()["logits"].cpu().numpy())
         run.close()
     assert np.abs(out[0] - out[1]).max() < 2e-2
+
+
+@pytest.mark.parametrize("splits", [1, 5])
+def test_rows_attention_bounded_wait_times_out_and_recovers(weights, splits, monkeypatch):  # noqa: F811
+    """Failure injection without a GPU fault: one CTA of the step's first attention launch issues no MMA
+    (tss_inject_timeout), so the kernel's waits run out after their 2 s (the persistent kernel's would
+    after 200 ms), the step ends with TSS_ERR_TIMEOUT and the next ones match the oracle."""
+    wo, wg = weights
+    monkeypatch.setenv("TSS_WAIT_LIMIT_MS", "200")
+    run = runner(wg, 2, splits)
+    case = Case(run, CASES["largest"](), {0: 0, 1: 0b010})
+    case.step()
+    run.v.inject_timeout(1)
+    res = run.alloc_results(2, 256, path_stride=129)
+    t0 = time.monotonic()
+    run.verify(run.batch(case.reqs), res)
+    assert run.sync_status() == native.TSS_ERR_TIMEOUT
+    assert 1.9 < time.monotonic() - t0 < 6.0
+    assert run.sync_status() == native.TSS_OK  # reported once, then cleared
+    for _ in range(2):
+        for l in range(ARCH.n_layers):  # the failed step's appends are discarded
+            for b, r in enumerate(case.reqs):
+                run.kv[l][b, :, :, r.ctx_len:].fill_(float("nan"))
+        case.check(wo, case.step(), f"after a timeout, splits {splits}")
+    run.close()
