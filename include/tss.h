@@ -304,8 +304,9 @@ tss_status tss_sync_status(tss_ctx* ctx, void* stream);
 
 /* Fault injection for tests of the device-side timeout path; no GPU fault is involved.  The next
  * n_steps verification steps of ctx on the persistent path do not publish one dataflow flag (the
- * first 128-feature tile of the residual after the first active layer), so the waits that need
- * it run out after the context's wait limit (environment variable TSS_WAIT_LIMIT_MS at
+ * first 128-feature tile of the residual after the first active layer; with more than 8 rows, where
+ * several CTAs share the tile, one of its parts is not counted either), so the waits that need it
+ * run out after the context's wait limit (environment variable TSS_WAIT_LIMIT_MS at
  * tss_create, 1..600000, default 2000 ms): the kernel records TSS_ERR_TIMEOUT in the status word,
  * every CTA leaves its loops and frees its tensor memory, and tss_sync_status reports the code.
  * That step's outputs are undefined.  The context stays usable: every step starts with fresh

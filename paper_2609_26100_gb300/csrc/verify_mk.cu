@@ -1156,7 +1156,10 @@ __global__ void __launch_bounds__(kMkThreads, 1)
           if (e.et == 0) {
             const int f = mk_cta_of(t * ph.kb, T, geff);
             const int l = mk_cta_of((t + 1) * ph.kb - 1, T, geff);
-            const int last = atom_add_acq_rel_gpu(&counters[t], 1) == l - f;
+            // (fault injection: the first CTA of the first layer's first down tile does not arrive, so the
+            // waits for that tile's parts run out)
+            const bool missing = share && p.withhold_flag && ph.kind == kMkDown && ph.slot == 0 && t == 0 && c == f;
+            const int last = !missing && atom_add_acq_rel_gpu(&counters[t], 1) == l - f;
             if (last && !share) atomicExch(&counters[t], 0);
             int* pd = s_pend + 4 * n_pend;
             pd[0] = t;

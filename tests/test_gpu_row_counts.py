@@ -78,3 +78,37 @@ def test_rows_match_oracle(weights, name, rows, mixed):
     assert_logits(got[0], np.concatenate([ref for ref, _ in refs]), f"{name} rows {rows} mixed {mixed}")
     run.close()
     torch.cuda.empty_cache()
+
+
+@pytest.mark.parametrize("rows", [9, 129])
+def test_wait_for_parts_times_out_and_recovers(weights, rows, monkeypatch):
+    """Failure injection without a GPU fault: one part of a tile that several CTAs finish together is not
+    counted (tss_inject_timeout), so their waits for it run out; the step ends with TSS_ERR_TIMEOUT, and
+    the next steps match one of a context without the failure."""
+    from paper_2609_26100_gb300.runner import TssRunner
+    a = ARCHS["wide128"]
+    _, wg = weights("wide128")
+    blocks = BLOCKS[rows]
+    reqs = []
+    for b, n in enumerate(blocks):
+        parents = synth.chain_parents(n - 1)
+        reqs.append(synth.Request(20 + 7 * b, parents, synth.draft_tokens(parents, a.vocab, SEED, f"rows.{b}"), 2))
+    monkeypatch.setenv("TSS_WAIT_LIMIT_MS", "200")
+    out = []
+    for fail in (False, True):
+        run = TssRunner(a, wg, n_slots=len(reqs), kv_cap=220, max_batch=len(reqs))
+        for b, r in enumerate(reqs):
+            for l in range(a.n_layers):
+                run.kv[l][b, :, :, :r.ctx_len] = synth.kv_block(a, l, b, r.ctx_len, SEED, device="cuda")
+        res = run.alloc_results(len(reqs), rows)
+        if fail:
+            run.v.inject_timeout(1)
+            run.verify(run.batch(reqs), res)
+            assert run.sync_status() == native.TSS_ERR_TIMEOUT
+        for _ in range(2):
+            run.verify(run.batch(reqs), res)
+            assert run.sync_status() == native.TSS_OK
+            out.append(res["logits"].cpu().numpy())
+        run.close()
+    for o in out[1:]:
+        assert np.array_equal(out[0], o)
