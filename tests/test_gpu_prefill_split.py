@@ -74,3 +74,28 @@ def test_split_attention_matches_oracle(weights, context, lengths):
                 np.testing.assert_allclose(g, r, atol=5e-2, rtol=3e-2, err_msg=f"request {b} layer {l}")
                 assert float(np.abs(g - r).mean()) < 4e-3
     run.close()
+
+
+def test_wait_for_parts_times_out_and_recovers(weights):
+    """Failure injection without a GPU fault: CTA 0 of the first GEMM, whose items are split over all CTAs,
+    issues no MMA (tss_inject_timeout); the CTAs that share its item wait for its part until their bound
+    (2 s), the call ends with TSS_ERR_TIMEOUT, and the next ones give the bits of a context without it."""
+    from paper_2609_26100_gb300.runner import TssRunner
+    _, wg = weights
+    prompt = synth.uniform_ints(300, ARCH.vocab, SEED, "split.to").tolist()
+    out = []
+    for fail in (False, True):
+        run = TssRunner(ARCH, wg, n_slots=1, kv_cap=512, max_batch=1)
+        if fail:
+            run.v.inject_timeout(1)
+            run.prefill([prompt], [0], [0])
+            assert run.sync_status() == native.TSS_ERR_TIMEOUT
+        for _ in range(2):
+            for t in run.kv:
+                t.zero_()
+            run.prefill([prompt], [0], [0])
+            assert run.sync_status() == native.TSS_OK
+            out.append([t.clone() for t in run.kv])
+        run.close()
+    for o in out[1:]:
+        assert all(torch.equal(x, y) for x, y in zip(out[0], o))
