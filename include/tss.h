@@ -246,7 +246,8 @@ tss_status tss_verify(tss_ctx* ctx, const tss_verify_batch* batch, const tss_kv_
 /* The attention kernel of the last step enqueued on ctx (tss_verify, tss_verify_grouped's last
  * group, tss_verify_profiled):
  *   0  the separate split-KV attention kernel for blocks of up to 64 rows (head_dim 128 on the
- *      persistent path: tcgen05, the rows on the MMA's 128-row side; else warp-level MMA),
+ *      persistent path: tcgen05, the rows on the MMA's 128-row side, unless many items of small
+ *      blocks make warp-level MMA shorter; else warp-level MMA),
  *   1  the tcgen05 attention kernel: blocks of at most 16 rows and head_dim 128, the keys on the
  *      MMA's 128-row side, K/V tiles by TMA, scores and outputs in tensor memory (the default for
  *      such steps; the environment variable TSS_ATTN_TC=0 at tss_create turns it off),

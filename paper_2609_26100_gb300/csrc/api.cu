@@ -292,6 +292,7 @@ tss_status run_gemm(tss_ctx* c, int epi, const CUtensorMap& tmW, const CUtensorM
 
 struct StepPlan {
   int B, M, n_act, mode, splits, n_pad;
+  bool rows_pays;     // attn_rows_pays
   int rows_splits;    // key splits of attn_rows_kernel
   int max_nodes;      // rows of the largest request's block
   int tiles;          // 64-key tiles of the longest request (context + block)
@@ -310,7 +311,7 @@ int attn_variant(const tss_ctx* c, const StepPlan& sp) {
 // Whether a separate attention launch of the persistent path runs on attn_rows_kernel: blocks of more
 // than kTcMaxNodes rows (attn_variant 0 or 2 otherwise the warp-level kernel).
 bool attn_rows(const tss_ctx* c, const StepPlan& sp) {
-  return c->attn_tc && c->D == 128 && sp.max_nodes > kTcMaxNodes && c->kvmap_ok;
+  return c->attn_tc && c->D == 128 && sp.max_nodes > kTcMaxNodes && c->kvmap_ok && sp.rows_pays;
 }
 
 AttnTcParams tc_params(const tss_ctx* c, float scale_log2) {
@@ -1101,6 +1102,9 @@ tss_status prepare_step(const tss_ctx* c, const tss_verify_batch* bt, const tss_
   sp->mode = bt->mode;
   sp->splits = splits;
   sp->rows_splits = c->attn_splits_force > 0 ? splits : rows_splits(c, sd, B);
+  sp->rows_pays = attn_rows_pays(
+      B, [&](int b) { return (sd->req_ctx[b] + sd->req_nodes[b] + 63) / 64; }, [&](int b) { return sd->req_nodes[b]; },
+      c->H, c->num_sms);
   sp->n_pad = pad_to(M, 16);
   sp->max_nodes = 1;
   for (int b = 0; b < B; ++b) sp->max_nodes = std::max(sp->max_nodes, bt->n_nodes[b]);

@@ -164,6 +164,27 @@ struct AttnRowsParams {
   int* status;
   int withhold;                  // fault injection: the first CTA at work issues no MMA (its waits run out)
 };
+// Whether a step whose largest block has 17 to 128 rows runs its separate attention there (head_dim 128)
+// rather than on the warp-level kernel.  A 64-key tile costs attn_rows_kernel the same for any block, the
+// warp-level one in time with the block's 16-row query tiles: 13, 16 and 25 for one, two and four against
+// 20 (7B layers, keys in plenty), and blocks of more than 64 rows far more.  So with as many items
+// (request, head) as SMs, or tiles enough to keep them all busy, the sum over the requests' tiles decides;
+// below that the launch is bound by its chain of latencies, where the tcgen05 one is shorter.  us a step of two
+// layers, attn_rows / warp-level: 8 requests of 17 rows at 16000 tokens 2069 / 1714, of 32 at 4000 1097 / 1012;
+// 4 of 33 at 4000 726 / 829, of 64 at 1000 723 / 804; one of 64 and 30 of 5 rows at 4000 2130 / 1611; one of 17
+// rows at 2000 323 / 329, one of 24 at 16000 524 / 543; one of 128 and 30 of 2 at 4000 2101 / 2414.
+// Tile counts: `tiles(b)` 64-key tiles of request b, which has `nodes(b)` rows.
+template <typename Tiles, typename Nodes>
+inline bool attn_rows_pays(int n_req, Tiles tiles, Nodes nodes, int n_heads, int num_sms) {
+  long long rows = 0, warps = 0;
+  for (int b = 0; b < n_req; ++b) {
+    if (nodes(b) > kNarrowNodes) return true;
+    rows += 20LL * tiles(b);
+    warps += (nodes(b) <= 16 ? 13LL : nodes(b) <= 32 ? 16LL : 25LL) * tiles(b);
+  }
+  const bool busy = n_req * n_heads > num_sms || rows / 20 * n_heads >= 100LL * num_sms;
+  return !busy || rows <= warps;
+}
 cudaError_t attn_rows_prepare();
 cudaError_t launch_attention_rows(const AttnRowsParams& p, int B, cudaStream_t s, bool pdl);
 

@@ -22,8 +22,9 @@ ARCHS = {
     "tiny": synth.TINY,
 }
 # block sizes of the requests: 8 and 9 rows (the edge between the two ways), 16 / 17 (a second
-# 16-row chunk), 61 in one block, 129 (two operand blocks per k-block) and the most rows of a step
-BLOCKS = {1: [1], 8: [3, 5], 9: [4, 2, 3], 16: [16], 17: [9, 8], 61: [61], 129: [9] * 13 + [12], 256: [16] * 16}
+# 16-row chunk), 61 in one block, 85 (more (request, head) items than SMs, most of small blocks: the
+# warp-level attention at either head size), 129 (two operand blocks per k-block) and the most rows of a step
+BLOCKS = {1: [1], 8: [3, 5], 9: [4, 2, 3], 16: [16], 17: [9, 8], 61: [61], 85: [40] + [5] * 9, 129: [9] * 13 + [12], 256: [16] * 16}
 PHI = {0: 0b010, 1: 0b101, 2: 0}
 
 
