@@ -592,10 +592,10 @@ bool mk_config_for(const MkPlanIn& c, int B, int M, int tiles, MkConfig* out) {
   // The deepest pair of rings that fits, in the order measured: weight stages of 48 KiB, then the
   // bytes of weights in flight (three stages where there is room), then the B operand's stages, which
   // hold the same k-blocks.  A stage costs the role that handles it a few hundred cycles, so one
-  // k-block a stage is the last resort (7B layers, us a step, six rows: three k-blocks a stage
+  // k-block a stage is left to TSS_MK_KPS=1 (7B layers, us a step, six rows: three k-blocks a stage
   // 553, two 587, one 761; 61 rows: 48 KiB x 2 590, 32 KiB x 3 586, one k-block 709).
-  static const int kRings[][4] = {{3, 3, 3, 3}, {3, 3, 3, 2}, {3, 2, 3, 2}, {2, 3, 2, 2}, {2, 2, 2, 2}, {2, 4, 1, 2},
-                                  {2, 3, 1, 2}, {2, 2, 1, 2}, {1, 3, 1, 2}, {1, 2, 1, 2}};
+  static const int kRings[][4] = {{3, 3, 3, 3}, {3, 3, 3, 2}, {3, 2, 3, 2}, {2, 3, 2, 2}, {2, 2, 2, 2}, {2, 3, 1, 2},
+                                  {2, 2, 1, 2}, {1, 3, 1, 2}, {1, 2, 1, 2}};
   // From 113 rows on the B operand's k-block is 32 KiB or more, twice the weights' and the larger share
   // of the copies: three stages of one k-block keep its copies going where two stages of two left gaps
   // (us a step: 128 rows 489 -> 481 and 764 -> 755, 144 rows 1148 -> 1139, 176 rows 925 -> 912, 13B 144 rows

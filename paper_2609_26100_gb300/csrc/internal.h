@@ -270,7 +270,7 @@ struct MkParams {
   __nv_bfloat16* xn;  // [kMaxRows][d] bf16(h * g) of the next norm phase, compacted rows
   float* partials0;  // stream-K partial tiles, alternating between consecutive phases
   float* partials1;
-  int* counters;     // [7 kinds][max_tiles]
+  int* counters;     // [7 kinds][max_tiles] arrivals at split tiles, then [7 kinds][max_tiles] shares finished
   float* ssp;        // [d/128][kMaxRows] per-tile partial sums of squares of h
   unsigned long long* hflag;    // [d/128]
   unsigned long long* qkvflag;  // [3d/128]

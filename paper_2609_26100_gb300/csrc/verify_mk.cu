@@ -707,7 +707,7 @@ __global__ void __launch_bounds__(kMkThreads, 1)
   uint64_t* accf = emptyx + SX;
   uint64_t* acce = accf + kMkMaxAcc;
   uint64_t* team = acce + kMkMaxAcc;  // all 256 threads: entry to / exit from a layer's attention
-  int* misc = reinterpret_cast<int*>(team + 1);  // [0] tmem addr, [1] abort, [2..4] bcast, [5] s_last
+  int* misc = reinterpret_cast<int*>(team + 1);  // [0] tmem addr, [1] abort, [5] s_last
   // (16-byte vectors from here on: the mbarriers before are an odd number of 8-byte words)
   float* xch = reinterpret_cast<float*>((reinterpret_cast<uintptr_t>(misc + 16) + 15) & ~uintptr_t(15));
   int* s_pend = reinterpret_cast<int*>(xch + 16 * 128);  // [2][4] split tiles of this CTA's phase: t, cf, cl, complete
@@ -806,7 +806,6 @@ __global__ void __launch_bounds__(kMkThreads, 1)
   e.rcos = s_rope;
   e.rsin = s_rope + 16 * 64;
   const int r = e.q * 32 + lane;
-  int* bcast = misc + 2;
   // the weight stages of this CTA's share of a phase: warp 0 lane 0 issues their bulk copies into
   // the ring (it never waits for activations, only for free ring stages)
   auto produce = [&](const MkPhase& ph, int pi) -> bool {
