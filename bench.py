@@ -156,8 +156,16 @@ KERNEL_SOURCES = {
     "attention_rows": ("attn_rows.cu", "common.cuh", "internal.h"),
 }
 
-# tss_attention_kernel -> the KERNEL_SOURCES entry of the separate attention kernel that ran
-ATTENTION_IMPL = {0: "attention_rows", 1: "attention_tc", 2: "attention_rows"}
+
+def attention_impl(code, head_dim, env=os.environ):
+    """The KERNEL_SOURCES entry of the separate attention kernel that a workload's steps ran, from
+    tss_attention_kernel's `code`: with larger blocks than the tcgen05 kernel of code 1 takes, the other
+    tcgen05 kernel where the head size and the switches allow it, else the warp-level one.  (The
+    workloads with such blocks have one request, so the rule on many small blocks does not apply.)"""
+    if code == 1:
+        return "attention_tc"
+    warp_level = head_dim != 128 or env.get("TSS_PATH") == "multi" or env.get("TSS_ATTN_TC", "1").strip() == "0"
+    return "attention" if warp_level else "attention_rows"
 
 
 def kernel_sources_hash(kernel="verify_persistent"):
@@ -584,7 +592,7 @@ def run_tss(args):
         dom = max((n for n in kernels if n in kb), key=lambda n: kernels[n]["ms_per_step"])
         ach = kernels[dom]["gbs"]
         if "attention" in kernels:
-            kernels["attention"]["impl"] = ATTENTION_IMPL.get(run.v.attention_kernel(), "attention")
+            kernels["attention"]["impl"] = attention_impl(run.v.attention_kernel(), w.arch.head_dim)
         impl = kernels[dom].get("impl", dom)
         roofline = {"kernel": impl, "bound": "hbm", "achieved": ach, "peak": peak, "unit": "GB/s",
                     "frac": ach / peak, "peak_source": f"{peak_kind} copy bandwidth",

@@ -67,3 +67,11 @@ def test_traffic_record_needs_same_kernel_workload_and_sources(tmp_path):
     assert bench.find_traffic(str(tmp_path), "attention", "7b_long") is None  # kernel changed since
     # the hash ignores comments and blank lines but not code
     assert bench.kernel_sources_hash("attention") != bench.kernel_sources_hash("verify_persistent")
+
+
+@pytest.mark.parametrize("code,head_dim,env,impl", [
+    (1, 128, {}, "attention_tc"), (0, 128, {}, "attention_rows"), (2, 128, {}, "attention_rows"), (0, 64, {}, "attention"),
+    (0, 128, {"TSS_ATTN_TC": "0"}, "attention"), (2, 128, {"TSS_PATH": "multi"}, "attention")])
+def test_attention_is_named_after_the_kernel_that_ran(code, head_dim, env, impl):
+    assert bench.attention_impl(code, head_dim, env) == impl
+    assert impl in bench.KERNEL_SOURCES
