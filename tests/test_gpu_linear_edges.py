@@ -1,6 +1,6 @@
 """The linear layer's GEMM at the edges of its stages and splits: k-blocks that do not fill a
 three-block stage, whole tiles per CTA and tiles split over many, row counts around the 16-row
-chunks; against float64 and, for the context's entry point, the same values."""
+chunks; against float64."""
 import ctypes
 
 import numpy as np
@@ -12,8 +12,13 @@ from paper_2609_26100_gb300 import native, synth
 pytestmark = pytest.mark.gpu
 
 
+# (k, n): relative 2-norm error allowed, about twice the largest of 12 measured (m as below, three seeds: 0.48,
+# 0.57, 0.71, 1.7 and 4.3 e-7).  The last one's tiles are whole, with four accumulators; with one it is 1.9e-6.
+LIMIT = {(64, 128): 1e-7, (128, 384): 1.1e-7, (448, 1280): 1.4e-7, (4160, 256): 3.4e-7, (1920, 12288): 8.5e-7}
+
+
 @pytest.mark.parametrize("m", [1, 16, 17, 64])
-@pytest.mark.parametrize("k,n", [(64, 128), (128, 384), (448, 1280), (4160, 256), (1920, 12288)])
+@pytest.mark.parametrize("k,n", list(LIMIT))
 def test_linear_static_edges(m, k, n):
     from paper_2609_26100_gb300 import build
     build.build()
@@ -27,8 +32,9 @@ def test_linear_static_edges(m, k, n):
         assert native.linear_static_status() == native.TSS_OK
         got.append(y.cpu().numpy())
     assert np.array_equal(got[0], got[1]) and np.array_equal(got[0], got[2])
-    # fp32 sums of k products of bf16 values: relative to the largest output
-    assert np.abs(got[0] - exact).max() <= 2 ** -24 * k * np.abs(exact).max()
+    assert np.linalg.norm(got[0] - exact) <= LIMIT[k, n] * np.linalg.norm(exact)
+    # (the largest error over the largest output measured at most 2.1 times the norms' ratio)
+    assert np.abs(got[0] - exact).max() <= 4 * LIMIT[k, n] * np.abs(exact).max()
 
 
 def captured_nodes(call):
