@@ -32,49 +32,6 @@ constexpr uint32_t kArTmem = 256;                  // S x 2 (64 columns each), O
 
 __host__ __device__ inline size_t ar_smem() { return 1024 + 2 * kArQPart + 2 * kArSlots * kArKV + 2 * 2 * kArPPart; }
 
-// Descriptor of an MN-major operand in 128-byte-swizzled atoms of 64 elements, atoms `lbo` bytes apart.
-__device__ __forceinline__ uint64_t ar_desc_mn(uint32_t saddr, uint32_t lbo) {
-  uint64_t d = 0;
-  d |= static_cast<uint64_t>((saddr & 0x3FFFFu) >> 4);
-  d |= static_cast<uint64_t>((lbo >> 4) & 0x3FFFu) << 16;
-  d |= static_cast<uint64_t>(1024 >> 4) << 32;
-  d |= static_cast<uint64_t>(1) << 46;
-  d |= static_cast<uint64_t>(2) << 61;
-  return d;
-}
-
-__device__ __forceinline__ void ar_tmem_st16(uint32_t taddr, const float* v) {
-  asm volatile(
-      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-      "%16};" ::"r"(taddr),
-      "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7]), "f"(v[8]), "f"(v[9]),
-      "f"(v[10]), "f"(v[11]), "f"(v[12]), "f"(v[13]), "f"(v[14]), "f"(v[15])
-      : "memory");
-  asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-}
-
-__device__ __forceinline__ void ar_fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-
-// OR of v over the 128 softmax threads (named barrier 1), which it also synchronises.
-__device__ __forceinline__ bool ar_or(bool v) {
-  uint32_t r;
-  asm volatile(
-      "{\n\t.reg .pred p, q;\n\t"
-      "setp.ne.u32 q, %1, 0;\n\t"
-      "bar.red.or.pred p, 1, 128, q;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}\n"
-      : "=r"(r)
-      : "r"(v ? 1u : 0u)
-      : "memory");
-  return r != 0;
-}
-
-__device__ __forceinline__ void ar_drain(uint64_t* bar, uint32_t parity) {
-  const uint64_t t0 = globaltimer_ns();
-  while (!mbar_try_wait(bar, parity))
-    if (globaltimer_ns() - t0 > kWaitLimitNs) return;
-}
-
 }  // namespace
 
 __global__ void __launch_bounds__(kArThreads, 1) attn_rows_kernel(const AttnRowsParams p) {
@@ -153,8 +110,8 @@ __global__ void __launch_bounds__(kArThreads, 1) attn_rows_kernel(const AttnRows
         ++nv;
       }
       // the copies issued last into each slot have landed before the kernel returns
-      for (int u = nk - 1; u >= 0 && u >= nk - kArSlots; --u) ar_drain(&kfull[u % kArSlots], (u / kArSlots) & 1);
-      for (int u = nv - 1; u >= 0 && u >= nv - kArSlots; --u) ar_drain(&vfull[u % kArSlots], (u / kArSlots) & 1);
+      for (int u = nk - 1; u >= 0 && u >= nk - kArSlots; --u) mbar_drain(&kfull[u % kArSlots], (u / kArSlots) & 1);
+      for (int u = nv - 1; u >= 0 && u >= nv - kArSlots; --u) mbar_drain(&vfull[u % kArSlots], (u / kArSlots) & 1);
     }
   } else if (warp == 1) {
     // ---------------- MMA issuer: S(t) = Q K^T, then O += P(t - 1) V ----------------
@@ -193,7 +150,7 @@ __global__ void __launch_bounds__(kArThreads, 1) attn_rows_kernel(const AttnRows
 #pragma unroll
             for (int kk = 0; kk < kArKeys / 16; ++kk)
               umma_bf16(tm + 128, sdesc_sw128(pb + part * kArPPart + kk * 32),
-                        ar_desc_mn(v_a + s * kArKV + kk * 16 * 128, kArKV / 2), idPV, (u | part | kk) ? 1u : 0u);
+                        sdesc_sw128_mn(v_a + s * kArKV + kk * 16 * 128, kArKV / 2), idPV, (u | part | kk) ? 1u : 0u);
           umma_commit(&vempty[s]);
           umma_commit(&p_free[u & 1]);
           if (u == n - 1) umma_commit(&o_full);
@@ -201,7 +158,7 @@ __global__ void __launch_bounds__(kArThreads, 1) attn_rows_kernel(const AttnRows
       }
       // every MMA issued has completed before the kernel returns
       umma_commit(&drain);
-      ar_drain(&drain, 0);
+      mbar_drain(&drain, 0);
     }
   } else {
     // ---------------- softmax: thread = row (TMEM lane) ----------------
@@ -235,7 +192,7 @@ __global__ void __launch_bounds__(kArThreads, 1) attn_rows_kernel(const AttnRows
         *reinterpret_cast<uint4*>(d + kArQPart) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
       }
     }
-    ar_fence_async_smem();
+    fence_async_smem();
     named_bar_sync(1, 128);
     if (sth == 0) mbar_arrive(&qfull);
     const int row0 = st->req_rowoff[b];
@@ -244,7 +201,7 @@ __global__ void __launch_bounds__(kArThreads, 1) attn_rows_kernel(const AttnRows
     bool ok = true;
     for (int t = 0; t < n; ++t) {
       ok = mbar_wait(&s_full[t & 1], (t >> 1) & 1, abort, p.status);
-      if (ar_or(!ok)) break;
+      if (bar_or<1>(!ok)) break;
       tc_fence_after();
       float s[kArKeys];
 #pragma unroll
@@ -293,7 +250,7 @@ __global__ void __launch_bounds__(kArThreads, 1) attn_rows_kernel(const AttnRows
           for (int i = 0; i < 8; ++i) v0[i] = v1[i] = make_uint4(0, 0, 0, 0);
         }
       }
-      if (ar_or(!ok)) break;
+      if (bar_or<1>(!ok)) break;
       if (rescale) {
         tc_fence_after();
         float o[16];
@@ -302,7 +259,7 @@ __global__ void __launch_bounds__(kArThreads, 1) attn_rows_kernel(const AttnRows
           tmem_ld16(tm + lanes + 128 + c * 16, o);
 #pragma unroll
           for (int i = 0; i < 16; ++i) o[i] *= alpha;
-          ar_tmem_st16(tm + lanes + 128 + c * 16, o);
+          tmem_st16(tm + lanes + 128 + c * 16, o);
         }
         tc_fence_before();
       }
@@ -323,12 +280,12 @@ __global__ void __launch_bounds__(kArThreads, 1) attn_rows_kernel(const AttnRows
         *reinterpret_cast<uint4*>(ph + sw) = make_uint4(hw[0], hw[1], hw[2], hw[3]);
         *reinterpret_cast<uint4*>(ph + kArPPart + sw) = make_uint4(lw[0], lw[1], lw[2], lw[3]);
       }
-      ar_fence_async_smem();
+      fence_async_smem();
       named_bar_sync(1, 128);
       if (sth == 0) mbar_arrive(&p_full[t & 1]);
     }
     if (ok) ok = mbar_wait(&o_full, 0, abort, p.status);
-    if (!ar_or(!ok)) {
+    if (!bar_or<1>(!ok)) {
       tc_fence_after();
       const size_t item = static_cast<size_t>(b) * H + h;
       if (used == 1) {

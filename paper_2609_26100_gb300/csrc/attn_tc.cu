@@ -72,60 +72,13 @@ __host__ __device__ inline size_t tc_dyn_smem() {
   return static_cast<size_t>(2 * kTcStages) * kSlotBytes + 2 * kQBytes + 2 * kPBytes + 1024;
 }
 
-// Descriptor of an MN-major operand in 128-byte-swizzled atoms of 64 elements along M (or N):
-// atoms `lbo` bytes apart, 8-row groups along K 1024 bytes apart.
-__device__ __forceinline__ uint64_t sdesc_sw128_mn(uint32_t saddr, uint32_t lbo) {
-  uint64_t d = 0;
-  d |= static_cast<uint64_t>((saddr & 0x3FFFFu) >> 4);
-  d |= static_cast<uint64_t>((lbo >> 4) & 0x3FFFu) << 16;
-  d |= static_cast<uint64_t>(1024 >> 4) << 32;
-  d |= static_cast<uint64_t>(1) << 46;
-  d |= static_cast<uint64_t>(2) << 61;
-  return d;
-}
-
 // Byte offset of element (row r, column k) of a 32-row operand in K-major 128-byte swizzle:
 // 64-column blocks of kOpBytes, rows of 128 B, 16-byte chunks permuted by the row.
 __device__ __forceinline__ uint32_t op_off(int r, int k) {
   return static_cast<uint32_t>((k >> 6) * kOpBytes + r * 128 + ((((k & 63) >> 3) ^ (r & 7)) << 4) + (k & 7) * 2);
 }
 
-// OR of v over the 128 threads of named barrier ID (which it also synchronises).
-template <int ID>
-__device__ __forceinline__ bool bar_or(bool v) {
-  uint32_t r;
-  asm volatile(
-      "{\n\t.reg .pred p, q;\n\t"
-      "setp.ne.u32 q, %1, 0;\n\t"
-      "bar.red.or.pred p, %2, 128, q;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}\n"
-      : "=r"(r)
-      : "r"(v ? 1u : 0u), "n"(ID)
-      : "memory");
-  return r != 0;
-}
-
 constexpr int kBarSoftmax = 1, kBarEpi = 2;
-
-__device__ __forceinline__ void tmem_st16(uint32_t taddr, const float* v) {
-  asm volatile(
-      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-      "%16};" ::"r"(taddr),
-      "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7]), "f"(v[8]), "f"(v[9]),
-      "f"(v[10]), "f"(v[11]), "f"(v[12]), "f"(v[13]), "f"(v[14]), "f"(v[15])
-      : "memory");
-  asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-}
-
-__device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-
-// Wait for a phase that an already-issued copy or MMA will complete, whatever the abort state
-// (used before the kernel returns so that nothing writes shared or tensor memory afterwards).
-__device__ __forceinline__ void mbar_drain(uint64_t* bar, uint32_t parity) {
-  const uint64_t t0 = globaltimer_ns();
-  while (!mbar_try_wait(bar, parity))
-    if (globaltimer_ns() - t0 > kWaitLimitNs) return;
-}
 
 // The CTA (of C) whose range holds global tile g of T: ranges are [c T / C, (c + 1) T / C).
 __device__ __forceinline__ int tc_cta_of(long long g, long long T, int C) {

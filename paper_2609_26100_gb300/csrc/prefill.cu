@@ -39,8 +39,6 @@ __host__ __device__ inline size_t pf_gemm_smem() {
   return 1024 + static_cast<size_t>(kPfStages) * kPfStage + kPgGroups * 16 * 128 * 4;  // + exchange per group
 }
 
-__device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-
 // Four consecutive elements as bf16 hi and lo parts: one 8-byte store each.
 __device__ __forceinline__ void pf_split_store4(__nv_bfloat16* hi, __nv_bfloat16* lo, size_t i, const float* x) {
   uint32_t h[2], l[2];
@@ -555,40 +553,6 @@ __host__ __device__ inline size_t pf_attn_smem() {
   return 1024 + 2 * kPaQPart + 2 * kPaSlots * kPaKV + 2 * 2 * kPaPPart;
 }
 
-__device__ __forceinline__ uint64_t pa_desc_mn(uint32_t saddr, uint32_t lbo) {
-  uint64_t d = 0;
-  d |= static_cast<uint64_t>((saddr & 0x3FFFFu) >> 4);
-  d |= static_cast<uint64_t>((lbo >> 4) & 0x3FFFu) << 16;
-  d |= static_cast<uint64_t>(1024 >> 4) << 32;
-  d |= static_cast<uint64_t>(1) << 46;
-  d |= static_cast<uint64_t>(2) << 61;
-  return d;
-}
-
-__device__ __forceinline__ void pa_st16(uint32_t taddr, const float* v) {
-  asm volatile(
-      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-      "%16};" ::"r"(taddr),
-      "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7]), "f"(v[8]), "f"(v[9]),
-      "f"(v[10]), "f"(v[11]), "f"(v[12]), "f"(v[13]), "f"(v[14]), "f"(v[15])
-      : "memory");
-  asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-}
-
-// OR of v over the 128 softmax threads (named barrier 1), which it also synchronises.
-__device__ __forceinline__ bool pa_or(bool v) {
-  uint32_t r;
-  asm volatile(
-      "{\n\t.reg .pred p, q;\n\t"
-      "setp.ne.u32 q, %1, 0;\n\t"
-      "bar.red.or.pred p, 1, 128, q;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}\n"
-      : "=r"(r)
-      : "r"(v ? 1u : 0u)
-      : "memory");
-  return r != 0;
-}
-
 // A split item's end, by the softmax threads: this CTA's part of O (raw sums, tensor memory at tm) and
 // its rows' (max, sum) go to p.partials; the last CTA of the item to arrive adds the parts in split
 // order and writes the outputs.  wgt: [split][128] floats of shared memory.
@@ -799,7 +763,7 @@ __global__ void __launch_bounds__(kPfThreads, 1) pf_attn_kernel(const __grid_con
 #pragma unroll
             for (int kk = 0; kk < kPaKeys / 16; ++kk)
               umma_bf16(tm + 128, sdesc_sw128(pb + part * kPaPPart + kk * 32),
-                        pa_desc_mn(v_a + s * kPaKV + kk * 16 * 128, kPaKV / 2), idPV, (u | part | kk) ? 1u : 0u);
+                        sdesc_sw128_mn(v_a + s * kPaKV + kk * 16 * 128, kPaKV / 2), idPV, (u | part | kk) ? 1u : 0u);
           umma_commit(&vempty[s]);
           umma_commit(&p_free[u & 1]);
           if (u == n - 1) umma_commit(&o_full);
@@ -822,7 +786,7 @@ __global__ void __launch_bounds__(kPfThreads, 1) pf_attn_kernel(const __grid_con
     bool ok = true;
     for (int t = 0; t < n; ++t) {
       ok = mbar_wait(&s_full[t & 1], (t >> 1) & 1, abort, p.status);
-      if (pa_or(!ok)) break;
+      if (bar_or<1>(!ok)) break;
       tc_fence_after();
       float s[kPaKeys];
 #pragma unroll
@@ -860,7 +824,7 @@ __global__ void __launch_bounds__(kPfThreads, 1) pf_attn_kernel(const __grid_con
           for (int i = 0; i < 8; ++i) v0[i] = v1[i] = make_uint4(0, 0, 0, 0);
         }
       }
-      if (pa_or(!ok)) break;
+      if (bar_or<1>(!ok)) break;
       if (t >= 1 && __any_sync(0xffffffffu, raise && alpha != 1.f)) {
         tc_fence_after();
         float o[16];
@@ -869,7 +833,7 @@ __global__ void __launch_bounds__(kPfThreads, 1) pf_attn_kernel(const __grid_con
           tmem_ld16(tm + lanes + 128 + c * 16, o);
 #pragma unroll
           for (int i = 0; i < 16; ++i) o[i] *= alpha;
-          pa_st16(tm + lanes + 128 + c * 16, o);
+          tmem_st16(tm + lanes + 128 + c * 16, o);
         }
         tc_fence_before();
       }
@@ -898,7 +862,7 @@ __global__ void __launch_bounds__(kPfThreads, 1) pf_attn_kernel(const __grid_con
     }
     if (ok) {
       ok = mbar_wait(&o_full, 0, abort, p.status);
-      const bool fail = pa_or(!ok);
+      const bool fail = bar_or<1>(!ok);
       if (!fail && used > 1) {
         pa_merge(p, reinterpret_cast<float*>(sp), &s_last, tm + lanes, st, qr, q0, nrow, used, m, l);
       } else if (!fail) {
