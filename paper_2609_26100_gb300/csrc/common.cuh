@@ -307,7 +307,7 @@ __device__ __forceinline__ void store_split4(const SplitAt& s, int j, const floa
 // divisor is scaled, so that its reciprocal stays normal.  The division operator's call for special
 // operands stands in the middle of the persistent kernel's epilogues, and __fdividef is off by up to
 // 2 ulp and 0 where the divisor exceeds 2^126 (gates below -87.3).  us a step with the operator / this /
-// __fdividef: tiny decoder's chain 131 / 124 / 124, 7B chain 2667 / 2655 / 2650, 61-row tree 536 / 531 / 527.
+// __fdividef: 7B chain 2667 / 2655 / 2650, 61-row tree of 4 layers 536 / 531 / 527.
 __device__ __forceinline__ float silu(float g) {
   const float e = 1.f + expf(-g);
   const float s = e > 0x1p100f ? 0x1p-32f : 1.f;
